@@ -82,11 +82,14 @@ __device__ __forceinline__ void equilibrium_cell(double r, double th, const doub
     });
 }
 
+// Writers of a state copy g also write the rest populations of the sets that leave them alone
+// (rest_static) into the other copy, `other`: a step neither reads nor writes them.
+
 // g_i = g_i^eq(rho', u', theta') (Sec. 7 initial condition), encoded into storage type T.
 template <class S, class T>
 __global__ void k_init_equilibrium(const double *__restrict__ rho, const double *__restrict__ u,
-                                   const double *__restrict__ theta, T *__restrict__ g, long long cells, long long pitch,
-                                   SetConsts k) {
+                                   const double *__restrict__ theta, T *__restrict__ g, T *__restrict__ other,
+                                   long long cells, long long pitch, SetConsts k) {
     constexpr int SC = Store<T>::scaled ? 1 : 0;
     for (long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x; x < cells; x += (long long)gridDim.x * blockDim.x) {
         double uu[3] = {0.0, 0.0, 0.0};
@@ -94,7 +97,9 @@ __global__ void k_init_equilibrium(const double *__restrict__ rho, const double 
         for (int a = 0; a < S::D; ++a) uu[a] = u[(long long)a * cells + x];
         equilibrium_cell<S, SC>(rho[x], theta[x], uu, k, [&](int i, double v) {
             if (SC) v *= k.scale;
-            g[(long long)i * pitch + x] = Store<T>::make((typename Store<T>::C)v);
+            const T e = Store<T>::make((typename Store<T>::C)v);
+            g[(long long)i * pitch + x] = e;
+            if (rest_static<S>() && i == 0) other[x] = e;
         });
     }
 }
@@ -150,7 +155,7 @@ __device__ __forceinline__ void edge_fixup_cell_from(T *__restrict__ dst, const 
     });
     collide_cell<S, 0>(pull, post, cf);
 #pragma unroll
-    for (int i = 0; i < S::Q; ++i) dst[(long long)i * gd.pitch + (long long)y * nx + x] = Store<T>::make(post[i][0]);
+    for (int i = rest_static<S>() ? 1 : 0; i < S::Q; ++i) dst[(long long)i * gd.pitch + (long long)y * nx + x] = Store<T>::make(post[i][0]);
 }
 template <class S, class T, class Ghost>
 __device__ __forceinline__ void edge_fixup_cell(const T *__restrict__ src, T *__restrict__ dst, const GridDesc &gd,
@@ -195,7 +200,8 @@ __global__ void k_edge_fixup(const T *__restrict__ src, T *__restrict__ dst, Gri
 // Applied once after init_fields so that the initial state is a post-collision state like every
 // later one (the equilibrium is its own collision; the frame damping is not).
 template <class S, class T>
-__global__ void k_sponge_damp(T *__restrict__ g, GridDesc gd, int w, typename Store<T>::C smax) {
+__global__ void k_sponge_damp(T *__restrict__ g, T *__restrict__ other, GridDesc gd, int w,
+                              typename Store<T>::C smax) {
     using C = typename Store<T>::C;
     const long long cells = (long long)gd.nx * gd.ny * gd.nz;
     for (long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x; x < cells; x += (long long)gridDim.x * blockDim.x) {
@@ -208,6 +214,7 @@ __global__ void k_sponge_damp(T *__restrict__ g, GridDesc gd, int w, typename St
         for (int i = 0; i < S::Q; ++i) {
             T *p = g + (long long)i * gd.pitch + x;
             *p = Store<T>::make(Store<T>::load(*p) * damp);
+            if (rest_static<S>() && i == 0) other[x] = *p;
         }
     }
 }
@@ -367,7 +374,8 @@ __global__ void k_export(const T *__restrict__ g, long long cells, long long pit
 }
 
 template <class S, class T>
-__global__ void k_import(const double *__restrict__ in, long long cells, long long pitch, SetConsts k, T *__restrict__ g) {
+__global__ void k_import(const double *__restrict__ in, long long cells, long long pitch, SetConsts k, T *__restrict__ g,
+                         T *__restrict__ other) {
     constexpr bool scaled = Store<T>::scaled;
     for (long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x; x < cells; x += (long long)gridDim.x * blockDim.x) {
         static_for<S::Q>([&](auto I) {
@@ -375,7 +383,9 @@ __global__ void k_import(const double *__restrict__ in, long long cells, long lo
             constexpr int s = S::shell(i);
             const double v = in[(long long)i * cells + x];
             const double st = scaled ? v * k.enc[s] : v;
-            g[(long long)i * pitch + x] = Store<T>::make((typename Store<T>::C)st);
+            const T e = Store<T>::make((typename Store<T>::C)st);
+            g[(long long)i * pitch + x] = e;
+            if (rest_static<S>() && i == 0) other[x] = e;
         });
     }
 }
@@ -441,8 +451,10 @@ __global__ void k_slab_unpack(T *__restrict__ g, long long pitch, long long plan
 // 8 lanes of a block share its exponent by shuffles; cells past the grid take part as zeros and
 // store nothing.  `value(i, x)` gives the FP32 value of velocity i at cell x.
 template <class S, class F>
-__device__ __forceinline__ void bfp_write_cells(Bfp16 *__restrict__ g, long long cells, long long pitch, F &&value) {
+__device__ __forceinline__ void bfp_write_cells(Bfp16 *__restrict__ g, Bfp16 *__restrict__ other, long long cells,
+                                                long long pitch, F &&value) {
     uint8_t *__restrict__ ex = bfp_exps<S::Q>(g, pitch);
+    uint8_t *__restrict__ ox = bfp_exps<S::Q>(other, pitch);
     const long long n = (cells + kBfpBlock - 1) / kBfpBlock * kBfpBlock;
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long w0 = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31); w0 < n; w0 += stride) {
@@ -455,6 +467,7 @@ __device__ __forceinline__ void bfp_write_cells(Bfp16 *__restrict__ g, long long
             const long long e = (long long)i * pitch + x;
             const float one[1] = {v[i]};
             bfp_store_vec<1>(g + e, ex + (e >> 3), one, valid);
+            if constexpr (!carried<S>(i)) bfp_store_vec<1>(other + e, ox + (e >> 3), one, valid);
         });
     }
 }
@@ -462,9 +475,9 @@ __device__ __forceinline__ void bfp_write_cells(Bfp16 *__restrict__ g, long long
 // g_i = g_i^eq(rho', u', theta') (Sec. 7 initial condition), rounded to FP32 and encoded.
 template <class S>
 __global__ void k_init_equilibrium_bfp(const double *__restrict__ rho, const double *__restrict__ u,
-                                       const double *__restrict__ theta, Bfp16 *__restrict__ g, long long cells,
-                                       long long pitch, SetConsts k) {
-    bfp_write_cells<S>(g, cells, pitch, [&](long long x, float (&v)[S::Q]) {
+                                       const double *__restrict__ theta, Bfp16 *__restrict__ g,
+                                       Bfp16 *__restrict__ other, long long cells, long long pitch, SetConsts k) {
+    bfp_write_cells<S>(g, other, cells, pitch, [&](long long x, float (&v)[S::Q]) {
         if (x < 0) {
 #pragma unroll
             for (int i = 0; i < S::Q; ++i) v[i] = 0.f;
@@ -479,8 +492,9 @@ __global__ void k_init_equilibrium_bfp(const double *__restrict__ rho, const dou
 
 // FP64 [q][cells] -> BFP16 (resume): each value rounded to FP32, then encoded.
 template <class S>
-__global__ void k_import_bfp(const double *__restrict__ in, long long cells, long long pitch, Bfp16 *__restrict__ g) {
-    bfp_write_cells<S>(g, cells, pitch, [&](long long x, float (&v)[S::Q]) {
+__global__ void k_import_bfp(const double *__restrict__ in, long long cells, long long pitch, Bfp16 *__restrict__ g,
+                             Bfp16 *__restrict__ other) {
+    bfp_write_cells<S>(g, other, cells, pitch, [&](long long x, float (&v)[S::Q]) {
 #pragma unroll
         for (int i = 0; i < S::Q; ++i) v[i] = x < 0 ? 0.f : (float)in[(long long)i * cells + x];
     });
@@ -489,10 +503,10 @@ __global__ void k_import_bfp(const double *__restrict__ in, long long cells, lon
 // Sponge damping of a stored BFP16 state (after init_fields): decoded, damped as in the FP32
 // kernel, re-encoded (in place: each warp reads its blocks before it writes them).
 template <class S>
-__global__ void k_sponge_damp_bfp(Bfp16 *__restrict__ g, GridDesc gd, int w, float smax) {
+__global__ void k_sponge_damp_bfp(Bfp16 *__restrict__ g, Bfp16 *__restrict__ other, GridDesc gd, int w, float smax) {
     const long long cells = (long long)gd.nx * gd.ny * gd.nz;
     const uint8_t *ex = bfp_exps<S::Q>(g, gd.pitch);
-    bfp_write_cells<S>(g, cells, gd.pitch, [&](long long x, float (&v)[S::Q]) {
+    bfp_write_cells<S>(g, other, cells, gd.pitch, [&](long long x, float (&v)[S::Q]) {
         if (x < 0) {
 #pragma unroll
             for (int i = 0; i < S::Q; ++i) v[i] = 0.f;

@@ -558,7 +558,8 @@ lee_status lee_batch_init_fields(lee_batch *b, int32_t d, const double *rho, con
         du = b->fields + c;
         dt = b->fields + 3 * c;
     }
-    BCK(b, b->ops->init(b->storage, dr, du, dt, dom_ptr(b, b->cur, d), c, b->pitch[d], consts_for(b->set, 1.0), b->st),
+    BCK(b, b->ops->init(b->storage, dr, du, dt, dom_ptr(b, b->cur, d), dom_ptr(b, b->cur ^ 1, d), c, b->pitch[d],
+                        consts_for(b->set, 1.0), b->st),
         "init kernel");
     if (!on_device) BCK(b, cudaStreamSynchronize(b->st), "sync");
     return LEE_OK;

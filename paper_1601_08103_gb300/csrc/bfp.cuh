@@ -217,7 +217,7 @@ __device__ __forceinline__ void stream_collide_chunk_bfp(const Bfp16 *__restrict
     const bool has_right = (lane < 31) && (xc < gd.nxc - 1);
 
     C pull[S::Q][V];
-    static_for<S::Q>([&](auto I) {
+    static_for_carried<S>([&](auto I) {
         constexpr int i = decltype(I)::value;
         constexpr int cx = S::c(i, 0), cy = S::c(i, 1), cz = S::c(i, 2);
         int ys = y - cy, zs = z - cz;
@@ -283,13 +283,21 @@ __device__ __forceinline__ void stream_collide_chunk_bfp(const Bfp16 *__restrict
             for (int k = 0; k < V; ++k) {
                 const C damp = sponge_factor<C>(x0 + k, y, z, gd, S::D, ob.sponge_w, ob.sponge_smax);
 #pragma unroll
-                for (int i = 0; i < S::Q; ++i) post[i][k] *= damp;
+                for (int i = rest_static<S>() ? 1 : 0; i < S::Q; ++i) post[i][k] *= damp;
+            }
+            if constexpr (rest_static<S>()) {  // the frame damps its rest populations too; whole blocks
+                const long long x = ((long long)z * gd.ny + y) * gd.nx + x0;
+                C r[V];
+                bfp_load_vec<V>(src + x, sx + (x >> 3), r);
+#pragma unroll
+                for (int k = 0; k < V; ++k) r[k] *= sponge_factor<C>(x0 + k, y, z, gd, S::D, ob.sponge_w, ob.sponge_smax);
+                bfp_store_vec<V>(dst + x, dx + (x >> 3), r, active);
             }
         }
     }
 
     const long long outi = ((long long)z * gd.ny + y) * gd.nx + x0;
-    static_for<S::Q>([&](auto I) {
+    static_for_carried<S>([&](auto I) {
         constexpr int i = decltype(I)::value;
         const long long e = (long long)i * gd.pitch + outi;
         bfp_store_vec<V>(dst + e, dx + (e >> 3), post[i], active);

@@ -2,9 +2,10 @@
 //
 // Hot path: one fused pull-stream + BGK-collide kernel per time step (Sec. 6, eq. "LBE update
 // scheme").  Populations live in structure-of-arrays layout, one array per velocity, x fastest,
-// in a ping-pong pair of buffers.  With SoA and a pull step every stored population is read
-// exactly once and written exactly once per step, so DRAM traffic equals the algorithmic
-// 2 * q * sizeof(storage) bytes per cell without any shared-memory staging:
+// in a ping-pong pair of buffers.  With SoA and a pull step every stored population that a step
+// changes (all but the rest ones for most sets, see rest_static) is read exactly once and written exactly
+// once, so DRAM traffic equals the algorithmic 2 * sizeof(storage) bytes per such population
+// without any shared-memory staging:
 //   - each thread owns V consecutive cells of one x-row (one 16-byte vector per velocity);
 //   - a velocity with c_x = 0 is a plain aligned vector load from row (y - c_y, z - c_z);
 //   - c_x = +1 / -1 shifts the vector by one element: the missing element comes from the
@@ -211,18 +212,63 @@ __host__ __device__ constexpr int moving_shells() {
     return n;
 }
 
+// Sets whose moving velocities share one shell (all but D3Q19).  Mass is P_0 + P_1 and energy is
+// proportional to P_1, so the collision conserves the shell sums P_0 and P_1 one by one:
+// mhat[0] = (1, 0) and mhat[1] = (0, 1/q_1) in the folded coefficients.  Two things follow.
+//  - The rest population of a cell never changes (only a sponge frame damps it), so a step neither
+//    reads nor writes it: both state copies hold it, written when the state is set.  A D2Q5 FP32 step
+//    moves 32 bytes per cell instead of 40, a D3Q7 one 48 instead of 56.
+//  - The moving populations collide among themselves.
+template <class S>
+__host__ __device__ constexpr bool rest_static() {
+    return moving_shells<S>() == 1;
+}
+// Whether a step changes velocity i (velocity 0 is the rest one in every set).
+template <class S>
+__host__ __device__ constexpr bool carried(int i) {
+    return !(rest_static<S>() && S::shell(i) == 0);
+}
+// Whether shell s takes part in the collision's sums.
+template <class S>
+__host__ __device__ constexpr bool mixes(int s) {
+    return shell_present<S>(s) && !(rest_static<S>() && s == 0);
+}
+template <class S, class F>
+__device__ __forceinline__ void static_for_carried(F &&f) {
+    static_for<S::Q>([&](auto I) {
+        if constexpr (carried<S>(decltype(I)::value)) f(I);
+    });
+}
+
+// Rest and axis velocities only (D1Q3, D2Q5, D3Q7 and the diatomic sets).  There the momentum part of
+// the equilibrium, f*_1 (b / rho0) c_i . J = (g_+a - g_-a) / 2, is the odd part of the pair itself for
+// every set of Sec. 8, so relaxation leaves the odd parts alone and
+//     g*_+-a = g_+-a + (w / 2D) (P_1 - D s_a),     s_a = g_+a + g_-a,
+// which is 7 operations per cell for D2Q5 (22 in the matrix form) and 14 for D3Q7, and nothing at all
+// for D1Q3 (H = I, Sec. 8.1).  Its roundings are fewer than the matrix form's (FP64, D3Q7 diatomic, 50
+// steps against 80-bit arithmetic: 7e-17 instead of 6e-15); the corrections of a cell add up to zero
+// whatever w / 2D rounds to, so that coefficient needs no residual.  FP64 steps are bound by GB300's
+// FP64 pipe, so there it pays most: D2Q5 FP64 2048^2 28.1 -> 71 GLUPS, D3Q7 diatomic FP64 193x161x135
+// 20.5 -> 36 GLUPS.
+template <class S>
+__host__ __device__ constexpr bool axis_set() {
+    bool axis = rest_static<S>() && shell_present<S>(1) && S::Q == 2 * S::D + 1;
+    for (int a = 0; a < S::D; ++a) axis = axis && S::c(1 + 2 * a, a) == 1 && S::c(2 + 2 * a, a) == -1;
+    return axis;
+}
+
 // Every rounding is spelled out so that no result depends on the compiler's contraction of a
 // multiply and an add: with one moving shell the momentum term of velocity i is one fused
 // multiply-add per axis, eq = fma(+-N[t][s1], J[s1][a], eq); with several moving shells the sums
 // KJ[t][a] = sum_s N[t][s] J[s][a] (a chain of fused multiply-adds) are added to eq.
 template <class S, int K, class C, int V>
-__device__ __forceinline__ void collide_cell(const C (&g)[S::Q][V], C (&out)[S::Q][V], const CollideCoef<C> &cf) {
+__device__ __forceinline__ void collide_shells_cell(const C (&g)[S::Q][V], C (&out)[S::Q][V], const CollideCoef<C> &cf) {
     // Accumulators start at -0.0 so that the first addition folds away exactly.
     C P[4] = {C(-0.0), C(-0.0), C(-0.0), C(-0.0)};
     C J[4][3];
 #pragma unroll
     for (int s = 0; s < 4; ++s) J[s][0] = J[s][1] = J[s][2] = C(-0.0);
-    static_for<S::Q>([&](auto I) {
+    static_for_carried<S>([&](auto I) {
         constexpr int i = decltype(I)::value;
         constexpr int s = S::shell(i);
         const C v = g[i][K];
@@ -236,17 +282,17 @@ __device__ __forceinline__ void collide_cell(const C (&g)[S::Q][V], C (&out)[S::
     C B[4], KJ[4][3];
     static_for<4>([&](auto T) {
         constexpr int t = decltype(T)::value;
-        if constexpr (shell_present<S>(t)) {
+        if constexpr (mixes<S>(t)) {
             C acc = C(-0.0);
             if constexpr (std::is_same<C, float>::value) {
                 static_for<4>([&](auto Sx) {
                     constexpr int s = decltype(Sx)::value;
-                    if constexpr (shell_present<S>(s)) acc = fma(cf.Mlo[t][s], P[s], acc);
+                    if constexpr (mixes<S>(s)) acc = fma(cf.Mlo[t][s], P[s], acc);
                 });
             }
             static_for<4>([&](auto Sx) {
                 constexpr int s = decltype(Sx)::value;
-                if constexpr (shell_present<S>(s)) acc = fma(cf.M[t][s], P[s], acc);
+                if constexpr (mixes<S>(s)) acc = fma(cf.M[t][s], P[s], acc);
             });
             B[t] = acc;
             if constexpr (t > 0 && moving_shells<S>() > 1) {
@@ -262,7 +308,7 @@ __device__ __forceinline__ void collide_cell(const C (&g)[S::Q][V], C (&out)[S::
             }
         }
     });
-    static_for<S::Q>([&](auto I) {
+    static_for_carried<S>([&](auto I) {
         constexpr int i = decltype(I)::value;
         constexpr int t = S::shell(i);
         C eq = B[t];
@@ -282,6 +328,38 @@ __device__ __forceinline__ void collide_cell(const C (&g)[S::Q][V], C (&out)[S::
     });
 }
 
+template <class S, int K, class C, int V>
+__device__ __forceinline__ void collide_axis_cell(const C (&g)[S::Q][V], C (&out)[S::Q][V], const CollideCoef<C> &cf) {
+    const C w = cf.M[1][1];  // w / 2D
+    if constexpr (S::D == 1) {
+        out[1][K] = g[1][K];
+        out[2][K] = g[2][K];
+    } else if constexpr (S::D == 2) {
+        const C d = (g[3][K] + g[4][K]) - (g[1][K] + g[2][K]);
+        out[1][K] = fma(w, d, g[1][K]);
+        out[2][K] = fma(w, d, g[2][K]);
+        out[3][K] = fma(-w, d, g[3][K]);
+        out[4][K] = fma(-w, d, g[4][K]);
+    } else {
+        const C sx = g[1][K] + g[2][K], sy = g[3][K] + g[4][K], sz = g[5][K] + g[6][K];
+        const C P = (sx + sy) + sz;
+        const C tx = fma(C(-3), sx, P), ty = fma(C(-3), sy, P), tz = fma(C(-3), sz, P);
+        out[1][K] = fma(w, tx, g[1][K]);
+        out[2][K] = fma(w, tx, g[2][K]);
+        out[3][K] = fma(w, ty, g[3][K]);
+        out[4][K] = fma(w, ty, g[4][K]);
+        out[5][K] = fma(w, tz, g[5][K]);
+        out[6][K] = fma(w, tz, g[6][K]);
+    }
+}
+
+template <class S, int K, class C, int V>
+__device__ __forceinline__ void collide_cell(const C (&g)[S::Q][V], C (&out)[S::Q][V], const CollideCoef<C> &cf) {
+    if constexpr (rest_static<S>()) out[0][K] = g[0][K];
+    if constexpr (axis_set<S>()) collide_axis_cell<S, K>(g, out, cf);
+    else collide_shells_cell<S, K>(g, out, cf);
+}
+
 // FP32 collision of two cells (K, K+1) at once with the packed f32x2 add, mul and fma of sm_100
 // and later.  Every packed operation rounds each half exactly like the scalar operation it
 // replaces in collide_cell (a - b is a + (-b); a first accumulation into -0.0 is the value itself,
@@ -291,11 +369,10 @@ __device__ __forceinline__ float2 splat2(float c) { return make_float2(c, c); }
 __device__ __forceinline__ float2 neg2(float2 v) { return make_float2(-v.x, -v.y); }
 
 template <class S, int K, int V>
-__device__ __forceinline__ void collide_pair(const float (&g)[S::Q][V], float (&out)[S::Q][V],
+__device__ __forceinline__ void collide_shells_pair(const float (&g)[S::Q][V], float (&out)[S::Q][V],
                                              const CollideCoef<float> &cf) {
-    static_assert(K + 1 < V, "a pair needs two cells");
     float2 P[4], J[4][3];
-    static_for<S::Q>([&](auto I) {
+    static_for_carried<S>([&](auto I) {
         constexpr int i = decltype(I)::value;
         constexpr int s = S::shell(i);
         const float2 v = make_float2(g[i][K], g[i][K + 1]);
@@ -314,19 +391,19 @@ __device__ __forceinline__ void collide_pair(const float (&g)[S::Q][V], float (&
     float2 B[4], KJ[4][3];
     static_for<4>([&](auto T) {
         constexpr int t = decltype(T)::value;
-        if constexpr (shell_present<S>(t)) {
-            constexpr int s0 = first_present_shell<S>(0);
+        if constexpr (mixes<S>(t)) {
+            constexpr int s0 = first_present_shell<S>(rest_static<S>() ? 1 : 0);
             float2 acc;
             static_for<4>([&](auto Sx) {
                 constexpr int s = decltype(Sx)::value;
-                if constexpr (shell_present<S>(s)) {
+                if constexpr (mixes<S>(s)) {
                     if constexpr (s == s0) acc = __fmul2_rn(splat2(cf.Mlo[t][s]), P[s]);
                     else acc = __ffma2_rn(splat2(cf.Mlo[t][s]), P[s], acc);
                 }
             });
             static_for<4>([&](auto Sx) {
                 constexpr int s = decltype(Sx)::value;
-                if constexpr (shell_present<S>(s)) acc = __ffma2_rn(splat2(cf.M[t][s]), P[s], acc);
+                if constexpr (mixes<S>(s)) acc = __ffma2_rn(splat2(cf.M[t][s]), P[s], acc);
             });
             B[t] = acc;
             if constexpr (t > 0 && moving_shells<S>() > 1) {
@@ -347,7 +424,7 @@ __device__ __forceinline__ void collide_pair(const float (&g)[S::Q][V], float (&
         }
     });
     const float2 omm = splat2(cf.one_minus_omega);
-    static_for<S::Q>([&](auto I) {
+    static_for_carried<S>([&](auto I) {
         constexpr int i = decltype(I)::value;
         constexpr int t = S::shell(i);
         float2 eq = B[t];
@@ -367,6 +444,53 @@ __device__ __forceinline__ void collide_pair(const float (&g)[S::Q][V], float (&
         out[i][K] = r.x;
         out[i][K + 1] = r.y;
     });
+}
+
+template <class S, int K, int V>
+__device__ __forceinline__ void collide_axis_pair(const float (&g)[S::Q][V], float (&out)[S::Q][V],
+                                                  const CollideCoef<float> &cf) {
+            const float w = cf.M[1][1];
+            auto in = [&](int i) { return make_float2(g[i][K], g[i][K + 1]); };
+            auto put = [&](int i, float c, float2 t) {
+                const float2 r = __ffma2_rn(splat2(c), t, in(i));
+                out[i][K] = r.x;
+                out[i][K + 1] = r.y;
+            };
+            if constexpr (S::D == 1) {
+    #pragma unroll
+                for (int i = 1; i < 3; ++i) {
+                    out[i][K] = g[i][K];
+                    out[i][K + 1] = g[i][K + 1];
+                }
+            } else if constexpr (S::D == 2) {
+                const float2 d = __fadd2_rn(__fadd2_rn(in(3), in(4)), neg2(__fadd2_rn(in(1), in(2))));
+                put(1, w, d);
+                put(2, w, d);
+                put(3, -w, d);
+                put(4, -w, d);
+            } else {
+                const float2 sx = __fadd2_rn(in(1), in(2)), sy = __fadd2_rn(in(3), in(4)), sz = __fadd2_rn(in(5), in(6));
+                const float2 P = __fadd2_rn(__fadd2_rn(sx, sy), sz), m3 = splat2(-3.0f);
+                const float2 tx = __ffma2_rn(m3, sx, P), ty = __ffma2_rn(m3, sy, P), tz = __ffma2_rn(m3, sz, P);
+                put(1, w, tx);
+                put(2, w, tx);
+                put(3, w, ty);
+                put(4, w, ty);
+                put(5, w, tz);
+                put(6, w, tz);
+            }
+}
+
+template <class S, int K, int V>
+__device__ __forceinline__ void collide_pair(const float (&g)[S::Q][V], float (&out)[S::Q][V],
+                                             const CollideCoef<float> &cf) {
+    static_assert(K + 1 < V, "a pair needs two cells");
+    if constexpr (rest_static<S>()) {
+        out[0][K] = g[0][K];
+        out[0][K + 1] = g[0][K + 1];
+    }
+    if constexpr (axis_set<S>()) collide_axis_pair<S, K>(g, out, cf);
+    else collide_shells_pair<S, K>(g, out, cf);
 }
 
 // All V cells of a chunk: FP32 pairs on the packed path, anything else one cell at a time (both
@@ -422,7 +546,7 @@ __device__ __forceinline__ void stream_collide_chunk(const T *__restrict__ src, 
     const bool has_right = (lane < 31) && (xc < gd.nxc - 1);
 
     C pull[S::Q][V];
-    static_for<S::Q>([&](auto I) {
+    static_for_carried<S>([&](auto I) {
         constexpr int i = decltype(I)::value;
         constexpr int cx = S::c(i, 0), cy = S::c(i, 1), cz = S::c(i, 2);
         int ys = y - cy, zs = z - cz;
@@ -501,7 +625,13 @@ __device__ __forceinline__ void stream_collide_chunk(const T *__restrict__ src, 
             for (int k = 0; k < V; ++k) {
                 const C damp = sponge_factor<C>(x0 + k, y, z, gd, S::D, ob.sponge_w, ob.sponge_smax);
 #pragma unroll
-                for (int i = 0; i < S::Q; ++i) post[i][k] *= damp;
+                for (int i = rest_static<S>() ? 1 : 0; i < S::Q; ++i) post[i][k] *= damp;
+                if constexpr (rest_static<S>()) {  // the frame damps its rest populations too
+                    if (active && damp != C(1)) {
+                        const long long x = ((long long)z * gd.ny + y) * gd.nx + x0 + k;
+                        dst[x] = Store<T>::make(Store<T>::load(src[x]) * damp);
+                    }
+                }
             }
         }
     }
@@ -512,7 +642,7 @@ __device__ __forceinline__ void stream_collide_chunk(const T *__restrict__ src, 
             if (ob.skip_border) {
                 if (y == 0 || y == gd.ny - 1) return;
                 if (x0 == 0 || x0 + V >= gd.nx) {  // a chunk that holds x = 0 or x = nx - 1
-                    static_for<S::Q>([&](auto I) {
+                    static_for_carried<S>([&](auto I) {
                         constexpr int i = decltype(I)::value;
 #pragma unroll
                         for (int k = 0; k < V; ++k) {
@@ -524,7 +654,7 @@ __device__ __forceinline__ void stream_collide_chunk(const T *__restrict__ src, 
                 }
             }
         }
-        static_for<S::Q>([&](auto I) {
+        static_for_carried<S>([&](auto I) {
             constexpr int i = decltype(I)::value;
             store_vec<T, V>(outp + (long long)i * gd.pitch, post[i]);
         });
@@ -693,7 +823,7 @@ __device__ __forceinline__ void tb_tile(const float *__restrict__ src, float *__
         const int a = y0 - 1 + 4 * k + warp;
         if (a <= y0 + H) {
             const int rows[3] = {rn == 0 ? ny - 1 : rn - 1, rn, rn + 1 == ny ? 0 : rn + 1};  // a-1, a, a+1
-            static_for<Q>([&](auto I) {
+            static_for_carried<S>([&](auto I) {
                 constexpr int i = decltype(I)::value;
                 constexpr int cx = S::c(i, 0), cy = S::c(i, 1);
                 const float *rowp = src + (long long)i * pitch + (long long)rows[1 - cy] * nx;
@@ -715,7 +845,7 @@ __device__ __forceinline__ void tb_tile(const float *__restrict__ src, float *__
             // one lane per 128-byte line of the warp's 512 bytes, only for rows the tile needs
             if ((lane & 7) == 0 && a + 4 <= y0 + H) {
                 const int rows2[3] = {rn == 0 ? ny - 1 : rn - 1, rn, rn + 1 == ny ? 0 : rn + 1};
-                static_for<Q>([&](auto I) {
+                static_for_carried<S>([&](auto I) {
                     constexpr int i = decltype(I)::value;
                     constexpr int cy = S::c(i, 1);
                     prefetch_l2(src + (long long)i * pitch + (long long)rows2[1 - cy] * nx + xa);
@@ -728,7 +858,7 @@ __device__ __forceinline__ void tb_tile(const float *__restrict__ src, float *__
     // B_k: S(t+2) row b from S(t+1) rows b-1 .. b+1 of the ring, collided and stored.
     auto pass_b = [&](int b) {
         float pb[Q][kTbV];
-        static_for<Q>([&](auto I) {
+        static_for_carried<S>([&](auto I) {
             constexpr int i = decltype(I)::value;
             constexpr int cx = S::c(i, 0), cy = S::c(i, 1);
             const int rr = b - cy - (y0 - 1);  // row within the S(t+1) blocks
@@ -739,7 +869,7 @@ __device__ __forceinline__ void tb_tile(const float *__restrict__ src, float *__
         if (b < ny && x0 + kTbV * lane < nx) {
             float *outp = dst + (long long)b * nx + x0 + kTbV * lane;
 #pragma unroll
-            for (int i = 0; i < Q; ++i) tb_st(outp + (long long)i * pitch, post[i]);
+            for (int i = 1; i < Q; ++i) tb_st(outp + (long long)i * pitch, post[i]);
         }
     };
 
@@ -747,7 +877,7 @@ __device__ __forceinline__ void tb_tile(const float *__restrict__ src, float *__
         const int a = y0 - 1 + 4 * k + warp;
         if (a <= y0 + H) {  // warp-uniform; rows past y0 + H are not needed
             float pa[Q][kTbV];
-            static_for<Q>([&](auto I) {
+            static_for_carried<S>([&](auto I) {
                 constexpr int i = decltype(I)::value;
                 constexpr int cx = S::c(i, 0);
                 const float4 t = pre.t[i];
@@ -766,14 +896,14 @@ __device__ __forceinline__ void tb_tile(const float *__restrict__ src, float *__
             float post[Q][kTbV];
             collide_chunk<S, kTbPacked>(pa, post, cf);
 #pragma unroll
-            for (int i = 0; i < Q; ++i) tb_st(r1(k, warp, i) + kTbV * lane + 4, post[i]);
+            for (int i = 1; i < Q; ++i) tb_st(r1(k, warp, i) + kTbV * lane + 4, post[i]);
             // the two halo columns of S(t+1), x0 - 1 (offset 3) and x0 + 128 (offset kTbW + 4), as
             // one pair in lane 0
             if (lane == 0) {
                 float q1[Q][2];
                 collide_chunk<S, kTbPacked>(pre.halo, q1, cf);
 #pragma unroll
-                for (int i = 0; i < Q; ++i) {
+                for (int i = 1; i < Q; ++i) {
                     r1(k, warp, i)[3] = q1[i][0];
                     r1(k, warp, i)[kTbW + 4] = q1[i][1];
                 }
@@ -975,7 +1105,7 @@ __device__ __forceinline__ void tbk_tile(const typename IO::Elem *__restrict__ s
         const int a = y0 - (K - 1) + 4 * k + w1;
         if (a <= lim1) {
             const int rows[3] = {rn == 0 ? ny - 1 : rn - 1, rn, rn + 1 == ny ? 0 : rn + 1};  // a-1, a, a+1
-            static_for<Q>([&](auto I) {
+            static_for_carried<S>([&](auto I) {
                 constexpr int i = decltype(I)::value;
                 constexpr int cx = S::c(i, 0), cy = S::c(i, 1);
                 const long long rb = (long long)i * pitch + (long long)rows[1 - cy] * nx;
@@ -1007,7 +1137,7 @@ __device__ __forceinline__ void tbk_tile(const typename IO::Elem *__restrict__ s
         rows[2] = ring(l - 1, (4 * jp + w + 2) & 7);
     };
     auto pull_level = [&](const float *const (&rows)[3], float (&pb)[Q][kTbV]) {
-        static_for<Q>([&](auto I) {
+        static_for_carried<S>([&](auto I) {
             constexpr int i = decltype(I)::value;
             constexpr int cx = S::c(i, 0), cy = S::c(i, 1);
             tb_pull<cx>(rows[1 - cy] + i * kTbRow, lane, pb[i]);
@@ -1015,7 +1145,7 @@ __device__ __forceinline__ void tbk_tile(const typename IO::Elem *__restrict__ s
     };
     // the halo cell at offset o, pulled from level l-1
     auto pull_halo = [&](const float *const (&rows)[3], int o, float (&hin)[Q][1]) {
-        static_for<Q>([&](auto I) {
+        static_for_carried<S>([&](auto I) {
             constexpr int i = decltype(I)::value;
             constexpr int cx = S::c(i, 0), cy = S::c(i, 1);
             hin[i][0] = rows[1 - cy][i * kTbRow + 4 + o - cx];
@@ -1030,7 +1160,7 @@ __device__ __forceinline__ void tbk_tile(const typename IO::Elem *__restrict__ s
         if (!halo_warp) {
             if (4 * k + warp <= H - 1 + 2 * (K - 1)) {
                 float pa[Q][kTbV];
-                static_for<Q>([&](auto I) {
+                static_for_carried<S>([&](auto I) {
                     constexpr int i = decltype(I)::value;
                     constexpr int cx = S::c(i, 0);
                     float t[kTbV];
@@ -1051,17 +1181,17 @@ __device__ __forceinline__ void tbk_tile(const typename IO::Elem *__restrict__ s
                 collide_chunk<S, kTbPacked>(pa, post, cf);
                 float *dst1 = ring(1, 4 * kp + warp);
 #pragma unroll
-                for (int i = 0; i < Q; ++i) tb_st(dst1 + i * kTbRow + kTbV * lane + 4, post[i]);
+                for (int i = 1; i < Q; ++i) tb_st(dst1 + i * kTbRow + kTbV * lane + 4, post[i]);
             }
         } else if (4 * k + w1 <= H - 1 + 2 * (K - 1)) {
             float hin[Q][1], hout[Q][1];
 #pragma unroll
-            for (int i = 0; i < Q; ++i) hin[i][0] = IO::cvt1(pre.halo[i]);
+            for (int i = 1; i < Q; ++i) hin[i][0] = IO::cvt1(pre.halo[i]);
             collide_chunk<S, kTbPacked>(hin, hout, cf);
             if (lane < 8 * h1) {
                 float *dst1 = ring(1, (4 * kp + w1) & 7);
 #pragma unroll
-                for (int i = 0; i < Q; ++i) dst1[i * kTbRow + 4 + o1] = hout[i][0];
+                for (int i = 1; i < Q; ++i) dst1[i * kTbRow + 4 + o1] = hout[i][0];
             }
         }
         if (k + 1 < iters) load_a(k + 1);
@@ -1080,7 +1210,7 @@ __device__ __forceinline__ void tbk_tile(const typename IO::Elem *__restrict__ s
                     collide_chunk<S, kTbPacked>(pb, post, cf);
                     float *dstl = ring(l, 4 * jp + warp);
 #pragma unroll
-                    for (int i = 0; i < Q; ++i) tb_st(dstl + i * kTbRow + kTbV * lane + 4, post[i]);
+                    for (int i = 1; i < Q; ++i) tb_st(dstl + i * kTbRow + kTbV * lane + 4, post[i]);
                 }
             } else {
                 const int wh = hrow(h), o = hoff(h);
@@ -1093,7 +1223,7 @@ __device__ __forceinline__ void tbk_tile(const typename IO::Elem *__restrict__ s
                     if (lane < 8 * h) {
                         float *dstl = ring(l, (4 * jp + wh) & 7);
 #pragma unroll
-                        for (int i = 0; i < Q; ++i) dstl[i * kTbRow + 4 + o] = hout[i][0];
+                        for (int i = 1; i < Q; ++i) dstl[i * kTbRow + 4 + o] = hout[i][0];
                     }
                 }
             }
@@ -1110,7 +1240,7 @@ __device__ __forceinline__ void tbk_tile(const typename IO::Elem *__restrict__ s
             const bool st = d < ny && x0 + kTbV * lane < nx;
             const long long ob = (long long)d * nx + x0 + kTbV * lane;
 #pragma unroll
-            for (int i = 0; i < Q; ++i) IO::st4(dst, pitch, (long long)i * pitch + ob, post[i], st);
+            for (int i = 1; i < Q; ++i) IO::st4(dst, pitch, (long long)i * pitch + ob, post[i], st);
         }
     };
     int k = 0;

@@ -556,9 +556,9 @@ lee_status lee_lbm_init_fields(lee_lbm *h, const double *rho, const double *u, c
         h->scale = S;
     }
     const SetConsts k = consts_for(h->cfg.set, h->scale);
-    LEE_CK(h, h->ops->init(h->cfg.storage, dr, du, dt, state(h, 0), h->cells, h->pitch, k, h->st), "init kernel");
+    LEE_CK(h, h->ops->init(h->cfg.storage, dr, du, dt, state(h, 0), state(h, 1), h->cells, h->pitch, k, h->st), "init kernel");
     if (sponge_active(h))
-        LEE_CK(h, h->ops->sponge_damp(h->cfg.storage, h->buf[0], (int)h->cfg.nx, (int)h->cfg.ny, (int)h->cfg.nz, h->pitch,
+        LEE_CK(h, h->ops->sponge_damp(h->cfg.storage, h->buf[0], h->buf[1], (int)h->cfg.nx, (int)h->cfg.ny, (int)h->cfg.nz, h->pitch,
                                       h->cfg.sponge_width, h->cfg.sponge_strength, h->st),
                "sponge damp");
     h->cur = 0;
@@ -786,7 +786,7 @@ lee_status lee_lbm_set_populations(lee_lbm *h, const double *g, int32_t on_devic
         src = h->pops64;
     }
     h->cur = 0;
-    LEE_CK(h, h->ops->import_f64(h->cfg.storage, src, h->cells, h->pitch, k, state(h, 0), h->st), "import");
+    LEE_CK(h, h->ops->import_f64(h->cfg.storage, src, h->cells, h->pitch, k, state(h, 0), state(h, 1), h->st), "import");
     h->steps = 0;
     if (!on_device) LEE_SYNC(h);
     return LEE_OK;
@@ -806,7 +806,14 @@ lee_status lee_lbm_set_boundary_mlp(lee_lbm *h, const float *params, int64_t npa
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
     cudaFree(tmp);
     LEE_CK(h, e, "install network");
-    if (!h->mlp_ready) drop_step_graphs(h);  // from the fallback edge to the network
+    if (!h->mlp_ready) {  // from the fallback edge to the network
+        drop_step_graphs(h);
+        // the fallback's frame damps rest populations from copy to copy; the learned step leaves them
+        // alone, so both copies must hold the current ones
+        LEE_CK(h, cudaMemcpyAsync(h->buf[h->cur ^ 1], h->buf[h->cur], h->elem * (size_t)h->cells, cudaMemcpyDeviceToDevice,
+                                  h->st),
+               "copy of the rest populations");
+    }
     h->mlp_ready = true;
     return LEE_OK;
 }

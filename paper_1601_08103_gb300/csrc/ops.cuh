@@ -59,9 +59,11 @@ struct SetOps {
     // and kernel (tma = 1: the TMA-fed tile, which also needs t3t_eligible grids)
     cudaError_t (*step3d2)(const StepLaunch &);
     cudaError_t (*step3d2_prepare)(int storage, int tma);
-    // g = g^eq(fields) (fields FP64 on device)
-    cudaError_t (*init)(int storage, const double *rho, const double *u, const double *theta, void *g, long long cells,
-                        long long pitch, const SetConsts &k, cudaStream_t st);
+    // g = g^eq(fields) (fields FP64 on device).  init, import_f64 and sponge_damp write a whole state
+    // copy g; `other` is the other copy, whose rest populations they write too where a step leaves
+    // those alone (rest_static)
+    cudaError_t (*init)(int storage, const double *rho, const double *u, const double *theta, void *g, void *other,
+                        long long cells, long long pitch, const SetConsts &k, cudaStream_t st);
     // max |g^eq / f*| of the fields into *maxbits (float bits; caller zeroes it)
     cudaError_t (*init_maxabs)(const double *rho, const double *u, const double *theta, long long cells, const SetConsts &k,
                                unsigned int *maxbits, cudaStream_t st);
@@ -73,7 +75,7 @@ struct SetOps {
     cudaError_t (*export_f64)(int storage, const void *g, long long cells, long long pitch, const SetConsts &k, double *out,
                               cudaStream_t st);
     cudaError_t (*import_f64)(int storage, const double *in, long long cells, long long pitch, const SetConsts &k, void *g,
-                              cudaStream_t st);
+                              void *other, cudaStream_t st);
     // all steps of a small 1D grid in one launch, in place on g (nullptr for 2D/3D sets);
     // returns cudaErrorInvalidValue when the grid does not fit in shared memory
     cudaError_t (*onchip_1d)(const StepLaunch &L, void *g, long long nsteps);
@@ -89,8 +91,8 @@ struct SetOps {
     cudaError_t (*slab_unpack)(int storage, void *g, long long pitch, long long plane, int nl, const void *recv_lo,
                                const void *recv_hi, cudaStream_t st);
     // sponge-frame damping of a stored state (after init_fields)
-    cudaError_t (*sponge_damp)(int storage, void *g, int nx, int ny, int nz, long long pitch, int w, double smax,
-                               cudaStream_t st);
+    cudaError_t (*sponge_damp)(int storage, void *g, void *other, int nx, int ny, int nz, long long pitch, int w,
+                               double smax, cudaStream_t st);
     // description for lee_velset_info
     int c[27][3];
     int shell[27];

@@ -76,8 +76,8 @@ struct SetImpl {
             return launch_step_t<S, T>(L);
         });
     }
-    static cudaError_t init(int storage, const double *rho, const double *u, const double *theta, void *g, long long cells,
-                            long long pitch, const SetConsts &k, cudaStream_t st) {
+    static cudaError_t init(int storage, const double *rho, const double *u, const double *theta, void *g, void *other,
+                            long long cells, long long pitch, const SetConsts &k, cudaStream_t st) {
         if (storage == LEE_STORE_SPLIT16) {
             k_split_init<S><<<aux_blocks(cells), 256, 0, st>>>(rho, u, theta, SplitView<S>::m(g),
                                                                SplitView<S>::n(g, pitch), cells, pitch, k);
@@ -86,11 +86,11 @@ struct SetImpl {
         return with_storage(storage, [&](auto *tp) {
             using T = std::remove_pointer_t<decltype(tp)>;
             if constexpr (std::is_same<T, Bfp16>::value)
-                k_init_equilibrium_bfp<S><<<aux_blocks(cells), 256, 0, st>>>(rho, u, theta, static_cast<T *>(g), cells,
-                                                                              pitch, k);
+                k_init_equilibrium_bfp<S><<<aux_blocks(cells), 256, 0, st>>>(
+                    rho, u, theta, static_cast<T *>(g), static_cast<T *>(other), cells, pitch, k);
             else
-                k_init_equilibrium<S, T><<<aux_blocks(cells), 256, 0, st>>>(rho, u, theta, static_cast<T *>(g), cells,
-                                                                            pitch, k);
+                k_init_equilibrium<S, T><<<aux_blocks(cells), 256, 0, st>>>(
+                    rho, u, theta, static_cast<T *>(g), static_cast<T *>(other), cells, pitch, k);
             return cudaGetLastError();
         });
     }
@@ -138,7 +138,7 @@ struct SetImpl {
         });
     }
     static cudaError_t import_f64(int storage, const double *in, long long cells, long long pitch, const SetConsts &k,
-                                  void *g, cudaStream_t st) {
+                                  void *g, void *other, cudaStream_t st) {
         if (storage == LEE_STORE_SPLIT16) {
             k_split_import<S><<<aux_blocks(cells), 256, 0, st>>>(in, cells, pitch, k, SplitView<S>::m(g),
                                                                  SplitView<S>::n(g, pitch));
@@ -147,9 +147,11 @@ struct SetImpl {
         return with_storage(storage, [&](auto *tp) {
             using T = std::remove_pointer_t<decltype(tp)>;
             if constexpr (std::is_same<T, Bfp16>::value)
-                k_import_bfp<S><<<aux_blocks(cells), 256, 0, st>>>(in, cells, pitch, static_cast<T *>(g));
+                k_import_bfp<S><<<aux_blocks(cells), 256, 0, st>>>(in, cells, pitch, static_cast<T *>(g),
+                                                                   static_cast<T *>(other));
             else
-                k_import<S, T><<<aux_blocks(cells), 256, 0, st>>>(in, cells, pitch, k, static_cast<T *>(g));
+                k_import<S, T><<<aux_blocks(cells), 256, 0, st>>>(in, cells, pitch, k, static_cast<T *>(g),
+                                                                  static_cast<T *>(other));
             return cudaGetLastError();
         });
     }
@@ -180,16 +182,18 @@ struct SetImpl {
             }
         });
     }
-    static cudaError_t sponge_damp(int storage, void *g, int nx, int ny, int nz, long long pitch, int w, double smax,
-                                   cudaStream_t st) {
+    static cudaError_t sponge_damp(int storage, void *g, void *other, int nx, int ny, int nz, long long pitch, int w,
+                                   double smax, cudaStream_t st) {
         return with_storage(storage, [&](auto *tp) {
             using T = std::remove_pointer_t<decltype(tp)>;
             using C = typename Store<T>::C;
             GridDesc gd{nx, ny, nz, nx, (long long)nx * ny * nz, pitch};
             if constexpr (std::is_same<T, Bfp16>::value)
-                k_sponge_damp_bfp<S><<<aux_blocks(gd.nchunks), 256, 0, st>>>(static_cast<T *>(g), gd, w, (C)smax);
+                k_sponge_damp_bfp<S><<<aux_blocks(gd.nchunks), 256, 0, st>>>(static_cast<T *>(g), static_cast<T *>(other),
+                                                                             gd, w, (C)smax);
             else
-                k_sponge_damp<S, T><<<aux_blocks(gd.nchunks), 256, 0, st>>>(static_cast<T *>(g), gd, w, (C)smax);
+                k_sponge_damp<S, T><<<aux_blocks(gd.nchunks), 256, 0, st>>>(static_cast<T *>(g), static_cast<T *>(other), gd,
+                                                                            w, (C)smax);
             return cudaGetLastError();
         });
     }

@@ -110,11 +110,11 @@ __global__ void __launch_bounds__((TY + 2) * 32, 1) k_stream_collide_3d2(const T
     const long long plane = (long long)nx * ny;
 
     // level-1 state carried between iterations (FP32 values of the stored type)
-    float r1[kT3V], px1[kT3V], mx1[kT3V];  // plane p1 - 1: rest, +x, -x
+    float px1[kT3V], mx1[kT3V];            // plane p1 - 1: +x, -x
     float hpx1 = 0.f, hmx1 = 0.f;          // plane p1 - 1: +x of the halo cell (lane 0), -x (lane 1)
     float pz1[kT3V], pz2[kT3V];            // +z of planes p1 - 1 and p1 - 2
 #pragma unroll
-    for (int e = 0; e < kT3V; ++e) r1[e] = px1[e] = mx1[e] = pz1[e] = pz2[e] = 0.f;
+    for (int e = 0; e < kT3V; ++e) px1[e] = mx1[e] = pz1[e] = pz2[e] = 0.f;
 
     const int iters = HZ + 2;
     // Level-1 inputs of plane p: the lane's vectors, the tile-edge element (lanes 0 and 31) and
@@ -134,7 +134,7 @@ __global__ void __launch_bounds__((TY + 2) * 32, 1) k_stream_collide_3d2(const T
     using Raw = std::conditional_t<kBfp, InBfp, In>;
     auto load_in = [&](int p, Raw &in) {
         const int pl[3] = {wrap(p - 1, nz), wrap(p, nz), wrap(p + 1, nz)};
-        static_for<Q>([&](auto I) {
+        static_for_carried<S>([&](auto I) {
             constexpr int i = decltype(I)::value;
             constexpr int cx = S::c(i, 0), cy = S::c(i, 1), cz = S::c(i, 2);
             const long long ri = (long long)i * pitch + pl[1 - cz] * plane + (long long)rows[1 - cy] * nx;
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__((TY + 2) * 32, 1) k_stream_collide_3d2(const T
     };
     auto widen = [&](const Raw &r, In &o) {
         if constexpr (kBfp) {
-            static_for<Q>([&](auto I) {
+            static_for_carried<S>([&](auto I) {
                 constexpr int i = decltype(I)::value;
                 constexpr int cx = S::c(i, 0);
                 const BfpDec k = bfp_dec(r.e[i]);
@@ -185,7 +185,7 @@ __global__ void __launch_bounds__((TY + 2) * 32, 1) k_stream_collide_3d2(const T
     auto prefetch_plane = [&](int p) {
         if ((lane & 7) == 0) {
             const int pl[3] = {wrap(p - 1, nz), wrap(p, nz), wrap(p + 1, nz)};
-            static_for<Q>([&](auto I) {
+            static_for_carried<S>([&](auto I) {
                 constexpr int i = decltype(I)::value;
                 constexpr int cy = S::c(i, 1), cz = S::c(i, 2);
                 prefetch_l2(src + (long long)i * pitch + pl[1 - cz] * plane + (long long)rows[1 - cy] * nx + xa);
@@ -202,7 +202,7 @@ __global__ void __launch_bounds__((TY + 2) * 32, 1) k_stream_collide_3d2(const T
         if (k + 1 < iters) load_in(p1 + 1, nxt);
         if (k + 2 < iters) prefetch_plane(p1 + 2);
         float pa[Q][kT3V], hin[Q][1];
-        static_for<Q>([&](auto I) {
+        static_for_carried<S>([&](auto I) {
             constexpr int i = decltype(I)::value;
             constexpr int cx = S::c(i, 0);
             const float *v = cur.v[i];
@@ -229,7 +229,7 @@ __global__ void __launch_bounds__((TY + 2) * 32, 1) k_stream_collide_3d2(const T
         collide_chunk<S, true>(hin, hout, cf);
         if constexpr (!kBfp) {  // a stored state (BFP16 keeps level 1 in FP32: one rounding per launch)
 #pragma unroll
-            for (int i = 0; i < Q; ++i) {
+            for (int i = 1; i < Q; ++i) {
 #pragma unroll
                 for (int e = 0; e < kT3V; ++e) post[i][e] = t3_round<T>(post[i][e]);
                 hout[i][0] = t3_round<T>(hout[i][0]);
@@ -253,7 +253,6 @@ __global__ void __launch_bounds__((TY + 2) * 32, 1) k_stream_collide_3d2(const T
             const float hright = __shfl_sync(kFull, hmx1, 1);
 #pragma unroll
             for (int e = 0; e < kT3V; ++e) {
-                pb[iR][e] = r1[e];
                 pb[iPZ][e] = pz2[e];
                 pb[iMZ][e] = post[iMZ][e];
             }
@@ -270,14 +269,14 @@ __global__ void __launch_bounds__((TY + 2) * 32, 1) k_stream_collide_3d2(const T
             const bool st = y < ny && p2 < nz && x0 + kT3V * lane < nx;
             const long long oi = (long long)p2 * plane + (long long)y * nx + x0 + kT3V * lane;
             if constexpr (kBfp) {  // every lane takes part in the block exponents of its pair
-                static_for<Q>([&](auto I) {
+                static_for_carried<S>([&](auto I) {
                     constexpr int i = decltype(I)::value;
                     const long long e = (long long)i * pitch + oi;
                     bfp_store_vec<kT3V>(dst + e, bfp_exps<Q>(dst, pitch) + (e >> 3), out[i], st);
                 });
             } else if (st) {
                 T *outp = dst + oi;
-                static_for<Q>([&](auto I) {
+                static_for_carried<S>([&](auto I) {
                     constexpr int i = decltype(I)::value;
                     store_vec<T, kT3V>(outp + (long long)i * pitch, out[i]);
                 });
@@ -286,7 +285,6 @@ __global__ void __launch_bounds__((TY + 2) * 32, 1) k_stream_collide_3d2(const T
         // ---- carry level 1 of plane p1 to the next iteration
 #pragma unroll
         for (int e = 0; e < kT3V; ++e) {
-            r1[e] = post[iR][e];
             px1[e] = post[iPX][e];
             mx1[e] = post[iMX][e];
             pz2[e] = pz1[e];
