@@ -35,17 +35,23 @@ NSTEPS = 1000
 TAU = 0.6
 SET = "D2Q5"
 STORAGE = "f32"
-BYTES_PER_LUP = 2 * 5 * 4  # read + write of q = 5 FP32 populations (algorithmic)
+BYTES_PER_LUP = 2 * 4 * 4  # read + write of the four moving FP32 populations (a step leaves the rest ones alone)
 L2_FLUSH_BYTES = 512 << 20
 NOMINAL_HBM_GBS = 8000.0  # HBM3e nominal bandwidth of the part (the measured copy peak is the denominator of frac)
 WORKLOAD = "2D D2Q5 periodic 2048x2048, FP32, tau=0.6, pulse+8 plane waves, 1000 steps/job"
 METRIC = "MLUPS (2D D2Q5 FP32 stream-collide job) and fraction of HBM roofline"
 # ncu summary of the stream-collide kernel the benchmark runs, by time steps fused per launch
-PROFILES = {k: os.path.join(ROOT, "profiles", f"stream_collide_{k}step_d2q5_f32_2048x2048.md") for k in (1, 2, 3, 4)}
-KERNEL_NAMES = {1: "k_stream_collide<D2Q5,float,V=4,periodic>", 2: "k_stream_collide_2step<D2Q5,float>",
-                3: "k_stream_collide_kstep<D2Q5,K=3,float>", 4: "k_stream_collide_kstep<D2Q5,K=4,float>"}
-KERNEL_SOURCES = ["paper_1601_08103_gb300/csrc/kernels.cuh", "paper_1601_08103_gb300/csrc/step_launch.cuh",
-                  "paper_1601_08103_gb300/csrc/velsets.cuh"]
+PROFILES = {8: os.path.join(ROOT, "profiles", "row_pipe_8step_d2q5_f32_2048x2048.md")}
+KERNEL_NAMES = {1: "k_stream_collide<D2Q5,float,V=4,periodic>", 8: "k_row_pipe<8,RpF32>"}
+KERNEL_SOURCES = ["paper_1601_08103_gb300/csrc/kernels.cuh", "paper_1601_08103_gb300/csrc/rowpipe.cuh",
+                  "paper_1601_08103_gb300/csrc/step_launch.cuh", "paper_1601_08103_gb300/csrc/velsets.cuh"]
+
+
+def steps_of_launch(sv) -> int:
+    """Time steps per launch of a long run: grids that fuse runs of four take two such runs (eight steps)
+    in one launch."""
+    spl = max(sv.steps_per_launch, 1)
+    return 8 if spl == 4 else spl
 
 
 def kernel_source_sha() -> str:
@@ -211,12 +217,10 @@ def run_ours(args, rank, world, local):
     flush = torch.empty(L2_FLUSH_BYTES // 4, dtype=torch.float32, device=dev)
     sv = lee.Solver(SET, (NX, NX, 1), TAU, storage=STORAGE, stream=stream)
 
-    # steps per stream-collide launch: 4 for this periodic 2D FP32 grid (four fused time steps
-    # per launch, the intermediate states in shared memory), 1 for the one-step kernel.  A job of
-    # NSTEPS steps is NSTEPS // spl fused launches and NSTEPS % spl single steps; every launch reads
-    # and writes the whole state once, so each moves the same algorithmic bytes.
-    spl = max(sv.steps_per_launch, 1)
-    step_launches = NSTEPS // spl + NSTEPS % spl
+    # a job of NSTEPS steps is NSTEPS // spl launches of spl steps, and one of the rest; every launch
+    # reads and writes the moving populations once
+    spl = steps_of_launch(sv)
+    step_launches = -(-NSTEPS // spl)
     launches_per_step = 1 + step_launches + 1 + 2  # init, steps, moments, reduce (partial + final)
 
     def one_step(ev):
@@ -307,7 +311,7 @@ def run_ours(args, rank, world, local):
                      "update_bound_mlups": round(peak / (BYTES_PER_LUP / spl) * 1e3, 1),
                      "kernel": KERNEL_NAMES.get(spl, "?"),
                      "steps_per_launch": spl,
-                     "launches_per_job": {"fused": NSTEPS // spl, "single_step": NSTEPS % spl},
+                     "launches_per_job": {"fused": NSTEPS // spl, "rest_steps": NSTEPS % spl},
                      "algorithmic_bytes_per_launch": BYTES_PER_LUP * cells,
                      "avg_launch_us": round(kernel_avg_s * 1e6, 3)},
         "e2e": {"value": round(e2e_value, 1), "unit": "MLUPS", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
@@ -408,11 +412,11 @@ def forms_3d():
             sv.moments(r, None, None)
             torch.cuda.synchronize()
             ms = e0.elapsed_time(e1)
-            spl = sv.steps_per_launch
+            spl = steps_of_launch(sv)
         if label == "f64":
             ref = r
         err = float(torch.linalg.norm(r - ref) / torch.linalg.norm(ref))
-        bpl = 2 * 7 * lee.STORAGE_BYTES[storage]
+        bpl = 2 * 6 * lee.STORAGE_BYTES[storage]
         out[label] = {"mlups": round(cells * steps / (ms / 1e3) / 1e6, 1),
                         "gbs": round(bpl * cells * steps / (ms / 1e3) / 1e9, 1), "rel_l2_rho_vs_f64": err,
                         "steps_per_launch": spl, "bytes_per_update": round(bpl / max(spl, 1), 3)}
@@ -476,10 +480,10 @@ def forms_mixed_2d(n: int = 8192, steps: int = 1000):
             sv.moments(r, None, None)
             torch.cuda.synchronize()
             ms = e0.elapsed_time(e1)
-            spl = sv.steps_per_launch
+            spl = steps_of_launch(sv)
         if ref is None:
             ref = r
-        bpl = 2 * 5 * lee.STORAGE_BYTES[storage]
+        bpl = 2 * 4 * lee.STORAGE_BYTES[storage]
         out[storage] = {"mlups": round(cells * steps / (ms / 1e3) / 1e6, 1), "steps_per_launch": spl,
                         "bytes_per_update": round(bpl / spl, 3),
                         "gbs_algorithmic_per_launch": round(bpl * cells * steps / spl / (ms / 1e3) / 1e9, 1),
@@ -545,7 +549,7 @@ def forms_configs():
             torch.cuda.synchronize()
             ms = e0.elapsed_time(e1)
             finite = sv.check_finite()
-            spl = sv.steps_per_launch
+            spl = steps_of_launch(sv)
         bpl = 2 * info["q"] * lee.STORAGE_BYTES[storage]
         out[key] = {"cells": cells, "steps": steps, "ms": round(ms, 3), "us_per_step": round(ms * 1e3 / steps, 3),
                     "mlups": round(cells * steps / (ms / 1e3) / 1e6, 1),

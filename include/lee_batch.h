@@ -47,11 +47,12 @@ lee_status lee_batch_init_fields(lee_batch *b, int32_t d, const double *rho, con
 /* Advances every domain n >= 0 steps (Sec. 6).  mode: lee_batch_mode.  The first GRAPH or
  * LAUNCH call runs the autotuner unless lee_batch_set_tuning fixed the launch shape.  In GRAPH
  * mode a run of up to 4096 steps is one launch of a graph holding all its steps (captured on
- * first use of that length and parity, then cached); longer runs replay a 100-step graph.  With
+ * first use of that length and parity, then cached); longer runs replay a 96-step graph.  With
  * FP32 storage and every nx a multiple of 4, GRAPH and LAUNCH modes advance several steps per
- * launch (the intermediate states kept in shared memory; tiles of 128 columns), with the count,
+ * launch (the intermediate states kept in registers; tiles of 112 columns), with the count,
  * tile rows and tile order the autotuner picks (lee_batch_tune_shape; LEE_TB_STEPS=1..4 in the
- * environment at create time fixes the count), bit-identical to single steps. */
+ * environment at create time fixes the count; a count of four that the tuner picked runs eight steps per
+ * launch while a call has that many left), bit-identical to single steps. */
 lee_status lee_batch_step(lee_batch *b, int64_t n, int32_t mode);
 
 /* Per-cell moments of domain d (as lee_lbm_moments).  NULL outputs are skipped. */
@@ -64,7 +65,7 @@ lee_status lee_batch_reduce(lee_batch *b, int32_t d, double *out, int32_t on_dev
 lee_status lee_batch_get_populations(lee_batch *b, int32_t d, double *g, int32_t on_device);
 
 /* Launch shape of a batch: the one-step batched kernel (threads per block, cells per thread) and
- * the fused multi-step kernel (steps per launch; tiles of 128 columns x tile_rows rows; dispatch
+ * the fused multi-step kernel (steps per launch; tiles of 112 columns x tile_rows rows; dispatch
  * order 0 = tiles with the most rows first, 1 = domain by domain).  steps_per_launch = 1 means
  * every step runs the one-step kernel.  us_per_step: the tuner's measurement of one time step of
  * the whole batch with this shape (0 when the shape was set by hand). */

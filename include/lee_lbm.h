@@ -184,25 +184,25 @@ lee_status lee_lbm_create(const lee_lbm_config *cfg, lee_lbm **out);
 lee_status lee_lbm_init_fields(lee_lbm *h, const double *rho, const double *u, const double *theta, int32_t on_device);
 
 /* Advances n >= 0 time steps of the LBE update scheme (Sec. 6): one fused pull-stream + BGK
- * collision kernel per step.  Asynchronous.  For n >= 8 the launches are replayed from a CUDA
- * graph (one graph holding all n steps for n <= 4096, else repeated 100-step graphs), captured on
+ * collision kernel per step.  Asynchronous.  Calls of eight launches or more are replayed from a CUDA
+ * graph (one graph holding all n steps for n <= 4096, else repeated 96-step graphs), captured on
  * first use of that length on a private stream and cached in the handle; results are identical to
  * direct launches.  Every form below also gives the same bits as single one-step launches:
- *  - periodic 2D FP32 grids with nx a multiple of 4 advance four steps per launch, the three
- *    intermediate states kept in shared memory (temporal blocking; LEE_TB_STEPS=1..4 in the
- *    environment at create time picks another count; lee_lbm_steps_per_launch reports it); a
- *    run of n steps is n / 4 such launches and n % 4 single steps;
+ *  - periodic 2D FP32 grids with nx a multiple of 4 advance several steps per launch, the
+ *    intermediate states kept in registers (temporal blocking): eight while the call has that many
+ *    left, then four, then the two or three or one that remain.  LEE_TB_STEPS=1..4 in the
+ *    environment at create time fixes the count instead (n / count launches, n % count single steps);
  *  - periodic 3D FP32 grids of D3Q7 and diatomic D3Q7 with nx a multiple of 4 advance two steps
  *    per launch (a z-marching tile; LEE_TB_STEPS=1 keeps one step per launch);
- *  - BFP16 storage on those periodic 2D grids with nx a multiple of 8 uses the same kernels (four
- *    steps, or three with LEE_TB_STEPS=3), but keeps the intermediate states in FP32 and encodes
- *    only the last one: a launch of k steps equals decoding the state, k FP32 steps and one
- *    encoding, bit for bit (LEE_TB_STEPS=1 or 2 keeps one step per launch, which equals decode,
- *    one FP32 step, encode).  On 3D grids BFP16 runs one step per launch unless LEE_TB_STEPS=2
- *    asks for the two-step tile (nx a multiple of 8), which is slower there;
- *  - FP16 and BF16 storage on periodic 2D grids with nx a multiple of 4 do the same: four (or
- *    three) steps per launch with the intermediate states in FP32, one rounding to the storage per
- *    launch (LEE_TB_STEPS=1 or 2 keeps one step per launch, rounding every step);
+ *  - BFP16 storage on those periodic 2D grids with nx a multiple of 8 uses the same kernels (eight steps
+ *    and four, the rest as single steps; or three or four with LEE_TB_STEPS), but keeps the
+ *    intermediate states in FP32 and encodes only the last one: a launch of k steps equals decoding
+ *    the state, k FP32 steps and one encoding, bit for bit (LEE_TB_STEPS=1 or 2 keeps one step per
+ *    launch, which equals decode, one FP32 step, encode).  On 3D grids BFP16 runs one step per launch
+ *    unless LEE_TB_STEPS=2 asks for the two-step tile (nx a multiple of 8), which is slower there;
+ *  - FP16 and BF16 storage on periodic 2D grids with nx a multiple of 4 do the same, with one
+ *    rounding to the storage per launch (LEE_TB_STEPS=1 or 2 keeps one step per launch, rounding
+ *    every step);
  *  - a 1D grid (not BFP16) whose two population copies fit in shared memory (2 q nx sizeof(storage) <= 227 KB,
  *    e.g. D1Q3 FP64 up to 4843 cells) runs all n >= 2 steps in one launch: one block, or from
  *    512 cells a thread-block cluster of 8 blocks;
@@ -290,13 +290,14 @@ lee_status lee_lbm_boundary_in_use(lee_lbm *h, int32_t *bc);
 lee_status lee_lbm_steps_done(lee_lbm *h, int64_t *steps);
 
 /* How lee_lbm_step runs this grid: *steps = 1 (one fused stream-collide launch per time step),
- * 2..4 (periodic 2D FP32 grids with nx a multiple of 4: that many time steps per launch, the
- * intermediate states kept in shared memory -- temporal blocking; 4 unless LEE_TB_STEPS was set
- * at create time; periodic 3D FP32 D3Q7 and diatomic D3Q7 grids with nx a multiple of 4: 2;
- * BFP16 storage: 3 or 4 in 2D on such grids with nx a multiple of 8, 2 in 3D only with
- * LEE_TB_STEPS=2; FP16 / BF16 storage: 3 or 4 in 2D on such grids) or 0 (small 1D
- * grid: all steps of a call in one on-chip launch).  All forms give bit-identical results, except
- * that BFP16, FP16 and BF16 storage round their state once per launch (see lee_lbm_step). */
+ * 2..4 (that many time steps per launch, the intermediate states kept on the SMs -- temporal blocking)
+ * or 0 (small 1D grid: all steps of a call in one on-chip launch).  Periodic 2D FP32 grids with nx a
+ * multiple of 4: 4 unless LEE_TB_STEPS was set at create time; a call takes two such runs, eight
+ * steps, in one launch where it can (not with LEE_TB_STEPS).  Periodic 3D FP32 D3Q7 and diatomic D3Q7
+ * grids with nx a multiple of 4: 2.  BFP16 storage: 3 or 4 in 2D on such grids with nx a multiple of 8, 2
+ * in 3D only with LEE_TB_STEPS=2; FP16 / BF16 storage: 3 or 4 in 2D on such grids.  All forms give
+ * bit-identical results, except that BFP16, FP16 and BF16 storage round their state once per launch
+ * (see lee_lbm_step). */
 lee_status lee_lbm_steps_per_launch(lee_lbm *h, int32_t *steps);
 
 /* The 16-bit storage scale S in use (1 for F64/F32/BFP16 storage). */

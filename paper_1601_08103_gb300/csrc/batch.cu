@@ -40,43 +40,33 @@ BatchedFn batched_fn(int V) {
     }
 }
 
-template <class S>
-cudaError_t launch_batched_2step(const void *src, void *dst, const void *doms, const void *tiles, int nblocks,
-                                 cudaStream_t st) {
-    k_stream_collide_2step_batched<S><<<nblocks, 128, tb_smem_bytes<S>(), st>>>(
-        static_cast<const float *>(src), static_cast<float *>(dst), static_cast<const TbDomain *>(doms),
-        static_cast<const int3 *>(tiles));
+// The row pipeline over many domains (rowpipe.cuh), K steps per launch.
+template <int K, int kStages>
+cudaError_t launch_batched_pipe(const void *src, void *dst, const void *doms, const void *tiles, int count,
+                                cudaStream_t st) {
+    k_row_pipe_batched<K, kStages>
+        <<<(count + kRpWarps - 1) / kRpWarps, 32 * kRpWarps, rp_smem_bytes<RpF32, kStages>(), st>>>(
+            static_cast<const float *>(src), static_cast<float *>(dst), static_cast<const RpDomain *>(doms),
+            static_cast<const int3 *>(tiles), count);
     return cudaGetLastError();
 }
-
-template <class S, int K>
-cudaError_t launch_batched_kstep(const void *src, void *dst, const void *doms, const void *tiles, int nblocks,
-                                 cudaStream_t st) {
-    k_stream_collide_kstep_batched<S, K><<<nblocks, kTbkThreads, tbk_smem_bytes<S, K>(), st>>>(
-        static_cast<const float *>(src), static_cast<float *>(dst), static_cast<const TbDomain *>(doms),
-        static_cast<const int3 *>(tiles));
-    return cudaGetLastError();
+// Its one-time set-up on the current device (outside any stream capture), and the launcher.
+template <int K>
+cudaError_t prepare_batched_pipe(bool near_l2, BatchedTbFn *fn) {
+    *fn = near_l2 ? &launch_batched_pipe<K, kRpStagesNear> : &launch_batched_pipe<K, kRpStagesFar>;
+    return near_l2 ? cudaFuncSetAttribute(k_row_pipe_batched<K, kRpStagesNear>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          rp_smem_bytes<RpF32, kRpStagesNear>())
+                   : cudaFuncSetAttribute(k_row_pipe_batched<K, kRpStagesFar>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          rp_smem_bytes<RpF32, kRpStagesFar>());
 }
-
-// Sets the shared-memory attribute of the batched multi-step kernel fusing `unit` steps on the
-// current device (outside any stream capture) and returns its launcher.
-template <class S>
-cudaError_t prepare_batched_tb(int unit, lee::BatchedTbFn *fn) {
-    cudaError_t e = cudaErrorInvalidValue;
-    if (unit == 2) {
-        e = cudaFuncSetAttribute(k_stream_collide_2step_batched<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 tb_smem_bytes<S>());
-        *fn = &launch_batched_2step<S>;
-    } else if (unit == 3) {
-        e = cudaFuncSetAttribute(k_stream_collide_kstep_batched<S, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 tbk_smem_bytes<S, 3>());
-        *fn = &launch_batched_kstep<S, 3>;
-    } else if (unit == 4) {
-        e = cudaFuncSetAttribute(k_stream_collide_kstep_batched<S, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 tbk_smem_bytes<S, 4>());
-        *fn = &launch_batched_kstep<S, 4>;
+cudaError_t batched_pipe(int k, bool near_l2, BatchedTbFn *fn) {
+    switch (k) {
+    case 2: return prepare_batched_pipe<2>(near_l2, fn);
+    case 3: return prepare_batched_pipe<3>(near_l2, fn);
+    case 4: return prepare_batched_pipe<4>(near_l2, fn);
+    case kRpDeep: return prepare_batched_pipe<kRpDeep>(near_l2, fn);
+    default: return cudaErrorInvalidValue;
     }
-    return e;
 }
 
 BatchedFn pick_batched(int set, int storage, int V) {
@@ -189,20 +179,22 @@ int full_vec(int storage) { return storage == LEE_STORE_F32 ? 4 : 2; }
 // four-step kernel: 64 rows 374 GLUPS, 48-80 rows 360-366, 128 rows 367, 256 rows 359).
 constexpr int kBatchTileRows = 64;
 
-// Multi-step tiles of 128 columns x `rows` rows (fewer for short domains), in dispatch order
+// Tiles of kRpBatchWidth columns x `rows` rows (fewer for short domains), in dispatch order
 // `order`: 0 = tiles with the most rows first, so that the block scheduler balances the uneven
 // domains; 1 = domain by domain, rows then columns.  Every shape gives the same bits.
 lee_status build_tb(lee_batch *b, int unit, int rows, int order) {
-    cudaError_t e = b->set == LEE_D2Q5 ? prepare_batched_tb<D2Q5>(unit, &b->tb_fn)
-                                       : prepare_batched_tb<D2Q5Di>(unit, &b->tb_fn);
-    if (e != cudaSuccess) return bfail(b, LEE_ERR_CUDA, std::string("multi-step prepare: ") + cudaGetErrorString(e));
-    std::vector<TbDomain> hd(b->count);
+    const bool near_l2 = 8LL * (long long)sizeof(float) * b->total_cells <= kRpNearL2Bytes;
+    b->deep_fn = nullptr;
+    cudaError_t e = batched_pipe(unit, near_l2, &b->tb_fn);
+    if (e == cudaSuccess && unit == 4 && b->unit_fixed == 0) e = batched_pipe(kRpDeep, near_l2, &b->deep_fn);
+    if (e != cudaSuccess) return bfail(b, LEE_ERR_CUDA, std::string("row pipeline prepare: ") + cudaGetErrorString(e));
+    std::vector<RpDomain> hd(b->count);
     struct Tile {
         int rows, d, x0, y0;
     };
     std::vector<Tile> tiles;
     for (int d = 0; d < b->count; ++d) {
-        TbDomain &D = hd[d];
+        RpDomain &D = hd[d];
         D.nx = (int)b->doms[d].nx;
         D.ny = (int)b->doms[d].ny;
         int H = rows;
@@ -214,15 +206,15 @@ lee_status build_tb(lee_batch *b, int unit, int rows, int order) {
         double M[4][4], N[4][4];
         const double omega = omega_for(b->storage, b->doms[d].tau);
         fold_coefficients(b->set, false, omega, M, N);
-        D.cf = make_coef<float>(omega, M, N);
+        D.w = make_coef<float>(omega, M, N).M[1][1];
         for (int y0 = 0; y0 < D.ny; y0 += H)
-            for (int x0 = 0; x0 < D.nx; x0 += kTbW) tiles.push_back({std::min(H, D.ny - y0), d, x0, y0});
+            for (int x0 = 0; x0 < D.nx; x0 += kRpBatchWidth) tiles.push_back({std::min(H, D.ny - y0), d, x0, y0});
     }
     if (order == 0)
         std::stable_sort(tiles.begin(), tiles.end(), [](const Tile &p, const Tile &q) { return p.rows > q.rows; });
     std::vector<int3> ht(tiles.size());
     for (size_t k = 0; k < tiles.size(); ++k) ht[k] = make_int3(tiles[k].d, tiles[k].x0, tiles[k].y0);
-    const size_t db = sizeof(TbDomain) * hd.size(), tb = sizeof(int3) * ht.size();
+    const size_t db = sizeof(RpDomain) * hd.size(), tb = sizeof(int3) * ht.size();
     if (db > b->d_tb_cap) {
         cudaFree(b->d_tb);
         b->d_tb = nullptr;
@@ -352,7 +344,8 @@ lee_status tune(lee_batch *b) {
         lee_status s = LEE_OK;
         auto one = [&]() -> lee_status {
             if (fused) {
-                BCK(b, b->tb_fn(b->buf[b->cur], b->buf[b->cur ^ 1], b->d_tb, b->d_tb_tiles, b->tb_blocks, b->st),
+                const BatchedTbFn fn = b->deep_fn ? b->deep_fn : b->tb_fn;
+                BCK(b, fn(b->buf[b->cur], b->buf[b->cur ^ 1], b->d_tb, b->d_tb_tiles, b->tb_blocks, b->st),
                     "tuning launch");
                 return LEE_OK;
             }
@@ -397,9 +390,10 @@ lee_status tune(lee_batch *b) {
                     if (s != LEE_OK) return s;
                     float us = 0.f;
                     if ((s = timed(6, true, &us)) != LEE_OK) return s;
-                    if (us / unit < best_us) {
-                        best_us = us / unit;
-                        best = BatchShape{one.threads, one.V, unit, rows, order, us / unit};
+                    us /= b->deep_fn ? kRpDeep : unit;
+                    if (us < best_us) {
+                        best_us = us;
+                        best = BatchShape{one.threads, one.V, unit, rows, order, us};
                     }
                 }
         }
@@ -414,11 +408,17 @@ lee_status tune(lee_batch *b) {
     return LEE_OK;
 }
 
-// One launch of the step unit (b->unit fused steps, or one step) reading buffer src_which and
-// writing the other one.
-cudaError_t launch_unit(lee_batch *b, int src_which, cudaStream_t st) {
-    if (b->unit > 1) return b->tb_fn(b->buf[src_which], b->buf[src_which ^ 1], b->d_tb, b->d_tb_tiles, b->tb_blocks, st);
-    return b->fn(b->buf[src_which], b->buf[src_which ^ 1], b->d_doms, b->d_table, b->nblocks, b->threads, st);
+// Steps of the next launch of a run with `left` steps to go (the same bits whatever the sizes).
+int next_launch(const lee_batch *b, int64_t left) {
+    if (b->unit > 1 && b->deep_fn && left >= kRpDeep) return kRpDeep;
+    return left >= b->unit ? b->unit : 1;
+}
+// One launch of k steps reading buffer src_which and writing the other one.
+cudaError_t launch_steps(lee_batch *b, int src_which, int k, cudaStream_t st) {
+    const void *src = b->buf[src_which];
+    void *dst = b->buf[src_which ^ 1];
+    if (k == 1) return b->fn(src, dst, b->d_doms, b->d_table, b->nblocks, b->threads, st);
+    return (k == kRpDeep ? b->deep_fn : b->tb_fn)(src, dst, b->d_tb, b->d_tb_tiles, b->tb_blocks, st);
 }
 
 lee_status ensure_graph(lee_batch *b, int parity, long long steps, cudaGraphExec_t *out) {
@@ -430,15 +430,15 @@ lee_status ensure_graph(lee_batch *b, int parity, long long steps, cudaGraphExec
     cudaGraph_t g = nullptr;
     BCK(b, cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal), "begin capture");
     int w = parity;
-    const int unit = b->unit;
-    for (long long k = 0; k < steps / unit; ++k) {
-        cudaError_t e = launch_unit(b, w, b->cap);
+    for (long long left = steps; left > 0; w ^= 1) {
+        const int k = next_launch(b, left);
+        cudaError_t e = launch_steps(b, w, k, b->cap);
         if (e != cudaSuccess) {
             cudaStreamEndCapture(b->cap, &g);
             if (g) cudaGraphDestroy(g);
             return bfail(b, LEE_ERR_CUDA, std::string("capture launch: ") + cudaGetErrorString(e));
         }
-        w ^= 1;
+        left -= k;
     }
     BCK(b, cudaStreamEndCapture(b->cap, &g), "end capture");
     cudaGraphExec_t ex = nullptr;
@@ -592,27 +592,26 @@ lee_status lee_batch_step(lee_batch *b, int64_t n, int32_t mode) {
         return LEE_OK;
     }
     if (!b->tuned && (s = tune(b)) != LEE_OK) return s;
-    const int unit = b->unit;
-    int64_t units = n / unit;
+    int64_t left = n;
     if (mode == LEE_BATCH_GRAPH) {
-        // up to kMaxGraphSteps steps: one graph of all of them (one launch of the whole run);
-        // longer runs: replays of a kChunkSteps graph.  Graphs hold an even number of launches.
-        const long long gunits = units * unit <= lee_batch::kMaxGraphSteps ? (units & ~1LL)
-                                                                           : (lee_batch::kChunkSteps / unit) & ~1LL;
-        while (gunits > 0 && units >= gunits) {
+        // up to kMaxGraphSteps steps: one graph of all of them (one launch of the whole run); longer
+        // runs: replays of a kChunkSteps graph
+        const int64_t steps = left <= lee_batch::kMaxGraphSteps ? left : lee_batch::kChunkSteps;
+        int flips = 0;
+        for (int64_t r = steps; r > 0; flips ^= 1) r -= next_launch(b, r);
+        while (steps > 1 && left >= steps) {
             cudaGraphExec_t ex = nullptr;
-            if ((s = ensure_graph(b, b->cur, gunits * unit, &ex)) != LEE_OK) return s;
-            BCK(b, cudaGraphLaunch(ex, b->st), "graph launch");  // even number of launches: parity kept
-            units -= gunits;
+            if ((s = ensure_graph(b, b->cur, steps, &ex)) != LEE_OK) return s;
+            BCK(b, cudaGraphLaunch(ex, b->st), "graph launch");
+            b->cur ^= flips;
+            left -= steps;
         }
     }
-    for (; units > 0; --units) {
-        BCK(b, launch_unit(b, b->cur, b->st), "batched launch");
+    while (left > 0) {
+        const int k = next_launch(b, left);
+        BCK(b, launch_steps(b, b->cur, k, b->st), "batched launch");
         b->cur ^= 1;
-    }
-    for (int64_t left = n % unit; left > 0; --left) {
-        if ((s = launch_one(b, b->cur, b->st)) != LEE_OK) return s;
-        b->cur ^= 1;
+        left -= k;
     }
     return LEE_OK;
 }

@@ -314,37 +314,4 @@ __global__ void __launch_bounds__(256) k_stream_collide_bfp(const Bfp16 *__restr
     stream_collide_chunk_bfp<S, V, OPEN>(src, dst, gd, cf, ob, (long long)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
-// K-level 2D tiles (tbk_tile) on BFP16 storage: level 1 decodes S(t) as it pulls it, levels 2 ..
-// K-1 stay FP32 in shared memory, level K encodes S(t+K).  So a launch equals decoding the state,
-// K FP32 steps and one encoding, bit for bit: the state is rounded to 16 bits once per K steps.
-// A lane's 4 cells are half a block (lane pairs share the exponent; nx a multiple of 8).
-template <int Q>
-struct TileIoBfp {
-    using Elem = Bfp16;
-    struct Vec {
-        uint2 m;     // four mantissas
-        unsigned e;  // their block's exponent byte
-    };
-    struct One {
-        unsigned u, e;
-    };
-    __device__ static __forceinline__ Vec ld4(const Bfp16 *__restrict__ base, long long pitch, long long idx) {
-        return Vec{__ldg(reinterpret_cast<const uint2 *>(base + idx)), (unsigned)__ldg(bfp_exps<Q>(base, pitch) + (idx >> 3))};
-    }
-    __device__ static __forceinline__ One ld1(const Bfp16 *__restrict__ base, long long pitch, long long idx) {
-        return One{(unsigned)__ldg(reinterpret_cast<const unsigned short *>(base + idx)),
-                   (unsigned)__ldg(bfp_exps<Q>(base, pitch) + (idx >> 3))};
-    }
-    __device__ static __forceinline__ void cvt4(const Vec &t, float (&v)[4]) {
-        const BfpDec k = bfp_dec(t.e);
-        const float2 a = bfp_pair(t.m.x, k), b = bfp_pair(t.m.y, k);
-        v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
-    }
-    __device__ static __forceinline__ float cvt1(const One &t) { return bfp_val(t.u, bfp_dec(t.e)); }
-    __device__ static __forceinline__ void st4(Bfp16 *__restrict__ base, long long pitch, long long idx, const float (&v)[4],
-                                               bool store) {
-        bfp_store_vec<4>(base + idx, bfp_exps<Q>(base, pitch) + (idx >> 3), v, store);
-    }
-};
-
 }  // namespace lee

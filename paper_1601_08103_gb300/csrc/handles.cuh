@@ -39,8 +39,8 @@ struct lee_lbm {
     int ghost_L = 0;
     void *mlp = nullptr;
     bool mlp_ready = false;
-    // captured step graphs keyed by (starting parity, number of steps), even lengths only, and
-    // the stream they are captured on
+    // captured step graphs keyed by (starting copy, number of steps), and the stream they are
+    // captured on
     std::map<std::pair<int, long long>, cudaGraphExec_t> exec;
     cudaStream_t cap = nullptr;
     // learned edge: the slots of the four corner cells in the one-launch step
@@ -52,7 +52,8 @@ struct lee_lbm {
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     // time steps fused per launch on periodic 2D FP32 grids (temporal blocking): 4 by default;
     // LEE_TB_STEPS=1..4 in the environment at create time overrides it, and LEE_SINGLE_STEP=1
-    // sets 1 (for comparisons between the one-, two-, three- and four-step kernels)
+    // sets 1 (for comparisons between the launch sizes; calls take two runs of four in one launch unless
+    // the count was set)
     int tb_steps = 4;
     bool tb_env = false;  // tb_steps came from LEE_TB_STEPS
     // set by LEE_FORCE_SCALAR=1 at create time: one cell per thread in every step kernel, and one
@@ -110,6 +111,7 @@ struct lee_batch {
     size_t d_tb_cap = 0, d_tb_tiles_cap = 0;
     int tb_blocks = 0;
     lee::BatchedTbFn tb_fn = nullptr;
+    lee::BatchedTbFn deep_fn = nullptr;  // two units of four steps in one launch (nullptr: not taken)
     // fused launch shape: tile rows (a multiple of 4) and dispatch order (0: tiles with the most
     // rows first, 1: domain by domain, row-major); fuse_ok: every domain can take a fused kernel;
     // unit_fixed: steps per launch fixed by the environment at create time (0: the tuner picks)
@@ -117,10 +119,9 @@ struct lee_batch {
     bool fuse_ok = false;
     int unit_fixed = 0;
     float tuned_us_per_step = 0.f;
-    // captured graphs, keyed by (starting parity, number of steps); every graph has an even
-    // number of steps, so replaying it leaves the buffer parity unchanged
+    // captured graphs, keyed by (starting copy, number of steps)
     static constexpr int kMaxGraphSteps = 4096;
-    static constexpr int kChunkSteps = 100;
+    static constexpr int kChunkSteps = 96;  // an even number of launches of every size
     std::map<std::pair<int, long long>, cudaGraphExec_t> exec;
     // aux
     double *fields = nullptr, *pops64 = nullptr, *partial = nullptr, *red_out = nullptr;

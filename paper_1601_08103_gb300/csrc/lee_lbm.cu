@@ -137,7 +137,9 @@ using namespace lee;
 
 namespace {
 
-constexpr long long kGraphMinSteps = 8, kMaxGraphSteps = 4096, kChunkGraphSteps = 100;
+// A call of at least kGraphMinLaunches launches is replayed from a graph.  kChunkGraphSteps: a
+// multiple of every launch size, in an even number of launches.
+constexpr long long kGraphMinLaunches = 8, kMaxGraphSteps = 4096, kChunkGraphSteps = 96;
 
 lee_status fail(lee_lbm *h, lee_status s, const std::string &msg) {
     if (h) {
@@ -188,10 +190,21 @@ int fused_steps(const lee_lbm *h) {
         const bool tiled = h->ops->stepk && h->cfg.bc == LEE_BC_PERIODIC && h->cfg.nx % 4 == 0 && h->cfg.ny >= 3;
         return tiled && h->tb_steps >= 3 ? h->tb_steps : 1;
     }
-    const bool tiled = h->ops->step2 && h->cfg.bc == LEE_BC_PERIODIC && h->cfg.storage == LEE_STORE_F32 &&
+    const bool tiled = h->ops->stepk && h->cfg.bc == LEE_BC_PERIODIC && h->cfg.storage == LEE_STORE_F32 &&
                        h->cfg.nx % 4 == 0 && h->cfg.ny >= 3;
-    if (!tiled) return 1;
-    return h->tb_steps >= 3 && h->ops->stepk ? h->tb_steps : 2;
+    return tiled ? h->tb_steps : 1;
+}
+
+// Steps of the next launch of a run with `left` steps to go.  2D grids on the row pipeline take kRpDeep
+// steps at a time while they can, unless LEE_TB_STEPS asked for a count, and FP32 ones the two or three
+// that remain in one launch too (the same bits; a 16-bit state would be rounded at other steps).
+// Measured on GB300 (D2Q5 FP32, GLUPS on 2048^2 / 8192^2): four steps per launch 740 / 811, eight 1490 / 1611.
+int next_launch(const lee_lbm *h, int unit, long long left) {
+    if (unit > 1 && h->D == 2 && !h->tb_env) {
+        if (left >= kRpDeep) return kRpDeep;
+        if (left < unit && left > 1 && h->cfg.storage == LEE_STORE_F32) return (int)left;
+    }
+    return left >= unit ? unit : 1;
 }
 
 // Whether the 1D on-chip path (all steps of a call in one launch) takes this grid.
@@ -488,12 +501,12 @@ lee_status lee_lbm_create(const lee_lbm_config *cfg, lee_lbm **out) {
         if (e == cudaSuccess) e = cudaMalloc(&h->corner, 4 * sizeof(unsigned long long));
         if (e == cudaSuccess) e = cudaMemsetAsync(h->corner, 0, 4 * sizeof(unsigned long long), h->st);
     }
-    if (e == cudaSuccess && o->step2_prepare && cfg->bc == LEE_BC_PERIODIC && cfg->storage == LEE_STORE_F32)
-        e = o->step2_prepare();
-    if (e == cudaSuccess && o->stepk_prepare && h->tb_steps >= 3 && cfg->bc == LEE_BC_PERIODIC &&
-        (cfg->storage == LEE_STORE_F32 || cfg->storage == LEE_STORE_BFP16 || cfg->storage == LEE_STORE_F16 ||
-         cfg->storage == LEE_STORE_BF16))
-        e = o->stepk_prepare(h->tb_steps, cfg->storage);
+    if (e == cudaSuccess && h->D == 2 && fused_steps(h) > 1) {
+        const int deep = h->tb_env ? 0 : kRpDeep;
+        for (int k : {2, 3, 4, deep})
+            if (e == cudaSuccess && k > 0 && (h->tb_env ? k == h->tb_steps : k != 2 || cfg->storage == LEE_STORE_F32))
+                e = o->stepk_prepare(k, cfg->storage);
+    }
     if (e == cudaSuccess && h->tb_steps >= 2 && tiled_3d(h)) e = o->step3d2_prepare(cfg->storage, tma_tile(h) ? 1 : 0);
     if (e == cudaSuccess && tma_tile(h)) {
         e = cudaHostAlloc(reinterpret_cast<void **>(&h->wait_host), sizeof(unsigned), cudaHostAllocMapped);
@@ -635,7 +648,6 @@ lee_status lee_lbm_step(lee_lbm *h, int64_t n) {
         if (e == cudaSuccess) e = cudaStreamWaitEvent(st, h->ev_join, 0);
         return e;
     };
-    int64_t left = n;
     // 1D grids that fit in shared memory: every step in one launch of the on-chip kernel
     if (n >= 2 && onchip(h)) {
         L.stream = h->st;
@@ -643,28 +655,34 @@ lee_status lee_lbm_step(lee_lbm *h, int64_t n) {
         h->steps += n;
         return LEE_OK;
     }
-    // Periodic 2D FP32 grids whose width is a multiple of 4: several steps per launch
-    // (temporal blocking; bit-identical to single steps).
     const int unit = fused_steps(h);
-    auto launch_unit = [&](int from, cudaStream_t st) -> cudaError_t {
-        if (unit == 1) return launch_step(from, st);
+    // one launch of k steps, reading copy `from`
+    auto launch = [&](int from, int k, cudaStream_t st) -> cudaError_t {
+        if (k == 1) return launch_step(from, st);
         L.src = h->buf[from];
         L.dst = h->buf[from ^ 1];
         L.stream = st;
-        if (h->D == 3) return h->ops->step3d2(L);
-        return unit == 2 ? h->ops->step2(L) : h->ops->stepk(L, unit);
+        return h->D == 3 ? h->ops->step3d2(L) : h->ops->stepk(L, k);
     };
-    int64_t units = n / unit;
-    if (units * unit >= kGraphMinSteps) {
-        // Runs of up to kMaxGraphSteps steps are one launch of a graph holding all of them;
-        // longer runs replay a kChunkGraphSteps graph.  Graphs hold an even number of launches,
-        // so a replay leaves the buffer parity unchanged; they are captured once per (parity,
-        // length) on a private stream and replayed on the handle's stream.
-        const long long gunits =
-            units * unit <= kMaxGraphSteps ? (units & ~1LL) : (kChunkGraphSteps / unit) & ~1LL;
-        while (gunits > 0 && units >= gunits) {
-            const long long gsteps = gunits * unit;
-            auto it = h->exec.find({h->cur, gsteps});
+    auto launches_of = [&](int64_t steps) {
+        int64_t c = 0;
+        while (steps > 0) {
+            const int k = next_launch(h, unit, steps);
+            const int64_t r = steps / k;  // as many of this size as fit
+            c += r;
+            steps -= r * k;
+        }
+        return c;
+    };
+    int64_t left = n;
+    if (launches_of(left) >= kGraphMinLaunches) {
+        // Runs of up to kMaxGraphSteps steps are one launch of a graph holding all of them; longer runs
+        // replay a kChunkGraphSteps graph.  Graphs are captured once per (starting copy, length) on a
+        // private stream and replayed on the handle's stream.
+        const int64_t steps = left <= kMaxGraphSteps ? left : kChunkGraphSteps;
+        const int flips = (int)(launches_of(steps) & 1);
+        while (left >= steps) {
+            auto it = h->exec.find({h->cur, steps});
             cudaGraphExec_t ex = it == h->exec.end() ? nullptr : it->second;
             if (!ex) {
                 if (!h->cap) LEE_CK(h, cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking), "capture stream");
@@ -672,29 +690,30 @@ lee_status lee_lbm_step(lee_lbm *h, int64_t n) {
                 LEE_CK(h, cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal), "begin capture");
                 cudaError_t e = cudaSuccess;
                 int w = h->cur;
-                for (long long k = 0; k < gunits && e == cudaSuccess; ++k, w ^= 1) e = launch_unit(w, h->cap);
+                for (int64_t r = steps; r > 0 && e == cudaSuccess; w ^= 1) {
+                    const int k = next_launch(h, unit, r);
+                    e = launch(w, k, h->cap);
+                    r -= k;
+                }
                 cudaError_t e2 = cudaStreamEndCapture(h->cap, &g);
                 if (e == cudaSuccess) e = e2;
                 if (e == cudaSuccess) e = cudaGraphInstantiate(&ex, g, 0);
                 if (g) cudaGraphDestroy(g);
                 LEE_CK(h, e, "step graph capture");
-                h->exec[{h->cur, gsteps}] = ex;
+                h->exec[{h->cur, steps}] = ex;
             }
             LEE_CK(h, cudaGraphLaunch(ex, h->st), "step graph launch");
-            units -= gunits;
-            h->steps += gsteps;
+            h->cur ^= flips;
+            left -= steps;
+            h->steps += steps;
         }
     }
-    for (; units > 0; --units) {
-        LEE_CK(h, launch_unit(h->cur, h->st), "step launch");
+    while (left > 0) {
+        const int k = next_launch(h, unit, left);
+        LEE_CK(h, launch(h->cur, k, h->st), "step launch");
         h->cur ^= 1;
-        h->steps += unit;
-    }
-    left = n % unit;
-    for (; left > 0; --left) {
-        LEE_CK(h, launch_step(h->cur, h->st), "step launch");
-        h->cur ^= 1;
-        h->steps++;
+        left -= k;
+        h->steps += k;
     }
     return LEE_OK;
 }

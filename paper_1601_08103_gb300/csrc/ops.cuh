@@ -10,6 +10,10 @@
 
 namespace lee {
 
+// Time steps that the 2D row pipeline takes in one launch where a call has that many left: two runs of
+// four.
+constexpr int kRpDeep = 8;
+
 // Launch description of one fused time step.
 struct StepLaunch {
     int storage;         // lee_storage
@@ -45,13 +49,10 @@ struct SetOps {
     int D, Q;
     // one fused pull-stream + collide step
     cudaError_t (*step)(const StepLaunch &);
-    // two fused steps per launch (periodic 2D FP32 grids with nx % 4 == 0; nullptr otherwise):
-    // reads L.src, writes the state two steps later into L.dst
-    cudaError_t (*step2)(const StepLaunch &);
-    // one-time set-up of the two-step kernel on the current device (outside stream capture)
-    cudaError_t (*step2_prepare)();
-    // k = 3 or 4 fused steps per launch on the same grids (FP32, or BFP16 with nx % 8 == 0), and
-    // its one-time set-up for a storage type
+    // k fused steps per launch of the 2D row pipeline (periodic grids; reads L.src, writes the state k
+    // steps later into L.dst): FP32 with nx % 4 == 0 and k = 2, 3, 4 or kRpDeep; FP16 / BF16 with
+    // nx % 4 == 0 and BFP16 with nx % 8 == 0 and k = 3, 4 or kRpDeep.  stepk_prepare: its one-time
+    // set-up on the current device for a storage type, outside stream capture
     cudaError_t (*stepk)(const StepLaunch &, int k);
     cudaError_t (*stepk_prepare)(int k, int storage);
     // two fused steps per launch for the 3D axis-velocity sets (periodic; FP32 with nx % 4 == 0

@@ -249,35 +249,47 @@ struct SetImpl {
             });
         }
     }
-    static cudaError_t step2_prepare() { return two_step_prepare<S>(); }
-    static cudaError_t step2(const StepLaunch &L) { return two_step_launch<S>(L); }
-    // K = 3 or 4 steps per launch: FP32 storage (bit-identical to single steps), or BFP16, FP16 and
-    // BF16 storage (FP32 levels in between, one rounding to the storage per launch)
-    template <class IO>
-    static cudaError_t stepk_prepare_io(int k) {
-        return k == 3 ? kstep_prepare<S, 3, IO>() : k == 4 ? kstep_prepare<S, 4, IO>() : cudaErrorInvalidValue;
+    // K steps per launch in 2D: FP32 storage with K = 2, 3, 4, 8 (the bits of single steps), or BFP16,
+    // FP16 and BF16 storage with K = 3, 4, 8 (FP32 levels in between, one rounding per launch)
+    template <class IO, class Fn>
+    static cudaError_t with_steps(int k, Fn &&fn) {
+        switch (k) {
+        case 2:
+            if constexpr (std::is_same<IO, RpF32>::value) return fn(std::integral_constant<int, 2>{});
+            return cudaErrorInvalidValue;
+        case 3: return fn(std::integral_constant<int, 3>{});
+        case 4: return fn(std::integral_constant<int, 4>{});
+        case kRpDeep: return fn(std::integral_constant<int, kRpDeep>{});
+        default: return cudaErrorInvalidValue;
+        }
     }
-    template <class IO>
-    static cudaError_t stepk_io(const StepLaunch &L, int k) {
-        return k == 3 ? kstep_launch<S, 3, IO>(L) : k == 4 ? kstep_launch<S, 4, IO>(L) : cudaErrorInvalidValue;
+    template <class Fn>
+    static cudaError_t with_pipe(int storage, int k, Fn &&fn) {
+        if constexpr (S::D != 2) {
+            return cudaErrorInvalidValue;
+        } else {
+            auto go = [&](auto *io) {
+                using IO = std::remove_pointer_t<decltype(io)>;
+                return with_steps<IO>(k, [&](auto Kc) { return fn(io, Kc); });
+            };
+            switch (storage) {
+            case LEE_STORE_BFP16: return go((RpBfp<S::Q> *)nullptr);
+            case LEE_STORE_F16: return go((Rp16<__half> *)nullptr);
+            case LEE_STORE_BF16: return go((Rp16<__nv_bfloat16> *)nullptr);
+            case LEE_STORE_F32: return go((RpF32 *)nullptr);
+            default: return cudaErrorInvalidValue;
+            }
+        }
     }
     static cudaError_t stepk_prepare(int k, int storage) {
-        switch (storage) {
-        case LEE_STORE_BFP16: return stepk_prepare_io<TileIoBfp<S::Q>>(k);
-        case LEE_STORE_F16: return stepk_prepare_io<TileIo16<__half>>(k);
-        case LEE_STORE_BF16: return stepk_prepare_io<TileIo16<__nv_bfloat16>>(k);
-        case LEE_STORE_F32: return stepk_prepare_io<TileIoF32>(k);
-        default: return cudaErrorInvalidValue;
-        }
+        return with_pipe(storage, k, [](auto *io, auto Kc) {
+            return row_pipe_prepare<decltype(Kc)::value, std::remove_pointer_t<decltype(io)>>();
+        });
     }
     static cudaError_t stepk(const StepLaunch &L, int k) {
-        switch (L.storage) {
-        case LEE_STORE_BFP16: return stepk_io<TileIoBfp<S::Q>>(L, k);
-        case LEE_STORE_F16: return stepk_io<TileIo16<__half>>(L, k);
-        case LEE_STORE_BF16: return stepk_io<TileIo16<__nv_bfloat16>>(L, k);
-        case LEE_STORE_F32: return stepk_io<TileIoF32>(L, k);
-        default: return cudaErrorInvalidValue;
-        }
+        return with_pipe(L.storage, k, [&](auto *io, auto Kc) {
+            return row_pipe_launch<decltype(Kc)::value, std::remove_pointer_t<decltype(io)>>(L);
+        });
     }
     // two steps per launch in 3D (axis-velocity sets; FP32 storage, or BFP16 with level 1 in FP32)
     // TMA-fed tile instantiations (one block per SM: the BFP16 tile needs 131 registers per thread
@@ -345,8 +357,6 @@ struct SetImpl {
         o.slab_unpack = S::D >= 2 ? &slab_unpack : nullptr;
         o.slab_crossing = slab_crossing<S>();
         o.onchip_1d = S::D == 1 ? &onchip_1d : nullptr;
-        o.step2 = S::D == 2 ? &step2 : nullptr;
-        o.step2_prepare = S::D == 2 ? &step2_prepare : nullptr;
         o.stepk = S::D == 2 ? &stepk : nullptr;
         o.stepk_prepare = S::D == 2 ? &stepk_prepare : nullptr;
         o.step3d2 = axis_only<S>() ? &step3d2 : nullptr;

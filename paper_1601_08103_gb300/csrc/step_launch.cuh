@@ -1,10 +1,11 @@
 // step_launch.cuh -- launch configuration of the fused stream-collide kernels for one velocity set:
-// the one-step kernel (cells per thread, grid) and the two-step and K-step 2D kernels (tile height
-// from the resident capacity).  Together with kernels.cuh and velsets.cuh this fixes what the
+// the one-step kernel (cells per thread, grid) and the 2D row pipeline (segment height from the
+// resident capacity).  Together with kernels.cuh and velsets.cuh this fixes what the
 // profiled hot-path launches execute.
 #pragma once
 
 #include "ops.cuh"
+#include "rowpipe.cuh"
 
 namespace lee {
 
@@ -104,130 +105,72 @@ cudaError_t with_storage(int storage, Fn &&fn) {
     }
 }
 
-// Resident capacity of the two-step kernel (blocks per SM x SMs) per device, set by
-// two_step_prepare outside any stream capture.
-template <class S>
-int *two_step_capacity() {
+// Row pipeline (rowpipe.cuh): the resident warps of a device, set by row_pipe_prepare outside any
+// stream capture, and the launch.
+template <int K, class IO, int kStages>
+int *row_pipe_capacity() {
     static int cap[64] = {0};
     return cap;
 }
-template <class S>
-cudaError_t two_step_prepare() {
-    if constexpr (S::D != 2) {
-        return cudaErrorInvalidValue;
+template <int K, class IO, int kStages>
+cudaError_t row_pipe_prepare_stages() {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (row_pipe_capacity<K, IO, kStages>()[dev]) return cudaSuccess;
+    constexpr int smem = rp_smem_bytes<IO, kStages>();
+    int per_sm = 0, sms = 0;
+    e = cudaFuncSetAttribute(k_row_pipe<K, IO, kStages>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_row_pipe<K, IO, kStages>, 32 * kRpWarps, smem);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    row_pipe_capacity<K, IO, kStages>()[dev] = per_sm * sms > 0 ? per_sm * sms * kRpWarps : 1;
+    return cudaSuccess;
+}
+template <int K, class IO, int kStages>
+cudaError_t row_pipe_launch_stages(const StepLaunch &L) {
+    using E = typename IO::Elem;
+    if (L.open || L.nx % IO::kAlign != 0 || L.nx % 4 != 0) return cudaErrorInvalidValue;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    const int capacity = row_pipe_capacity<K, IO, kStages>()[dev];
+    if (capacity == 0) return cudaErrorNotReady;  // prepare first
+    const CollideCoef<float> cf = make_coef<float>(L.omega, L.coefM, L.coefN);
+    // segment height: the smallest even number (at least kRpMinRows) that puts every tile in one resident
+    // wave (twice or half as many warps measured 10 to 40 % slower on 2048^2 .. 8192^2)
+    constexpr int width = rp_width<K, IO>();
+    const int strips = (L.nx + width - 1) / width;
+    const int segs = capacity / strips > 1 ? capacity / strips : 1;
+    int H = (L.ny + segs - 1) / segs;
+    H += H & 1;
+    if (H < kRpMinRows) H = kRpMinRows;
+    const int tiles = strips * ((L.ny + H - 1) / H);
+    k_row_pipe<K, IO, kStages><<<(tiles + kRpWarps - 1) / kRpWarps, 32 * kRpWarps, rp_smem_bytes<IO, kStages>(),
+                                 L.stream>>>(static_cast<const E *>(L.src), static_cast<E *>(L.dst), L.nx, L.ny, L.pitch,
+                                             H, strips, tiles, cf.M[1][1]);
+    return cudaGetLastError();
+}
+template <int K, class IO>
+cudaError_t row_pipe_prepare() {
+    if constexpr (std::is_same<IO, RpF32>::value) {
+        const cudaError_t e = row_pipe_prepare_stages<K, IO, kRpStagesNear>();
+        return e != cudaSuccess ? e : row_pipe_prepare_stages<K, IO, kRpStagesFar>();
     } else {
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e != cudaSuccess) return e;
-        if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-        if (two_step_capacity<S>()[dev]) return cudaSuccess;
-        constexpr int smem = tb_smem_bytes<S>();
-        e = cudaFuncSetAttribute(k_stream_collide_2step<S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_stream_collide_2step<S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        int per_sm = 0, per_sm_pf = 0, sms = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stream_collide_2step<S, false>, 128, smem);
-        if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_pf, k_stream_collide_2step<S, true>, 128, smem);
-        if (per_sm_pf < per_sm) per_sm = per_sm_pf;
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        two_step_capacity<S>()[dev] = per_sm * sms > 0 ? per_sm * sms : 1;
-        return cudaSuccess;
+        return row_pipe_prepare_stages<K, IO, kRpStages16>();
     }
 }
-template <class S>
-cudaError_t two_step_launch(const StepLaunch &L) {
-    if constexpr (S::D != 2) {
-        return cudaErrorInvalidValue;
+template <int K, class IO>
+cudaError_t row_pipe_launch(const StepLaunch &L) {
+    if constexpr (std::is_same<IO, RpF32>::value) {
+        return 8LL * (long long)sizeof(float) * L.nx * L.ny <= kRpNearL2Bytes
+                   ? row_pipe_launch_stages<K, IO, kRpStagesNear>(L)
+                   : row_pipe_launch_stages<K, IO, kRpStagesFar>(L);
     } else {
-        if (L.storage != LEE_STORE_F32 || L.open || L.nx % 4 != 0 || L.ny < 3) return cudaErrorInvalidValue;
-        const CollideCoef<float> cf = make_coef<float>(L.omega, L.coefM, L.coefN);
-        constexpr int smem = tb_smem_bytes<S>();
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e != cudaSuccess) return e;
-        if (dev < 0 || dev >= 64 || two_step_capacity<S>()[dev] == 0) return cudaErrorNotReady;  // prepare first
-        // tile height: the smallest multiple of 4 (>= 16) that puts every tile in one resident wave
-        const int strips = (L.nx + kTbW - 1) / kTbW;
-        int segs = two_step_capacity<S>()[dev] / strips;
-        if (segs < 1) segs = 1;
-        int H = (L.ny + segs - 1) / segs;
-        H = (H + 3) / 4 * 4;
-        if (H < 16) H = 16;
-        const dim3 grid(strips, (L.ny + H - 1) / H);
-        const long long bytes = 2LL * S::Q * (long long)sizeof(float) * L.nx * L.ny;
-        auto kern = bytes <= kTbL2PrefetchMaxBytes ? k_stream_collide_2step<S, true> : k_stream_collide_2step<S, false>;
-        kern<<<grid, 128, smem, L.stream>>>(static_cast<const float *>(L.src), static_cast<float *>(L.dst), L.nx, L.ny,
-                                            L.pitch, H, cf);
-        return cudaGetLastError();
-    }
-}
-
-
-// The same for K steps per launch (K = 3, 4): resident capacity per device, then the launch.
-// IO: the storage policy of the tile (TileIoF32, or TileIoBfp for BFP16 storage).
-template <class S, int K, class IO>
-int *kstep_capacity() {
-    static int cap[64] = {0};
-    return cap;
-}
-template <class S, int K, class IO = TileIoF32>
-cudaError_t kstep_prepare() {
-    if constexpr (S::D != 2) {
-        return cudaErrorInvalidValue;
-    } else {
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e != cudaSuccess) return e;
-        if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-        if (kstep_capacity<S, K, IO>()[dev]) return cudaSuccess;
-        constexpr int smem = tbk_smem_bytes<S, K>();
-        e = cudaFuncSetAttribute(k_stream_collide_kstep<S, K, IO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 smem);
-        if (e != cudaSuccess) return e;
-        int per_sm = 0, sms = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stream_collide_kstep<S, K, IO>, kTbkThreads, smem);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        kstep_capacity<S, K, IO>()[dev] = per_sm * sms > 0 ? per_sm * sms : 1;
-        return cudaSuccess;
-    }
-}
-template <class S, int K, class IO = TileIoF32>
-cudaError_t kstep_launch(const StepLaunch &L) {
-    if constexpr (S::D != 2) {
-        return cudaErrorInvalidValue;
-    } else {
-        using E = typename IO::Elem;
-        constexpr bool bfp = std::is_same<E, Bfp16>::value;
-        constexpr int storage = bfp ? LEE_STORE_BFP16
-                                    : std::is_same<E, float>::value ? LEE_STORE_F32
-                                    : std::is_same<E, __half>::value ? LEE_STORE_F16 : LEE_STORE_BF16;
-        if (L.storage != storage || L.open || L.nx % (bfp ? kBfpBlock : 4) != 0 || L.ny < 3)
-            return cudaErrorInvalidValue;
-        const CollideCoef<float> cf = make_coef<float>(L.omega, L.coefM, L.coefN);
-        constexpr int smem = tbk_smem_bytes<S, K>();
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e != cudaSuccess) return e;
-        if (dev < 0 || dev >= 64 || kstep_capacity<S, K, IO>()[dev] == 0) return cudaErrorNotReady;  // prepare first
-        // tile height: the smallest multiple of 4 (>= 16) that puts every tile in one resident wave
-        const int strips = (L.nx + kTbW - 1) / kTbW;
-        int segs = kstep_capacity<S, K, IO>()[dev] / strips;
-        if (segs < 1) segs = 1;
-        int H = (L.ny + segs - 1) / segs;
-        H = (H + 3) / 4 * 4;
-        if (H < 16) H = 16;
-        const dim3 grid(strips, (L.ny + H - 1) / H);
-        // No L2 prefetch: it helps the byte-bound two-step kernel on small grids, but this kernel
-        // is bound by instruction issue, and the prefetch instructions cost more than they save
-        // (measured on GB300, D2Q5 2048^2: 402 GLUPS without, 388 with).
-        k_stream_collide_kstep<S, K, IO><<<grid, kTbkThreads, smem, L.stream>>>(static_cast<const E *>(L.src),
-                                                                         static_cast<E *>(L.dst), L.nx, L.ny, L.pitch,
-                                                                         H, cf);
-        return cudaGetLastError();
+        return row_pipe_launch_stages<K, IO, kRpStages16>(L);
     }
 }
 

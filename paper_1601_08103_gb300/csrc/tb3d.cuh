@@ -76,6 +76,10 @@ __device__ __forceinline__ float t3_round(float v) {
     }
 }
 
+__device__ __forceinline__ void t3_st(float *p, const float (&v)[kT3V]) {
+    *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+
 constexpr int kT3Rows = 8;  // TY: rows per tile
 
 template <class S, class T, int TY>

@@ -77,7 +77,7 @@ struct T3tIoF32 {
     __device__ static __forceinline__ float round(float v) { return v; }
     __device__ static __forceinline__ void st4(float *__restrict__ g, long long, long long idx, const float (&v)[4],
                                                bool st) {
-        if (st) tb_st(g + idx, v);
+        if (st) t3_st(g + idx, v);
     }
 };
 
