@@ -48,10 +48,11 @@ KERNEL_SOURCES = ["paper_1601_08103_gb300/csrc/kernels.cuh", "paper_1601_08103_g
 
 
 def steps_of_launch(sv) -> int:
-    """Time steps per launch of a long run: grids that fuse runs of four take two such runs (eight steps)
-    in one launch."""
+    """Time steps per launch of a long run in the default configuration: grids that fuse runs of steps take two
+    such runs in one launch (BFP16 and the TMA-fed tile one)."""
     spl = max(sv.steps_per_launch, 1)
-    return 8 if spl == 4 else spl
+    tma = os.environ.get("LEE_T3_TMA") == "1"
+    return spl if spl == 1 or sv.storage == "bfp16" or tma else 2 * spl
 
 
 def kernel_source_sha() -> str:

@@ -192,17 +192,19 @@ lee_status lee_lbm_init_fields(lee_lbm *h, const double *rho, const double *u, c
  *    intermediate states kept in registers (temporal blocking): eight while the call has that many
  *    left, then four, then the two or three or one that remain.  LEE_TB_STEPS=1..4 in the
  *    environment at create time fixes the count instead (n / count launches, n % count single steps);
- *  - periodic 3D FP32 grids of D3Q7 and diatomic D3Q7 with nx a multiple of 4 advance two steps
- *    per launch (a z-marching tile; LEE_TB_STEPS=1 keeps one step per launch);
- *  - BFP16 storage on those periodic 2D grids with nx a multiple of 8 uses the same kernels (eight steps
- *    and four, the rest as single steps; or three or four with LEE_TB_STEPS), but keeps the
+ *  - periodic 3D FP32 grids of D3Q7 and diatomic D3Q7 with nx a multiple of 4 advance four steps per
+ *    launch (a pipeline of the planes), then two (a z-marching tile), then one; grids of fewer than
+ *    786432 cells, where that is slower, take single steps (LEE_TB_STEPS=1 or 2 fixes the count);
+ *  - BFP16 storage on those periodic 2D grids with nx a multiple of 8 uses the same kernels (four steps
+ *    per launch, the rest as single steps; or three with LEE_TB_STEPS=3), but keeps the
  *    intermediate states in FP32 and encodes only the last one: a launch of k steps equals decoding
  *    the state, k FP32 steps and one encoding, bit for bit (LEE_TB_STEPS=1 or 2 keeps one step per
  *    launch, which equals decode, one FP32 step, encode).  On 3D grids BFP16 runs one step per launch
  *    unless LEE_TB_STEPS=2 asks for the two-step tile (nx a multiple of 8), which is slower there;
- *  - FP16 and BF16 storage on periodic 2D grids with nx a multiple of 4 do the same, with one
- *    rounding to the storage per launch (LEE_TB_STEPS=1 or 2 keeps one step per launch, rounding
- *    every step);
+ *  - FP16 and BF16 storage on periodic 2D grids with nx a multiple of 4 do the same, rounding to the
+ *    storage after every four steps (or three with LEE_TB_STEPS=3; a launch of eight rounds after its first
+ *    four steps too), with single steps for the rest (LEE_TB_STEPS=1 or 2 keeps one step per launch,
+ *    rounding every step);
  *  - a 1D grid (not BFP16) whose two population copies fit in shared memory (2 q nx sizeof(storage) <= 227 KB,
  *    e.g. D1Q3 FP64 up to 4843 cells) runs all n >= 2 steps in one launch: one block, or from
  *    512 cells a thread-block cluster of 8 blocks;
@@ -292,11 +294,12 @@ lee_status lee_lbm_steps_done(lee_lbm *h, int64_t *steps);
 /* How lee_lbm_step runs this grid: *steps = 1 (one fused stream-collide launch per time step),
  * 2..4 (that many time steps per launch, the intermediate states kept on the SMs -- temporal blocking)
  * or 0 (small 1D grid: all steps of a call in one on-chip launch).  Periodic 2D FP32 grids with nx a
- * multiple of 4: 4 unless LEE_TB_STEPS was set at create time; a call takes two such runs, eight
- * steps, in one launch where it can (not with LEE_TB_STEPS).  Periodic 3D FP32 D3Q7 and diatomic D3Q7
- * grids with nx a multiple of 4: 2.  BFP16 storage: 3 or 4 in 2D on such grids with nx a multiple of 8, 2
+ * multiple of 4: 4 unless LEE_TB_STEPS was set at create time; FP32, FP16 and BF16 calls take two such
+ * runs, eight steps, in one launch where they can (not with LEE_TB_STEPS).  Periodic 3D FP32 D3Q7 and
+ * diatomic D3Q7 grids with nx a multiple of 4: 2 (calls take two such runs in one launch where they can,
+ * and small grids single steps).  BFP16 storage: 3 or 4 in 2D on such grids with nx a multiple of 8, 2
  * in 3D only with LEE_TB_STEPS=2; FP16 / BF16 storage: 3 or 4 in 2D on such grids.  All forms give
- * bit-identical results, except that BFP16, FP16 and BF16 storage round their state once per launch
+ * bit-identical results, except that BFP16, FP16 and BF16 storage round their state once per run of *steps
  * (see lee_lbm_step). */
 lee_status lee_lbm_steps_per_launch(lee_lbm *h, int32_t *steps);
 

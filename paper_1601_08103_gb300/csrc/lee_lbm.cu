@@ -195,14 +195,32 @@ int fused_steps(const lee_lbm *h) {
     return tiled ? h->tb_steps : 1;
 }
 
-// Steps of the next launch of a run with `left` steps to go.  2D grids on the row pipeline take kRpDeep
-// steps at a time while they can, unless LEE_TB_STEPS asked for a count, and FP32 ones the two or three
-// that remain in one launch too (the same bits; a 16-bit state would be rounded at other steps).
-// Measured on GB300 (D2Q5 FP32, GLUPS on 2048^2 / 8192^2): four steps per launch 740 / 811, eight 1490 / 1611.
+// Whether runs of this 3D grid take kPpDeep steps per launch (planepipe.cuh): not where the environment
+// asked for a count or the TMA-fed tile.
+bool plane_pipe(const lee_lbm *h) {
+    return h->ops->step3dk && h->cfg.bc == LEE_BC_PERIODIC && h->cfg.storage == LEE_STORE_F32 && h->tb_steps == 4 &&
+           !h->tb_env && !tma_tile(h) && plane_pipe_eligible(h->cfg.nx, h->cfg.ny);
+}
+
+constexpr long long kFuse3dCells = 3LL << 18;
+
+// Steps of the next launch of a run with `left` steps to go.  Unless LEE_TB_STEPS asked for a count, grids
+// on the row pipeline take kRpDeep steps at a time while they can (two units in one launch, with the
+// bits of two launches; BFP16 would need wider halos for that and stays on units), and FP32 ones the two
+// or three that remain in one launch too (a 16-bit state would be rounded at other steps); 3D grids on the
+// plane pipeline take kPpDeep.  3D FP32 grids of fewer than kFuse3dCells cells take single steps: their few
+// tiles leave SMs idle in either fused kernel (us per step of one / two / four steps per launch: 64^3 2.5 /
+// 3.7 / 2.9, 80^3 3.7 / 4.8 / 3.8, 96^3 4.8 / 5.9 / 4.5, 128^3 - / 10.2 / 7.9).
+// Measured on GB300, GLUPS: D2Q5 FP32 2048^2 / 8192^2 four steps per launch 740 / 811, eight 1490 / 1611; D3Q7
+// FP32 384^3 / 256^3 two 259 / 232, four 373 / 334.
 int next_launch(const lee_lbm *h, int unit, long long left) {
     if (unit > 1 && h->D == 2 && !h->tb_env) {
-        if (left >= kRpDeep) return kRpDeep;
+        if (left >= kRpDeep && h->cfg.storage != LEE_STORE_BFP16) return kRpDeep;
         if (left < unit && left > 1 && h->cfg.storage == LEE_STORE_F32) return (int)left;
+    }
+    if (h->D == 3 && plane_pipe(h)) {
+        if (h->cells < kFuse3dCells) return 1;
+        if (left >= kPpDeep) return kPpDeep;
     }
     return left >= unit ? unit : 1;
 }
@@ -502,11 +520,12 @@ lee_status lee_lbm_create(const lee_lbm_config *cfg, lee_lbm **out) {
         if (e == cudaSuccess) e = cudaMemsetAsync(h->corner, 0, 4 * sizeof(unsigned long long), h->st);
     }
     if (e == cudaSuccess && h->D == 2 && fused_steps(h) > 1) {
-        const int deep = h->tb_env ? 0 : kRpDeep;
+        const int deep = h->tb_env || cfg->storage == LEE_STORE_BFP16 ? 0 : kRpDeep;
         for (int k : {2, 3, 4, deep})
             if (e == cudaSuccess && k > 0 && (h->tb_env ? k == h->tb_steps : k != 2 || cfg->storage == LEE_STORE_F32))
                 e = o->stepk_prepare(k, cfg->storage);
     }
+    if (e == cudaSuccess && plane_pipe(h)) e = o->step3dk_prepare();
     if (e == cudaSuccess && h->tb_steps >= 2 && tiled_3d(h)) e = o->step3d2_prepare(cfg->storage, tma_tile(h) ? 1 : 0);
     if (e == cudaSuccess && tma_tile(h)) {
         e = cudaHostAlloc(reinterpret_cast<void **>(&h->wait_host), sizeof(unsigned), cudaHostAllocMapped);
@@ -662,7 +681,8 @@ lee_status lee_lbm_step(lee_lbm *h, int64_t n) {
         L.src = h->buf[from];
         L.dst = h->buf[from ^ 1];
         L.stream = st;
-        return h->D == 3 ? h->ops->step3d2(L) : h->ops->stepk(L, k);
+        if (h->D == 3) return k == kPpDeep ? h->ops->step3dk(L) : h->ops->step3d2(L);
+        return h->ops->stepk(L, k);
     };
     auto launches_of = [&](int64_t steps) {
         int64_t c = 0;

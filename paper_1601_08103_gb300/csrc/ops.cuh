@@ -13,6 +13,10 @@ namespace lee {
 // Time steps that the 2D row pipeline takes in one launch where a call has that many left: two runs of
 // four.
 constexpr int kRpDeep = 8;
+// Time steps per launch of the 3D plane pipeline, and the grids it takes (a launch has at most 65535 tiles
+// along y, of one row at least).
+constexpr int kPpDeep = 4;
+inline bool plane_pipe_eligible(long long nx, long long ny) { return nx % 4 == 0 && ny <= 65535; }
 
 // Launch description of one fused time step.
 struct StepLaunch {
@@ -60,6 +64,10 @@ struct SetOps {
     // and kernel (tma = 1: the TMA-fed tile, which also needs t3t_eligible grids)
     cudaError_t (*step3d2)(const StepLaunch &);
     cudaError_t (*step3d2_prepare)(int storage, int tma);
+    // kPpDeep fused steps per launch for the same sets (FP32, plane_pipe_eligible grids), and its one-time
+    // set-up
+    cudaError_t (*step3dk)(const StepLaunch &);
+    cudaError_t (*step3dk_prepare)();
     // g = g^eq(fields) (fields FP64 on device).  init, import_f64 and sponge_damp write a whole state
     // copy g; `other` is the other copy, whose rest populations they write too where a step leaves
     // those alone (rest_static)

@@ -28,7 +28,7 @@
 // What bounds it: with K = 8 a D2Q5 FP32 update takes 4 bytes of DRAM and about 10 instructions per thread,
 // 2 warps per scheduler.  Far beyond L2 FP32 is bound by DRAM (8192^2: 1611 GLUPS, 6.4 TB/s algorithmic,
 // 0.95 of the measured copy), 16-bit storage by issue and instruction latency (issue slots 54 % busy; FP16
-// 2228 GLUPS, BFP16 1284).  The tile it replaced (four levels through shared memory, three barriers per
+// 2126 GLUPS; BFP16 with K = 4 919).  The tile it replaced (four levels through shared memory, three barriers per
 // four rows, 39 instructions per update) ran 8192^2 at 517 (FP32), 553 (FP16) and 403 (BFP16) GLUPS and
 // 2048^2 FP32 at 426, against 1490 now.  Measured and not taken: loads two rows ahead into registers
 // instead of the ring (8192^2 FP32 1304 GLUPS, FP16 1955: 3 of 5.6 stall cycles per issue waited for
@@ -38,7 +38,7 @@
 //
 // Every level is rounded to FP32 as a stored state is, with the operations of collide_axis_cell: on
 // FP32 storage a launch gives the bits of K single steps.  On 16-bit storage S(t) is widened, the
-// levels in between stay FP32, and S(t+K) is rounded to the storage once.  The shell factors of the
+// levels in between stay FP32, and S(t+K) is rounded to the storage (with K = 8 S(t+4) too).  The shell factors of the
 // scaled storages are the same for all moving velocities, so the same kernel serves every set.
 #pragma once
 
@@ -63,22 +63,24 @@ __device__ __forceinline__ void copy_wait() {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
-// Memory side of the pipeline: fetch() starts the copy of a lane's four cells of a velocity into its
-// own slot of a shared-memory row, take() reads the slot and widens it, store() rounds and stores
-// four cells.  `idx` is an element of one velocity array starting at `base` (BFP16: with its
-// exponent bytes at `ex`).  kAlign: a warp's first column is a multiple of it.  kRow: bytes of a
-// row of one velocity in shared memory.
+// Memory side of the pipelines: fetch() starts the copy of a lane's four cells of a velocity into its
+// own slot of shared memory (kLane bytes at `to`; BFP16: and kLaneEx bytes at `to_ex`), take() reads
+// the slot and widens it, store() rounds and stores four cells, round() is what a stored and reloaded
+// value holds (not for BFP16).  `idx` is an element of one velocity
+// array starting at `base` (BFP16: with its exponent bytes at `ex`).  kAlign: a strip's first column is
+// a multiple of it.
 struct RpF32 {
     using Elem = float;
-    static constexpr int kAlign = 4, kRow = 32 * 16;
+    static constexpr int kAlign = 4, kLane = 16, kLaneEx = 0;
     static __host__ __device__ const uint8_t *exps(const float *, long long) { return nullptr; }
-    __device__ static __forceinline__ void fetch(unsigned to, int lane, const float *__restrict__ base, const uint8_t *,
+    __device__ static __forceinline__ void fetch(unsigned to, unsigned, const float *__restrict__ base, const uint8_t *,
                                                  int idx) {
-        copy_async<16>(to + 16 * lane, base + idx);
+        copy_async<16>(to, base + idx);
     }
-    __device__ static __forceinline__ float4 take(const char *from, int lane, int) {
-        return *reinterpret_cast<const float4 *>(from + 16 * lane);
+    __device__ static __forceinline__ float4 take(const char *from, const char *, int) {
+        return *reinterpret_cast<const float4 *>(from);
     }
+    __device__ static __forceinline__ float2 round(float2 v) { return v; }
     __device__ static __forceinline__ void store(float *__restrict__ base, uint8_t *, int idx, const float4 &v, bool live) {
         if (live) *reinterpret_cast<float4 *>(base + idx) = v;
     }
@@ -88,18 +90,21 @@ struct RpF32 {
 template <class T>
 struct Rp16 {
     using Elem = T;
-    static constexpr int kAlign = 4, kRow = 32 * 8;
+    static constexpr int kAlign = 4, kLane = 8, kLaneEx = 0;
     static __host__ __device__ const uint8_t *exps(const T *, long long) { return nullptr; }
-    __device__ static __forceinline__ void fetch(unsigned to, int lane, const T *__restrict__ base, const uint8_t *, int idx) {
-        copy_async<8>(to + 8 * lane, base + idx);
+    __device__ static __forceinline__ void fetch(unsigned to, unsigned, const T *__restrict__ base, const uint8_t *, int idx) {
+        copy_async<8>(to, base + idx);
     }
-    __device__ static __forceinline__ float4 take(const char *from, int lane, int) {
+    __device__ static __forceinline__ float4 take(const char *from, const char *, int) {
         union {
             uint2 r;
             T e[4];
         } u;
-        u.r = *reinterpret_cast<const uint2 *>(from + 8 * lane);
+        u.r = *reinterpret_cast<const uint2 *>(from);
         return make_float4(Store<T>::load(u.e[0]), Store<T>::load(u.e[1]), Store<T>::load(u.e[2]), Store<T>::load(u.e[3]));
+    }
+    __device__ static __forceinline__ float2 round(float2 v) {
+        return make_float2(Store<T>::load(Store<T>::make(v.x)), Store<T>::load(Store<T>::make(v.y)));
     }
     __device__ static __forceinline__ void store(T *__restrict__ base, uint8_t *, int idx, const float4 &v, bool live) {
         const float a[4] = {v.x, v.y, v.z, v.w};
@@ -112,26 +117,33 @@ struct Rp16 {
 template <int Q>
 struct RpBfp {
     using Elem = Bfp16;
-    static constexpr int kAlign = 8, kRow = 32 * (8 + 4);
+    static constexpr int kAlign = 8, kLane = 8, kLaneEx = 4;
     static __host__ __device__ const uint8_t *exps(const Bfp16 *g, long long pitch) { return bfp_exps<Q>(g, pitch); }
-    __device__ static __forceinline__ void fetch(unsigned to, int lane, const Bfp16 *__restrict__ base,
+    __device__ static __forceinline__ void fetch(unsigned to, unsigned to_ex, const Bfp16 *__restrict__ base,
                                                  const uint8_t *__restrict__ ex, int idx) {
-        copy_async<8>(to + 8 * lane, base + idx);
-        copy_async<4>(to + 32 * 8 + 4 * lane, ex + ((idx >> 3) & ~3));
+        copy_async<8>(to, base + idx);
+        copy_async<4>(to_ex, ex + ((idx >> 3) & ~3));
     }
-    __device__ static __forceinline__ float4 take(const char *from, int lane, int idx) {
-        const uint2 m = *reinterpret_cast<const uint2 *>(from + 8 * lane);
-        const unsigned e = *reinterpret_cast<const unsigned *>(from + 32 * 8 + 4 * lane);
+    __device__ static __forceinline__ float4 take(const char *from, const char *from_ex, int idx) {
+        const uint2 m = *reinterpret_cast<const uint2 *>(from);
+        const unsigned e = *reinterpret_cast<const unsigned *>(from_ex);
         const BfpDec k = bfp_dec((e >> (8 * ((idx >> 3) & 3))) & 255u);
         const float2 a = bfp_pair(m.x, k), b = bfp_pair(m.y, k);
         return make_float4(a.x, a.y, b.x, b.y);
     }
+    __device__ static float2 round(float2 v);  // (declared only: no launch of eight on blocks)
     __device__ static __forceinline__ void store(Bfp16 *__restrict__ base, uint8_t *__restrict__ ex, int idx,
                                                  const float4 &v, bool live) {
         const float a[4] = {v.x, v.y, v.z, v.w};
         bfp_store_vec<4>(base + idx, ex + (idx >> 3), a, live);
     }
 };
+
+// Shared memory of one velocity's row for `lanes` lanes.
+template <class IO>
+__host__ __device__ constexpr int rp_row_bytes(int lanes = 32) {
+    return lanes * (IO::kLane + IO::kLaneEx);
+}
 
 // Columns on either side of a strip that are computed but not stored.
 template <int K, class IO>
@@ -156,7 +168,7 @@ template <int K, class IO, int kHalo, int kStages>
 __device__ __forceinline__ void rp_tile(const typename IO::Elem *__restrict__ src, typename IO::Elem *__restrict__ dst,
                                         int nx, int ny, long long pitch, float w, int x0, int y0, int rows, char *ring) {
     using Elem = typename IO::Elem;
-    constexpr int kStage = 4 * IO::kRow;
+    constexpr int kRow = rp_row_bytes<IO>(), kStage = 4 * kRow;
     static_assert(kHalo >= K && kHalo % IO::kAlign == 0 && kHalo % 4 == 0, "columns that the levels spoil");
     const int lane = threadIdx.x & 31;
     const int col = x0 - kHalo + 4 * lane;
@@ -199,7 +211,10 @@ __device__ __forceinline__ void rp_tile(const typename IO::Elem *__restrict__ sr
     int slot = 0, free_slot = kStages - 1;  // the row to use now; the slot to fetch into
     auto fetch = [&](int to) {
 #pragma unroll
-        for (int v = 0; v < 4; ++v) IO::fetch(ring_at + to * kStage + v * IO::kRow, lane, in[v], in_ex[v], far.idx);
+        for (int v = 0; v < 4; ++v) {
+            const unsigned at = ring_at + to * kStage + v * kRow;
+            IO::fetch(at + lane * IO::kLane, at + 32 * IO::kLane + lane * IO::kLaneEx, in[v], in_ex[v], far.idx);
+        }
         next_row(far);
     };
     auto take = [&]() {
@@ -208,7 +223,8 @@ __device__ __forceinline__ void rp_tile(const typename IO::Elem *__restrict__ sr
         copy_wait<kStages - 2>();
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-            const float4 t = IO::take(ring + slot * kStage + v * IO::kRow, lane, now.idx);
+            const char *at = ring + slot * kStage + v * kRow;
+            const float4 t = IO::take(at + lane * IO::kLane, at + 32 * IO::kLane + lane * IO::kLaneEx, now.idx);
             to[v][0] = make_float2(t.x, t.z);
             to[v][1] = make_float2(t.y, t.w);
         }
@@ -233,7 +249,8 @@ __device__ __forceinline__ void rp_tile(const typename IO::Elem *__restrict__ sr
         hy[l][p][1] = r.py[1];
     };
     const float2 wp = splat2(w), wm = splat2(-w), m1 = splat2(-1.0f);
-    // level l + 1 from level l, whose newest row is r: r becomes level l + 1's newest row
+    // level l + 1 from level l, whose newest row is r: r becomes level l + 1's newest row.  A launch of eight
+    // rounds 16-bit storage after its first four levels too, so that it gives the bits of two launches.
     auto advance = [&](auto L, auto P, RpRow &r) {
         constexpr int l = decltype(L)::value, p = decltype(P)::value;
         const float2 pe = hx[l][p ^ 1][0], po = hx[l][p ^ 1][1], me = hx[l][p ^ 1][2], mo = hx[l][p ^ 1][3];
@@ -250,6 +267,12 @@ __device__ __forceinline__ void rp_tile(const typename IO::Elem *__restrict__ sr
             r.mx[h] = __ffma2_rn(wp, e, b[h]);
             r.py[h] = __ffma2_rn(wm, e, c[h]);
             r.my[h] = __ffma2_rn(wm, e, d[h]);
+            if constexpr (K == 8 && l + 1 == 4) {
+                r.px[h] = IO::round(r.px[h]);
+                r.mx[h] = IO::round(r.mx[h]);
+                r.py[h] = IO::round(r.py[h]);
+                r.my[h] = IO::round(r.my[h]);
+            }
         }
     };
 
@@ -296,13 +319,13 @@ __device__ __forceinline__ void rp_tile(const typename IO::Elem *__restrict__ sr
 // Slots of the ring.  FP32 states beyond L2 take four: more rows on their way make the warps drift apart
 // and the halo columns and rows that neighbours share miss L2 (D2Q5 8192^2, GLUPS with 4 / 6 / 9 slots:
 // 1611 / 1396 / 1391; 2048^2: 1374 / 1474 / 1509).  16-bit rows are half as long (8192^2 FP16 with 4 / 6 / 9:
-// 2197 / 2228 / 2222).
+// 2197 / 2228 / 2222, before the rounding of the fourth level).
 constexpr long long kRpNearL2Bytes = 256LL << 20;  // both copies
 constexpr int kRpStagesFar = 4, kRpStagesNear = 8, kRpStages16 = 6;
 
 template <class IO, int kStages>
 __host__ __device__ constexpr int rp_smem_bytes() {
-    return kRpWarps * kStages * 4 * IO::kRow;
+    return kRpWarps * kStages * 4 * rp_row_bytes<IO>();
 }
 
 // Blocks per SM: 16 registers per level and about 90 more.  Eight levels leave room for two blocks of four
@@ -317,7 +340,7 @@ __global__ void __launch_bounds__(32 * kRpWarps, rp_min_blocks<K>()) k_row_pipe(
     const typename IO::Elem *__restrict__ src, typename IO::Elem *__restrict__ dst, int nx, int ny, long long pitch,
     int H, int strips, int tiles, float w) {
     extern __shared__ __align__(16) char rp_smem[];
-    char *ring = rp_smem + (threadIdx.x >> 5) * (kStages * 4 * IO::kRow);
+    char *ring = rp_smem + (threadIdx.x >> 5) * (kStages * 4 * rp_row_bytes<IO>());
     const int tile = blockIdx.x * kRpWarps + (threadIdx.x >> 5);
     if (tile >= tiles) return;
     const int seg = tile / strips, y0 = seg * H;
@@ -339,7 +362,7 @@ __global__ void __launch_bounds__(32 * kRpWarps, rp_min_blocks<K>()) k_row_pipe_
     const float *__restrict__ src, float *__restrict__ dst, const RpDomain *__restrict__ doms,
     const int3 *__restrict__ tiles, int count) {
     extern __shared__ __align__(16) char rp_smem[];
-    char *ring = rp_smem + (threadIdx.x >> 5) * (kStages * 4 * RpF32::kRow);
+    char *ring = rp_smem + (threadIdx.x >> 5) * (kStages * 4 * rp_row_bytes<RpF32>());
     const int tile = blockIdx.x * kRpWarps + (threadIdx.x >> 5);
     if (tile >= count) return;
     const int3 t = tiles[tile];

@@ -249,8 +249,8 @@ struct SetImpl {
             });
         }
     }
-    // K steps per launch in 2D: FP32 storage with K = 2, 3, 4, 8 (the bits of single steps), or BFP16,
-    // FP16 and BF16 storage with K = 3, 4, 8 (FP32 levels in between, one rounding per launch)
+    // K steps per launch in 2D: FP32 storage with K = 2, 3, 4, 8 (the bits of single steps), FP16 and BF16
+    // with K = 3, 4, 8 and BFP16 with K = 3, 4 (FP32 levels in between; see rowpipe.cuh)
     template <class IO, class Fn>
     static cudaError_t with_steps(int k, Fn &&fn) {
         switch (k) {
@@ -259,7 +259,9 @@ struct SetImpl {
             return cudaErrorInvalidValue;
         case 3: return fn(std::integral_constant<int, 3>{});
         case 4: return fn(std::integral_constant<int, 4>{});
-        case kRpDeep: return fn(std::integral_constant<int, kRpDeep>{});
+        case kRpDeep:
+            if constexpr (IO::kAlign == 4) return fn(std::integral_constant<int, kRpDeep>{});
+            return cudaErrorInvalidValue;
         default: return cudaErrorInvalidValue;
         }
     }
@@ -361,6 +363,8 @@ struct SetImpl {
         o.stepk_prepare = S::D == 2 ? &stepk_prepare : nullptr;
         o.step3d2 = axis_only<S>() ? &step3d2 : nullptr;
         o.step3d2_prepare = axis_only<S>() ? &step3d2_prepare : nullptr;
+        o.step3dk = axis_only<S>() ? &plane_pipe_launch : nullptr;
+        o.step3dk_prepare = axis_only<S>() ? &plane_pipe_prepare : nullptr;
         o.edge_fixup = S::D == 2 ? &edge_fixup : nullptr;
         for (int i = 0; i < S::Q; ++i) {
             for (int a = 0; a < 3; ++a) o.c[i][a] = S::c(i, a);

@@ -1,10 +1,11 @@
 // step_launch.cuh -- launch configuration of the fused stream-collide kernels for one velocity set:
-// the one-step kernel (cells per thread, grid) and the 2D row pipeline (segment height from the
-// resident capacity).  Together with kernels.cuh and velsets.cuh this fixes what the
+// the one-step kernel (cells per thread, grid) the 2D row pipeline (segment height from the
+// resident capacity) and the 3D plane pipeline (tiles and segments likewise).  Together with kernels.cuh and velsets.cuh this fixes what the
 // profiled hot-path launches execute.
 #pragma once
 
 #include "ops.cuh"
+#include "planepipe.cuh"
 #include "rowpipe.cuh"
 
 namespace lee {
@@ -172,6 +173,46 @@ cudaError_t row_pipe_launch(const StepLaunch &L) {
     } else {
         return row_pipe_launch_stages<K, IO, kRpStages16>(L);
     }
+}
+
+// Plane pipeline (planepipe.cuh): the resident blocks of a device, set by plane_pipe_prepare outside any
+// stream capture, and the launch.
+inline int *plane_pipe_capacity() {
+    static int cap[64] = {0};
+    return cap;
+}
+inline cudaError_t plane_pipe_prepare() {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (plane_pipe_capacity()[dev]) return cudaSuccess;
+    constexpr int smem = pp_smem_bytes<kPpDeep>();
+    int per_sm = 0, sms = 0;
+    e = cudaFuncSetAttribute(k_plane_pipe<kPpDeep>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_plane_pipe<kPpDeep>, kPpThreads, smem);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    plane_pipe_capacity()[dev] = per_sm * sms > 0 ? per_sm * sms : 1;
+    return cudaSuccess;
+}
+inline cudaError_t plane_pipe_launch(const StepLaunch &L) {
+    if (L.storage != LEE_STORE_F32 || L.open || L.nx % 4 != 0) return cudaErrorInvalidValue;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    const int capacity = plane_pipe_capacity()[dev];
+    if (capacity == 0) return cudaErrorNotReady;  // prepare first
+    const PpCut cut = plane_pipe_cut(kPpDeep, pp_halo<kPpDeep>(), L.nx, L.ny, L.nz, capacity);
+    const long long gy = cut.C ? (L.ny + cut.height - 1) / cut.height : 0, gz = cut.C ? (L.nz + cut.HZ - 1) / cut.HZ : 0;
+    if (cut.C == 0 || gy > 65535 || gz > 65535) return cudaErrorInvalidValue;
+    const CollideCoef<float> cf = make_coef<float>(L.omega, L.coefM, L.coefN);
+    k_plane_pipe<kPpDeep><<<dim3((L.nx + cut.width - 1) / cut.width, (unsigned)gy, (unsigned)gz), kPpThreads,
+                            pp_smem_bytes<kPpDeep>(), L.stream>>>(static_cast<const float *>(L.src),
+                                                                  static_cast<float *>(L.dst), L.nx, L.ny, L.nz, L.pitch,
+                                                                  cut, cf.M[1][1]);
+    return cudaGetLastError();
 }
 
 }  // namespace lee

@@ -1,6 +1,7 @@
 // tb3d.cuh -- two time steps per launch (temporal blocking) in 3D for the axis-aligned
 // seven-velocity sets (D3Q7 and diatomic D3Q7, Sec. 8.3), periodic grids with nx % 4 == 0.
-// The solver uses it for FP32 storage, and for BFP16 storage (bfp.cuh; level 1 then stays in FP32,
+// The solver uses it for FP32 storage, for the two steps that runs of four (planepipe.cuh) leave and where
+// LEE_TB_STEPS=2 asks for it, and for BFP16 storage (bfp.cuh; level 1 then stays in FP32,
 // so a launch rounds to the storage once) when LEE_TB_STEPS=2 asks for it: with FP16/BF16, and with
 // BFP16's decoding and encoding, this latency-bound tile measured slower than the one-step kernel
 // (below; BFP16 on D3Q7 384^3: 124 against 196 GLUPS).

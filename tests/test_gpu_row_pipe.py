@@ -39,16 +39,19 @@ def test_fp32_runs_equal_single_steps(gpu_lib, monkeypatch, name, shape):
         assert np.array_equal(a, b), n
 
 
-@pytest.mark.parametrize("shape", [(16, 5, 1), (104, 7, 1), (112, 16, 1), (120, 9, 1), (264, 41, 1), (456, 203, 1)])
-@pytest.mark.parametrize("storage", ["f16", "bf16", "bfp16"])
-def test_16bit_launch_is_eight_fp32_steps(gpu_lib, monkeypatch, storage, shape):
-    """One launch of eight: the stored state widened, eight FP32 steps, rounded to the storage once.
-    (D2Q5's weights and the storage scale are powers of two, so the scaled steps round alike.)"""
+@pytest.mark.parametrize("shape", [(4, 3, 1), (12, 5, 1), (104, 7, 1), (112, 16, 1), (120, 9, 1), (264, 41, 1), (456, 203, 1)])
+@pytest.mark.parametrize("storage", ["f16", "bf16"])
+def test_16bit_launch_of_eight_is_two_of_four(gpu_lib, monkeypatch, storage, shape):
+    """The state is rounded to the storage after every four steps, whether one launch takes four or eight, so
+    runs give the same bits however the calls cut them at multiples of four."""
     lee = gpu_lib
-    kw = {"store_scale": 1024.0} if storage != "bfp16" else {}
     g0 = inputs.random_populations(5, int(np.prod(shape)), seed=6)
+    kw = {"store_scale": 1024.0}
+    a = _state(lee, monkeypatch, shape, storage, 24, g0, False, **kw)
+    b = _state(lee, monkeypatch, shape, storage, (4, 16, 4), g0, False, **kw)
     held = _state(lee, monkeypatch, shape, storage, 0, g0, False, **kw)
-    a = _state(lee, monkeypatch, shape, storage, 8, held, False, **kw)
-    f = _state(lee, monkeypatch, shape, "f32", 8, held, True)
-    b = _state(lee, monkeypatch, shape, storage, 0, f, False, **kw)
-    assert np.array_equal(a, b)
+    f = _state(lee, monkeypatch, shape, "f32", 4, held, True)
+    for _ in range(5):  # D2Q5's weights and the scale are powers of two: the FP32 steps round alike
+        f = _state(lee, monkeypatch, shape, "f32", 4, _state(lee, monkeypatch, shape, storage, 0, f, False, **kw), True)
+    c = _state(lee, monkeypatch, shape, storage, 0, f, False, **kw)
+    assert np.array_equal(a, b) and np.array_equal(a, c)
