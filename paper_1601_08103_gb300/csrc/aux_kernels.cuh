@@ -15,7 +15,7 @@ namespace lee {
 // on per-shell sums (every weight and coefficient depends on the shell |c_i|^2 only), so the
 // shell factors are folded on the host and each population costs one or two FP64 additions:
 //   g_i^eq = eqA[.][s] rho' + eqB[.][s] theta' + eqC[.][s] (c_i . u')   (i in shell s;
-//            [0] the population itself, [1] the scaled 16-bit value S g_i / f*_s, per unit S),
+//            [0] the population itself, [1] the scaled 16-bit value S g_i / f*_s),
 //   with eqA = F (a1 + s c1 / 2), eqB = F (a2 + s c2 / 2), eqC = F b, F = f*_s resp. 1;
 //   a stored 16-bit value decodes as g = dec[s] x stored, dec = f*_s / S (enc = 1 / dec);
 //   the energy moment weight of shell s is ew[s] = (s + beta_s) / 2;
@@ -82,6 +82,27 @@ __device__ __forceinline__ void equilibrium_cell(double r, double th, const doub
     });
 }
 
+// The auxiliary kernels are bound by GB300's FP64 pipe (two lanes per clock and SM), which also takes the
+// conversions between FP64 and the other types.  They keep FP64's precision with fewer of its
+// instructions: conversions and sums run on the integer pipes where that is exact.
+
+// (float)v, rounded to nearest even: on the integer pipe where v is a normal FP32 number.
+__device__ __forceinline__ float to_f32(double v) {
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    if (((hi >> 20) & 0x7FFu) - 897u < 254u) {
+        // half an FP32 unit less one, plus the kept part's last bit, carries exactly where v rounds up
+        const unsigned long long r = (((unsigned long long)hi << 32) | lo) + 0x0FFFFFFFull + ((lo >> 29) & 1u);
+        const unsigned kept = (unsigned)((r - (896ull << 52)) >> 29);
+        return __uint_as_float((kept & 0x7FFFFFFFu) | (hi & 0x80000000u));
+    }
+    return (float)v;
+}
+template <class C>
+__device__ __forceinline__ C to_store(double v) {
+    if constexpr (std::is_same<C, float>::value) return to_f32(v);
+    else return v;
+}
+
 // Writers of a state copy g also write the rest populations of the sets that leave them alone
 // (rest_static) into the other copy, `other`: a step neither reads nor writes them.
 
@@ -96,8 +117,7 @@ __global__ void k_init_equilibrium(const double *__restrict__ rho, const double 
 #pragma unroll
         for (int a = 0; a < S::D; ++a) uu[a] = u[(long long)a * cells + x];
         equilibrium_cell<S, SC>(rho[x], theta[x], uu, k, [&](int i, double v) {
-            if (SC) v *= k.scale;
-            const T e = Store<T>::make((typename Store<T>::C)v);
+            const T e = Store<T>::make(to_store<typename Store<T>::C>(v));
             g[(long long)i * pitch + x] = e;
             if (rest_static<S>() && i == 0) other[x] = e;
         });
@@ -110,13 +130,17 @@ template <class S>
 __global__ void k_init_maxabs(const double *__restrict__ rho, const double *__restrict__ u,
                               const double *__restrict__ theta, long long cells, SetConsts k,
                               unsigned int *__restrict__ maxbits) {
-    float m = 0.f;
+    unsigned long long mb = 0;  // of the magnitudes' bits, which order like the magnitudes
     for (long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x; x < cells; x += (long long)gridDim.x * blockDim.x) {
         double uu[3] = {0.0, 0.0, 0.0};
 #pragma unroll
         for (int a = 0; a < S::D; ++a) uu[a] = u[(long long)a * cells + x];
-        equilibrium_cell<S, 1>(rho[x], theta[x], uu, k, [&](int, double v) { m = fmaxf(m, (float)fabs(v)); });
+        equilibrium_cell<S, 1>(rho[x], theta[x], uu, k, [&](int, double v) {
+            const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
+            if (b <= 0x7FF0000000000000ull && b > mb) mb = b;  // (a NaN is left out, as fmaxf does)
+        });
     }
+    float m = (float)__longlong_as_double((long long)mb);  // the rounding keeps the order
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, off));
     if ((threadIdx.x & 31) == 0) atomicMax(maxbits, __float_as_uint(m));
@@ -220,7 +244,8 @@ __global__ void k_sponge_damp(T *__restrict__ g, T *__restrict__ other, GridDesc
 }
 
 // Per-shell sums of one cell's stored populations: P[slot] = sum g, J[slot][a] = sum c_a g (in
-// stored units), and whether every value is finite.
+// stored units), Sq[slot] = sum g^2, and whether every value is finite.  Velocities 2k-1 and 2k are
+// opposite, so every pair gives one sum and one difference.
 template <class S, class T>
 __device__ __forceinline__ bool shell_sums(const T *__restrict__ g, long long pitch, long long x,
                                            double (&P)[n_shells<S>()], double (&J)[n_shells<S>()][3],
@@ -228,51 +253,169 @@ __device__ __forceinline__ bool shell_sums(const T *__restrict__ g, long long pi
     bool finite = true;
     static_for<n_shells<S>()>([&](auto K) {
         constexpr int k = decltype(K)::value;
-        P[k] = 0.0;
+        P[k] = -0.0;  // the first addition folds away
         Sq[k] = 0.0;
-        J[k][0] = J[k][1] = J[k][2] = 0.0;
+        J[k][0] = J[k][1] = J[k][2] = -0.0;
     });
-    static_for<S::Q>([&](auto I) {
-        constexpr int i = decltype(I)::value;
+    const double rest = (double)load_elem<S, T>(g, pitch, x);
+    finite = isfinite(rest);
+    P[shell_slot<S>(0)] = rest;
+    Sq[shell_slot<S>(0)] = rest * rest;
+    static_for<S::Q / 2>([&](auto H) {
+        constexpr int i = 1 + 2 * decltype(H)::value;
         constexpr int k = shell_slot<S>(S::shell(i));
         const double v = (double)load_elem<S, T>(g, pitch, (long long)i * pitch + x);
-        finite = finite && isfinite(v);
-        P[k] += v;
-        Sq[k] = fma(v, v, Sq[k]);
+        const double o = (double)load_elem<S, T>(g, pitch, (long long)(i + 1) * pitch + x);
+        finite = finite && isfinite(v) && isfinite(o);
+        P[k] += v + o;
+        Sq[k] = fma(o, o, fma(v, v, Sq[k]));
+        const double d = v - o;
         static_for<3>([&](auto A) {
             constexpr int a = decltype(A)::value;
-            if constexpr (S::c(i, a) == 1) J[k][a] += v;
-            if constexpr (S::c(i, a) == -1) J[k][a] -= v;
+            if constexpr (S::c(i, a) == 1) J[k][a] += d;
+            if constexpr (S::c(i, a) == -1) J[k][a] -= d;
         });
     });
     return finite;
 }
 
+// Exact sums of values that are FP32 numbers (every storage but FP64) on the integer pipe.  With E the
+// largest biased exponent among them, a value is its 24-bit mantissa, shifted left by kFixBits and right by
+// its own distance from E: a 64-bit integer in units of 2^(E - 150 - kFixBits).  Nothing is lost down to
+// 2^-34 of the largest value and no more than 2^-58 of it below, which is finer than FP64 sums of them;
+// the sums are rounded to FP64 once.  Zeros and denormals (E of their own 0) shift out to nothing where E is
+// kFixLeast or more; smaller values, infinities and NaN take FP64 sums.
+constexpr int kFixBits = 34, kFixBitsSq = 10;
+constexpr unsigned kFixLeast = 64;
+__device__ __forceinline__ int fix_shift(unsigned bits, unsigned E) {
+    const int s = (int)(E - ((bits >> 23) & 0xFFu));
+    return s < 63 ? s : 63;
+}
+__device__ __forceinline__ long long fix_value(unsigned bits, int shift) {
+    const long long m = (long long)(((unsigned long long)((bits & 0x7FFFFFu) | 0x800000u) << kFixBits) >> shift);
+    const long long sign = (int)bits >> 31;
+    return (m ^ sign) - sign;
+}
+// Its square, in units of 2^(2 (E - 150) - kFixBitsSq); 63 of them fit in 64 bits.
+__device__ __forceinline__ unsigned long long fix_square(unsigned bits, int shift) {
+    const unsigned m = (bits & 0x7FFFFFu) | 0x800000u;
+    const int s = 2 * shift;
+    return (((unsigned long long)m * m) << kFixBitsSq) >> (s < 63 ? s : 63);
+}
+// v 2^e as FP64 (v rounded once, the exponent moved on the integer pipe).
+template <class I>
+__device__ __forceinline__ double fix_double(I v, int e) {
+    const double d = (double)v;
+    return v == 0 ? 0.0 : __hiloint2double(__double2hiint(d) + (e << 20), __double2loint(d));
+}
+template <class T>
+__host__ __device__ constexpr bool fixed_sums() {
+    return !std::is_same<T, double>::value;
+}
+
 // Per-cell moments (Sec. 4 discrete moments, Sec. 5 temperature) in FP64.
+// D3Q7 384^3 FP32: 2.89 ms with FP64 sums and conversions, 1.26 ms with integer ones (0.57 at the copy rate);
+// D3Q19 256^3: 2.44 -> 0.46 ms.
 template <class S, class T>
 __global__ void k_moments(const T *__restrict__ g, long long cells, long long pitch, SetConsts k, double *__restrict__ rho,
                           double *__restrict__ u, double *__restrict__ theta) {
     constexpr bool scaled = Store<T>::scaled;
-    constexpr int NS = n_shells<S>();
+    constexpr int NS = n_shells<S>(), D = S::D;
     for (long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x; x < cells; x += (long long)gridDim.x * blockDim.x) {
-        double P[NS], J[NS][3], Sq[NS];
-        shell_sums<S, T>(g, pitch, x, P, J, Sq);
-        double r = 0.0, e = 0.0, j[3] = {0.0, 0.0, 0.0};
+        // shell sums; where the storage is not scaled their total and the momentum over all shells, else the
+        // momentum of each
+        constexpr int NJ = scaled ? NS : 1;
+        double P[NS], J[NJ][3], total = 0.0;
+        bool done = false;
+        if constexpr (fixed_sums<T>()) {
+            unsigned b[S::Q], most = 0;
+            static_for<S::Q>([&](auto I) {
+                constexpr int i = decltype(I)::value;
+                b[i] = __float_as_uint((float)load_elem<S, T>(g, pitch, (long long)i * pitch + x));
+                const unsigned a = b[i] & 0x7FFFFFFFu;
+                most = a > most ? a : most;
+            });
+            const unsigned E = most >> 23;
+            if (most == 0) {
+                done = true;
+#pragma unroll
+                for (int s = 0; s < NS; ++s) P[s] = 0.0;
+#pragma unroll
+                for (int s = 0; s < NJ; ++s) J[s][0] = J[s][1] = J[s][2] = 0.0;
+            } else if (E >= kFixLeast && E < 255u) {
+                done = true;
+                long long p[NS], j[NJ][3];
+#pragma unroll
+                for (int s = 0; s < NS; ++s) p[s] = 0;
+#pragma unroll
+                for (int s = 0; s < NJ; ++s) j[s][0] = j[s][1] = j[s][2] = 0;
+                static_for<S::Q>([&](auto I) {
+                    constexpr int i = decltype(I)::value;
+                    constexpr int s = shell_slot<S>(S::shell(i)), sj = scaled ? s : 0;
+                    const long long v = fix_value(b[i], fix_shift(b[i], E));
+                    p[s] += v;
+                    static_for<D>([&](auto A) {
+                        constexpr int a = decltype(A)::value;
+                        if constexpr (S::c(i, a) == 1) j[sj][a] += v;
+                        if constexpr (S::c(i, a) == -1) j[sj][a] -= v;
+                    });
+                });
+                const int e = (int)E - 150 - kFixBits;
+                long long all = 0;
+#pragma unroll
+                for (int s = 0; s < NS; ++s) {
+                    all += p[s];
+                    if (scaled || s > 0) P[s] = fix_double(p[s], e);
+                }
+                if constexpr (!scaled) total = fix_double(all, e);
+                if (u) {
+#pragma unroll
+                    for (int s = 0; s < NJ; ++s)
+#pragma unroll
+                        for (int a = 0; a < D; ++a) J[s][a] = fix_double(j[s][a], e);
+                }
+            }
+        }
+        if (!done) {
+            double Js[NS][3], Sq[NS];
+            shell_sums<S, T>(g, pitch, x, P, Js, Sq);
+            total = -0.0;
+#pragma unroll
+            for (int s = 0; s < NS; ++s) total += P[s];
+#pragma unroll
+            for (int a = 0; a < D; ++a) {
+                if constexpr (scaled) {
+#pragma unroll
+                    for (int s = 0; s < NS; ++s) J[s][a] = Js[s][a];
+                } else {
+                    J[0][a] = -0.0;
+#pragma unroll
+                    for (int s = 1; s < NS; ++s) J[0][a] += Js[s][a];
+                }
+            }
+        }
+        double r = scaled ? -0.0 : total, e = -0.0, j[3] = {-0.0, -0.0, -0.0};
         static_for<4>([&](auto Sx) {
             constexpr int s = decltype(Sx)::value;
             if constexpr (shell_present<S>(s)) {
                 constexpr int kk = shell_slot<S>(s);
-                const double p = scaled ? P[kk] * k.dec[s] : P[kk];
-                r += p;
-                e = fma(k.ew[s], p, e);
+                if constexpr (scaled) r = fma(P[kk], k.dec[s], r);
+                if constexpr (s > 0) {  // (the rest shell has no energy and no momentum)
+                    e = fma(k.ew[s], scaled ? P[kk] * k.dec[s] : P[kk], e);
+                    if constexpr (scaled) {
 #pragma unroll
-                for (int a = 0; a < S::D; ++a) j[a] += scaled ? J[kk][a] * k.dec[s] : J[kk][a];
+                        for (int a = 0; a < D; ++a) j[a] = fma(J[kk][a], k.dec[s], j[a]);
+                    }
+                }
             }
         });
         if (rho) rho[x] = r;
         if (u) {
 #pragma unroll
-            for (int a = 0; a < S::D; ++a) u[(long long)a * cells + x] = j[a] * k.inv_rho0;
+            for (int a = 0; a < D; ++a) {
+                const double ja = scaled ? j[a] : J[0][a];
+                u[(long long)a * cells + x] = k.inv_rho0 == 1.0 ? ja : ja * k.inv_rho0;
+            }
         }
         if (theta) theta[x] = fma(k.kE, e, -k.kR * r);
     }
@@ -290,46 +433,153 @@ __host__ __device__ constexpr int reduce_nraw() {
     return 2 * n_shells<S>() + n_shells<S>() * S::D + 1;
 }
 
+// Adds one cell in FP64: the cells that the integer form leaves.
+template <class S, class T>
+__device__ __forceinline__ void reduce_cell(const T *__restrict__ g, long long pitch, long long x,
+                                            double (&acc)[reduce_nraw<S>()]) {
+    constexpr int NS = n_shells<S>(), D = S::D, NR = reduce_nraw<S>();
+    static_for<S::Q>([&](auto I) {
+        constexpr int i = decltype(I)::value;
+        constexpr int k = shell_slot<S>(S::shell(i));
+        const double v = (double)load_elem<S, T>(g, pitch, (long long)i * pitch + x);
+        if (isfinite(v)) {
+            acc[k] += v;
+            acc[NS + k] = fma(v, v, acc[NS + k]);
+            static_for<D>([&](auto A) {
+                constexpr int a = decltype(A)::value;
+                if constexpr (S::c(i, a) == 1) acc[2 * NS + k * D + a] += v;
+                if constexpr (S::c(i, a) == -1) acc[2 * NS + k * D + a] -= v;
+            });
+        } else {
+            acc[NR - 1] += 1.0;  // counted and left out
+        }
+    });
+}
+// FP64 accumulators of a thread for FP64 states: one sum per velocity and one sum of squares per shell (two
+// FP64 instructions per value; the shells' sums and momenta are put together once, at the end).
+template <class S>
+struct ReduceSums {
+    double g[S::Q], sq[n_shells<S>()], bad;
+};
+template <class S>
+__device__ __forceinline__ void reduce_cell(const double *__restrict__ g, long long pitch, long long x,
+                                            ReduceSums<S> &acc) {
+    static_for<S::Q>([&](auto I) {
+        constexpr int i = decltype(I)::value;
+        const double v = g[(long long)i * pitch + x];
+        if (isfinite(v)) {
+            acc.g[i] += v;
+            acc.sq[shell_slot<S>(S::shell(i))] = fma(v, v, acc.sq[shell_slot<S>(S::shell(i))]);
+        } else {
+            acc.bad += 1.0;
+        }
+    });
+}
+
+// One block's share: chunks of kReduceGroup cells per thread, a block's width apart.  FP32 and 16-bit values
+// of a thread's group are added as integers and reach the FP64 accumulators as one value per sum
+// (D3Q7 384^3 FP32: 4.32 ms with FP64 sums of every value, 0.70 ms so, 0.24 at the copy rate; D3Q19 256^3 3.81 ->
+// 0.70 ms).
+constexpr int kReduceGroup = 4;
 template <class S, class T>
 __global__ void __launch_bounds__(kReduceThreads) k_reduce_partial(const T *__restrict__ g, long long cells, long long pitch,
                                                                    double *__restrict__ partial) {
-    constexpr int NS = n_shells<S>(), D = S::D, NR = reduce_nraw<S>();
+    constexpr int NS = n_shells<S>(), D = S::D, NR = reduce_nraw<S>(), G = kReduceGroup;
     static_assert(NR <= kReduceMax, "raw accumulators do not fit");
+    static_assert(G * 12 <= 63, "integer sums of a shell of up to 12 velocities");
     double acc[NR];
 #pragma unroll
     for (int v = 0; v < NR; ++v) acc[v] = 0.0;
-    for (long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x; x < cells; x += (long long)gridDim.x * blockDim.x) {
-        double P[NS], J[NS][3], Sq[NS];
-        if (!shell_sums<S, T>(g, pitch, x, P, J, Sq)) {
-            // count the non-finite values of this cell; its finite ones still add up
-            static_for<S::Q>([&](auto I) {
-                constexpr int i = decltype(I)::value;
-                const double v = (double)load_elem<S, T>(g, pitch, (long long)i * pitch + x);
-                if (!isfinite(v)) acc[NR - 1] += 1.0;
-            });
-            static_for<S::Q>([&](auto I) {
-                constexpr int i = decltype(I)::value;
-                constexpr int k = shell_slot<S>(S::shell(i));
-                const double v = (double)load_elem<S, T>(g, pitch, (long long)i * pitch + x);
-                if (isfinite(v)) {
-                    acc[k] += v;
-                    acc[NS + k] = fma(v, v, acc[NS + k]);
-                    static_for<D>([&](auto A) {
-                        constexpr int a = decltype(A)::value;
-                        if constexpr (S::c(i, a) == 1) acc[2 * NS + k * D + a] += v;
-                        if constexpr (S::c(i, a) == -1) acc[2 * NS + k * D + a] -= v;
+    [[maybe_unused]] ReduceSums<S> each;
+    if constexpr (!fixed_sums<T>()) {
+#pragma unroll
+        for (int v = 0; v < S::Q; ++v) each.g[v] = 0.0;
+#pragma unroll
+        for (int v = 0; v < NS; ++v) each.sq[v] = 0.0;
+        each.bad = 0.0;
+    }
+    const long long span = (long long)kReduceThreads * G;
+    for (long long x0 = (long long)blockIdx.x * span + threadIdx.x; x0 < cells; x0 += (long long)gridDim.x * span) {
+        if constexpr (fixed_sums<T>()) {
+            unsigned b[G][S::Q], most = 0;
+#pragma unroll
+            for (int c = 0; c < G; ++c) {
+                const long long x = x0 + (long long)c * kReduceThreads;
+                const bool in = x < cells;
+                static_for<S::Q>([&](auto I) {
+                    constexpr int i = decltype(I)::value;
+                    b[c][i] = in ? __float_as_uint((float)load_elem<S, T>(g, pitch, (long long)i * pitch + x)) : 0u;
+                    const unsigned a = b[c][i] & 0x7FFFFFFFu;
+                    most = a > most ? a : most;
+                });
+            }
+            const unsigned E = most >> 23;
+            if (most == 0) continue;  // (zeros add nothing)
+            if (E >= kFixLeast && E < 255u) {
+                long long p[NS], j[NS][3];
+                unsigned long long q[NS];
+#pragma unroll
+                for (int s = 0; s < NS; ++s) {
+                    q[s] = 0;
+                    p[s] = j[s][0] = j[s][1] = j[s][2] = 0;
+                }
+#pragma unroll
+                for (int c = 0; c < G; ++c) {
+                    static_for<S::Q>([&](auto I) {
+                        constexpr int i = decltype(I)::value;
+                        constexpr int s = shell_slot<S>(S::shell(i));
+                        const int shift = fix_shift(b[c][i], E);
+                        const long long v = fix_value(b[c][i], shift);
+                        p[s] += v;
+                        q[s] += fix_square(b[c][i], shift);
+                        static_for<D>([&](auto A) {
+                            constexpr int a = decltype(A)::value;
+                            if constexpr (S::c(i, a) == 1) j[s][a] += v;
+                            if constexpr (S::c(i, a) == -1) j[s][a] -= v;
+                        });
                     });
                 }
-            });
-            continue;
-        }
-        static_for<NS>([&](auto K) {
-            constexpr int k = decltype(K)::value;
-            acc[k] += P[k];
-            acc[NS + k] += Sq[k];
+                const int e = (int)E - 150;
+                static_for<NS>([&](auto Kx) {
+                    constexpr int k = decltype(Kx)::value;
+                    acc[k] += fix_double(p[k], e - kFixBits);
+                    acc[NS + k] += fix_double(q[k], 2 * e - kFixBitsSq);
+                    if constexpr (k > 0) {
 #pragma unroll
-            for (int a = 0; a < D; ++a) acc[2 * NS + k * D + a] += J[k][a];
+                        for (int a = 0; a < D; ++a) acc[2 * NS + k * D + a] += fix_double(j[k][a], e - kFixBits);
+                    }
+                });
+                continue;
+            }
+        }
+        if constexpr (fixed_sums<T>()) {
+#pragma unroll 1
+            for (int c = 0; c < G; ++c) {
+                const long long x = x0 + (long long)c * kReduceThreads;
+                if (x < cells) reduce_cell<S, T>(g, pitch, x, acc);
+            }
+        } else {
+#pragma unroll
+            for (int c = 0; c < G; ++c) {
+                const long long x = x0 + (long long)c * kReduceThreads;
+                if (x < cells) reduce_cell<S>(g, pitch, x, each);
+            }
+        }
+    }
+    if constexpr (!fixed_sums<T>()) {
+        static_for<S::Q>([&](auto I) {
+            constexpr int i = decltype(I)::value;
+            constexpr int k = shell_slot<S>(S::shell(i));
+            acc[k] += each.g[i];
+            static_for<D>([&](auto A) {
+                constexpr int a = decltype(A)::value;
+                if constexpr (S::c(i, a) == 1) acc[2 * NS + k * D + a] += each.g[i];
+                if constexpr (S::c(i, a) == -1) acc[2 * NS + k * D + a] -= each.g[i];
+            });
         });
+#pragma unroll
+        for (int k = 0; k < NS; ++k) acc[NS + k] = each.sq[k];
+        acc[NR - 1] = each.bad;
     }
     __shared__ double sh[kReduceThreads / 32][NR];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -486,7 +736,7 @@ __global__ void k_init_equilibrium_bfp(const double *__restrict__ rho, const dou
         double uu[3] = {0.0, 0.0, 0.0};
 #pragma unroll
         for (int a = 0; a < S::D; ++a) uu[a] = u[(long long)a * cells + x];
-        equilibrium_cell<S, 0>(rho[x], theta[x], uu, k, [&](int i, double val) { v[i] = (float)val; });
+        equilibrium_cell<S, 0>(rho[x], theta[x], uu, k, [&](int i, double val) { v[i] = to_f32(val); });
     });
 }
 

@@ -163,9 +163,9 @@ SetConsts host_consts(double scale) {
         k.eqA[0][s] = k.f[s] * fa;
         k.eqB[0][s] = k.f[s] * fb;
         k.eqC[0][s] = k.f[s] * k.b;
-        k.eqA[1][s] = fa;
-        k.eqB[1][s] = fb;
-        k.eqC[1][s] = k.b;
+        k.eqA[1][s] = scale * fa;  // (a power of two: exact)
+        k.eqB[1][s] = scale * fb;
+        k.eqC[1][s] = scale * k.b;
         k.dec[s] = k.f[s] / scale;
         k.enc[s] = k.f[s] > 0.0 ? scale / k.f[s] : 0.0;
         k.ew[s] = 0.5 * (s + k.beta[s]);
@@ -206,6 +206,16 @@ inline int aux_blocks(long long cells, int threads = 256) {
     if (b > kMaxAuxBlocks) b = kMaxAuxBlocks;
     if (b < 1) b = 1;
     return (int)b;
+}
+
+// Blocks of a reduction: as many as fit on the SMs at once.  A block's own reduction (a dozen FP64 sums over its
+// warps) costs as much as some thousand cells on GB300's FP64 pipe: with the 16 blocks per SM of the other
+// auxiliary kernels it took 45 us of a 2048^2 FP32 reduction.
+inline int reduce_blocks(long long cells) {
+    constexpr int kMost = 152 * 3;
+    static_assert(kMost <= kMaxAuxBlocks, "rows of the partial-sum buffers");
+    const long long b = (cells + kReduceThreads * kReduceGroup - 1) / (kReduceThreads * kReduceGroup);
+    return (int)(b > kMost ? kMost : b < 1 ? 1 : b);
 }
 
 }  // namespace lee

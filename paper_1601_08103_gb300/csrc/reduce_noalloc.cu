@@ -66,7 +66,7 @@ extern "C" lee_status lee_reduce_noalloc(int32_t set, int32_t storage, const voi
     if (cells < 1 || cells >= (1LL << 31) || pitch < cells) return LEE_ERR_INVALID_ARGUMENT;
     const bool is16 = storage == LEE_STORE_F16 || storage == LEE_STORE_BF16;
     if (is16 && !(store_scale > 0.0)) return LEE_ERR_INVALID_ARGUMENT;
-    const int nblocks = aux_blocks(cells, kReduceThreads);
+    const int nblocks = reduce_blocks(cells);
     if (nblocks > kMaxPartials) return LEE_ERR_INVALID_ARGUMENT;  // beyond the fixed scratch
     double *partials = nullptr;
     if (partials_on_current_device(&partials) != cudaSuccess) return LEE_ERR_CUDA;
