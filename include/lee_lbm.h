@@ -205,7 +205,10 @@ lee_status lee_lbm_init_fields(lee_lbm *h, const double *rho, const double *u, c
  *    storage after every four steps (or three with LEE_TB_STEPS=3; a launch of eight rounds after its first
  *    four steps too), with single steps for the rest (LEE_TB_STEPS=1 or 2 keeps one step per launch,
  *    rounding every step);
- *  - a 1D grid (not BFP16) whose two population copies fit in shared memory (2 q nx sizeof(storage) <= 227 KB,
+ *  - 1D grids without a sponge frame (FP64, FP32, FP16, BF16) run all n >= 2 steps in one launch that moves the
+ *    populations by n cells: the collision of the 1D set is the identity (Sec. 8.1).  LEE_TB_STEPS
+ *    or LEE_SINGLE_STEP in the environment at create time keeps the step kernels;
+ *  - else a 1D grid (not BFP16) whose two population copies fit in shared memory (2 q nx sizeof(storage) <= 227 KB,
  *    e.g. D1Q3 FP64 up to 4843 cells) runs all n >= 2 steps in one launch: one block, or from
  *    512 cells a thread-block cluster of 8 blocks;
  *  - OPEN_LEARNED: one launch per step whose first blocks run the boundary network and write the

@@ -231,6 +231,15 @@ bool onchip(const lee_lbm *h) {
            2 * h->elem * (size_t)h->Q * (size_t)h->cfg.nx <= (size_t)kMaxOnchipSmem;
 }
 
+// Whether a run of this 1D grid is one move of its populations (k_shift_1d): no frame, and not where the
+// environment asked for single steps.
+bool shifted(const lee_lbm *h) {
+    return h->ops->shift_1d && (h->cfg.bc == LEE_BC_PERIODIC || h->cfg.bc == LEE_BC_OPEN_ZERO) &&
+           (h->cfg.storage == LEE_STORE_F64 || h->cfg.storage == LEE_STORE_F32 || h->cfg.storage == LEE_STORE_F16 ||
+            h->cfg.storage == LEE_STORE_BF16) &&
+           h->tb_steps == 4 && !h->tb_env;
+}
+
 lee_status cuda_fail(lee_lbm *h, cudaError_t e, const char *what) {
     std::string m = std::string(what) + ": " + cudaGetErrorString(e);
     if (e == cudaErrorMemoryAllocation) return fail(h, LEE_ERR_OUT_OF_MEMORY, m);
@@ -667,6 +676,15 @@ lee_status lee_lbm_step(lee_lbm *h, int64_t n) {
         if (e == cudaSuccess) e = cudaStreamWaitEvent(st, h->ev_join, 0);
         return e;
     };
+    if (n >= 2 && shifted(h)) {
+        L.src = state(h, h->cur);
+        L.dst = state(h, h->cur ^ 1);
+        L.stream = h->st;
+        LEE_CK(h, h->ops->shift_1d(L, n), "1D shift launch");
+        h->cur ^= 1;
+        h->steps += n;
+        return LEE_OK;
+    }
     // 1D grids that fit in shared memory: every step in one launch of the on-chip kernel
     if (n >= 2 && onchip(h)) {
         L.stream = h->st;

@@ -88,6 +88,9 @@ struct SetOps {
     // all steps of a small 1D grid in one launch, in place on g (nullptr for 2D/3D sets);
     // returns cudaErrorInvalidValue when the grid does not fit in shared memory
     cudaError_t (*onchip_1d)(const StepLaunch &L, void *g, long long nsteps);
+    // n >= 1 steps of a 1D grid without a sponge frame in one launch, from L.src to L.dst (nullptr for 2D/3D
+    // sets; not for BFP16 and split storage)
+    cudaError_t (*shift_1d)(const StepLaunch &L, long long n);
     // the border cells of an open 2D grid for one step of the learned edge (k_edge_fixup): pulled
     // from L.src with the entering populations L.ghost, collided, stored in L.dst; nullptr for 1D/3D
     cudaError_t (*edge_fixup)(const StepLaunch &L);

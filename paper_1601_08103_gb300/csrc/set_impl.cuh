@@ -249,6 +249,25 @@ struct SetImpl {
             });
         }
     }
+    // n steps without a frame (k_shift_1d), from L.src to L.dst
+    static cudaError_t shift_1d(const StepLaunch &L, long long n) {
+        if constexpr (S::D != 1) {
+            return cudaErrorInvalidValue;
+        } else {
+            return with_storage(L.storage, [&](auto *tp) -> cudaError_t {
+                using T = std::remove_pointer_t<decltype(tp)>;
+                if constexpr (std::is_same<T, Bfp16>::value) {
+                    return cudaErrorInvalidValue;  // blocks are encoded anew where they move
+                } else {
+                    if (L.open && L.sponge_w > 0) return cudaErrorInvalidValue;
+                    const int by = L.open ? (int)(n < L.nx ? n : L.nx) : (int)(n % L.nx);
+                    k_shift_1d<T><<<aux_blocks(L.nx), 256, 0, L.stream>>>(static_cast<const T *>(L.src),
+                                                                         static_cast<T *>(L.dst), L.nx, L.pitch, by, L.open);
+                    return cudaGetLastError();
+                }
+            });
+        }
+    }
     // K steps per launch in 2D: FP32 storage with K = 2, 3, 4, 8 (the bits of single steps), FP16 and BF16
     // with K = 3, 4, 8 and BFP16 with K = 3, 4 (FP32 levels in between; see rowpipe.cuh)
     template <class IO, class Fn>
@@ -359,6 +378,7 @@ struct SetImpl {
         o.slab_unpack = S::D >= 2 ? &slab_unpack : nullptr;
         o.slab_crossing = slab_crossing<S>();
         o.onchip_1d = S::D == 1 ? &onchip_1d : nullptr;
+        o.shift_1d = S::D == 1 ? &shift_1d : nullptr;
         o.stepk = S::D == 2 ? &stepk : nullptr;
         o.stepk_prepare = S::D == 2 ? &stepk_prepare : nullptr;
         o.step3d2 = axis_only<S>() ? &step3d2 : nullptr;
