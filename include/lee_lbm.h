@@ -188,13 +188,14 @@ lee_status lee_lbm_init_fields(lee_lbm *h, const double *rho, const double *u, c
  * graph (one graph holding all n steps for n <= 4096, else repeated 96-step graphs), captured on
  * first use of that length on a private stream and cached in the handle; results are identical to
  * direct launches.  Every form below also gives the same bits as single one-step launches:
- *  - periodic 2D FP32 grids with nx a multiple of 4 advance several steps per launch, the
+ *  - periodic 2D FP32 grids advance several steps per launch, the
  *    intermediate states kept in registers (temporal blocking): eight while the call has that many
  *    left, then four, then the two or three or one that remain.  LEE_TB_STEPS=1..4 in the
- *    environment at create time fixes the count instead (n / count launches, n % count single steps);
- *  - periodic 3D FP32 grids of D3Q7 and diatomic D3Q7 with nx a multiple of 4 advance four steps per
- *    launch (a pipeline of the planes), then two (a z-marching tile), then one; grids of fewer than
- *    786432 cells, where that is slower, take single steps (LEE_TB_STEPS=1 or 2 fixes the count);
+ *    environment at create time fixes the count instead (n / count launches, n % count single steps;
+ *    grids with nx not a multiple of 4 then take single steps);
+ *  - periodic 3D FP32 grids of D3Q7 and diatomic D3Q7 advance four steps per launch (a pipeline of the
+ *    planes), then, with nx a multiple of 4, two (a z-marching tile), then one; grids of fewer than
+ *    786432 cells (2097152 where nx is not a multiple of 4), where that is slower, take single steps (LEE_TB_STEPS=1 or 2 fixes the count);
  *  - BFP16 storage on those periodic 2D grids with nx a multiple of 8 uses the same kernels (four steps
  *    per launch, the rest as single steps; or three with LEE_TB_STEPS=3), but keeps the
  *    intermediate states in FP32 and encodes only the last one: a launch of k steps equals decoding
@@ -300,7 +301,8 @@ lee_status lee_lbm_steps_done(lee_lbm *h, int64_t *steps);
  * multiple of 4: 4 unless LEE_TB_STEPS was set at create time; FP32, FP16 and BF16 calls take two such
  * runs, eight steps, in one launch where they can (not with LEE_TB_STEPS).  Periodic 3D FP32 D3Q7 and
  * diatomic D3Q7 grids with nx a multiple of 4: 2 (calls take two such runs in one launch where they can,
- * and small grids single steps).  BFP16 storage: 3 or 4 in 2D on such grids with nx a multiple of 8, 2
+ * and small grids single steps).  Other FP32 grids of these kinds, with nx not a multiple of 4, give 1 and
+ * are run in the same launches where LEE_TB_STEPS was not set.  BFP16 storage: 3 or 4 in 2D on such grids with nx a multiple of 8, 2
  * in 3D only with LEE_TB_STEPS=2; FP16 / BF16 storage: 3 or 4 in 2D on such grids.  All forms give
  * bit-identical results, except that BFP16, FP16 and BF16 storage round their state once per run of *steps
  * (see lee_lbm_step). */

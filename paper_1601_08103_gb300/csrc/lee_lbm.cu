@@ -199,10 +199,17 @@ int fused_steps(const lee_lbm *h) {
 // asked for a count or the TMA-fed tile.
 bool plane_pipe(const lee_lbm *h) {
     return h->ops->step3dk && h->cfg.bc == LEE_BC_PERIODIC && h->cfg.storage == LEE_STORE_F32 && h->tb_steps == 4 &&
-           !h->tb_env && !tma_tile(h) && plane_pipe_eligible(h->cfg.nx, h->cfg.ny);
+           !h->tb_env && !tma_tile(h) && plane_pipe_eligible(h->cfg.ny);
 }
 
-constexpr long long kFuse3dCells = 3LL << 18;
+constexpr long long kFuse3dCells = 3LL << 18, kFuse3dRaggedCells = 1LL << 21;
+
+// Whether this is a 2D FP32 grid for the row pipeline's form for widths that are not multiples of 4
+// (steps_per_launch is 1 there; the bits are those of single steps).
+bool ragged_2d(const lee_lbm *h) {
+    return h->ops->stepk && h->cfg.bc == LEE_BC_PERIODIC && h->cfg.storage == LEE_STORE_F32 && h->cfg.nx % 4 != 0 &&
+           h->cfg.ny >= 3 && h->tb_steps == 4 && !h->tb_env;
+}
 
 // Steps of the next launch of a run with `left` steps to go.  Unless LEE_TB_STEPS asked for a count, grids
 // on the row pipeline take kRpDeep steps at a time while they can (two units in one launch, with the
@@ -210,16 +217,19 @@ constexpr long long kFuse3dCells = 3LL << 18;
 // or three that remain in one launch too (a 16-bit state would be rounded at other steps); 3D grids on the
 // plane pipeline take kPpDeep.  3D FP32 grids of fewer than kFuse3dCells cells take single steps: their few
 // tiles leave SMs idle in either fused kernel (us per step of one / two / four steps per launch: 64^3 2.5 /
-// 3.7 / 2.9, 80^3 3.7 / 4.8 / 3.8, 96^3 4.8 / 5.9 / 4.5, 128^3 - / 10.2 / 7.9).
+// 3.7 / 2.9, 80^3 3.7 / 4.8 / 3.8, 96^3 4.8 / 5.9 / 4.5, 128^3 - / 10.2 / 7.9; widths that are not multiples of 4,
+// copied word by word, 97x99x98 8.2 / - / 8.4, 193x161x135 33.7 / - / 27.1).
+// 2D FP32 at such widths: 2047x2045 160 GLUPS with single steps, 920 on the row pipeline.
 // Measured on GB300, GLUPS: D2Q5 FP32 2048^2 / 8192^2 four steps per launch 740 / 811, eight 1490 / 1611; D3Q7
 // FP32 384^3 / 256^3 two 259 / 232, four 373 / 334.
 int next_launch(const lee_lbm *h, int unit, long long left) {
+    if (ragged_2d(h)) return left >= kRpDeep ? kRpDeep : left >= 4 ? 4 : (int)left;
     if (unit > 1 && h->D == 2 && !h->tb_env) {
         if (left >= kRpDeep && h->cfg.storage != LEE_STORE_BFP16) return kRpDeep;
         if (left < unit && left > 1 && h->cfg.storage == LEE_STORE_F32) return (int)left;
     }
     if (h->D == 3 && plane_pipe(h)) {
-        if (h->cells < kFuse3dCells) return 1;
+        if (h->cells < (h->cfg.nx % 4 == 0 ? kFuse3dCells : kFuse3dRaggedCells)) return 1;
         if (left >= kPpDeep) return kPpDeep;
     }
     return left >= unit ? unit : 1;
@@ -528,13 +538,13 @@ lee_status lee_lbm_create(const lee_lbm_config *cfg, lee_lbm **out) {
         if (e == cudaSuccess) e = cudaMalloc(&h->corner, 4 * sizeof(unsigned long long));
         if (e == cudaSuccess) e = cudaMemsetAsync(h->corner, 0, 4 * sizeof(unsigned long long), h->st);
     }
-    if (e == cudaSuccess && h->D == 2 && fused_steps(h) > 1) {
+    if (e == cudaSuccess && h->D == 2 && (fused_steps(h) > 1 || ragged_2d(h))) {
         const int deep = h->tb_env || cfg->storage == LEE_STORE_BFP16 ? 0 : kRpDeep;
         for (int k : {2, 3, 4, deep})
             if (e == cudaSuccess && k > 0 && (h->tb_env ? k == h->tb_steps : k != 2 || cfg->storage == LEE_STORE_F32))
-                e = o->stepk_prepare(k, cfg->storage);
+                e = o->stepk_prepare(k, cfg->storage, (int)cfg->nx);
     }
-    if (e == cudaSuccess && plane_pipe(h)) e = o->step3dk_prepare();
+    if (e == cudaSuccess && plane_pipe(h)) e = o->step3dk_prepare((int)cfg->nx);
     if (e == cudaSuccess && h->tb_steps >= 2 && tiled_3d(h)) e = o->step3d2_prepare(cfg->storage, tma_tile(h) ? 1 : 0);
     if (e == cudaSuccess && tma_tile(h)) {
         e = cudaHostAlloc(reinterpret_cast<void **>(&h->wait_host), sizeof(unsigned), cudaHostAllocMapped);

@@ -16,7 +16,7 @@ constexpr int kRpDeep = 8;
 // Time steps per launch of the 3D plane pipeline, and the grids it takes (a launch has at most 65535 tiles
 // along y, of one row at least).
 constexpr int kPpDeep = 4;
-inline bool plane_pipe_eligible(long long nx, long long ny) { return nx % 4 == 0 && ny <= 65535; }
+inline bool plane_pipe_eligible(long long ny) { return ny <= 65535; }
 
 // Launch description of one fused time step.
 struct StepLaunch {
@@ -54,20 +54,20 @@ struct SetOps {
     // one fused pull-stream + collide step
     cudaError_t (*step)(const StepLaunch &);
     // k fused steps per launch of the 2D row pipeline (periodic grids; reads L.src, writes the state k
-    // steps later into L.dst): FP32 with nx % 4 == 0 and k = 2, 3, 4 or kRpDeep; FP16 / BF16 with
-    // nx % 4 == 0 and BFP16 with nx % 8 == 0 and k = 3, 4 or kRpDeep.  stepk_prepare: its one-time
-    // set-up on the current device for a storage type, outside stream capture
+    // steps later into L.dst): FP32 with k = 2, 3, 4 or kRpDeep; FP16 / BF16 with nx % 4 == 0 and k = 3, 4 or
+    // kRpDeep; BFP16 with nx % 8 == 0 and k = 3 or 4.  stepk_prepare: its one-time set-up on the current
+    // device for a storage type and width, outside stream capture
     cudaError_t (*stepk)(const StepLaunch &, int k);
-    cudaError_t (*stepk_prepare)(int k, int storage);
+    cudaError_t (*stepk_prepare)(int k, int storage, int nx);
     // two fused steps per launch for the 3D axis-velocity sets (periodic; FP32 with nx % 4 == 0
     // or BFP16 with nx % 8 == 0; nullptr for other sets), and its one-time set-up for a storage type
     // and kernel (tma = 1: the TMA-fed tile, which also needs t3t_eligible grids)
     cudaError_t (*step3d2)(const StepLaunch &);
     cudaError_t (*step3d2_prepare)(int storage, int tma);
     // kPpDeep fused steps per launch for the same sets (FP32, plane_pipe_eligible grids), and its one-time
-    // set-up
+    // set-up for a width
     cudaError_t (*step3dk)(const StepLaunch &);
-    cudaError_t (*step3dk_prepare)();
+    cudaError_t (*step3dk_prepare)(int nx);
     // g = g^eq(fields) (fields FP64 on device).  init, import_f64 and sponge_damp write a whole state
     // copy g; `other` is the other copy, whose rest populations they write too where a step leaves
     // those alone (rest_static)

@@ -1,6 +1,5 @@
 // planepipe.cuh -- K time steps per launch on periodic 3D FP32 grids of the seven-velocity sets (D3Q7 and
-// diatomic D3Q7) with nx % 4 == 0: a block marches through the planes with all K levels of the pipeline
-// in registers.
+// diatomic D3Q7): a block marches through the planes with all K levels of the pipeline in registers.
 //
 // A block of T threads owns a tile of columns and rows and a segment of planes.  Thread t holds four
 // adjacent cells (chunk t % C of row t / C of the tile) as an even and an odd pair (see rowpipe.cuh).
@@ -96,7 +95,8 @@ inline PpCut plane_pipe_cut(int K, int halo, int nx, int ny, int nz, int capacit
     return best;
 }
 
-template <int K>
+// kRagged: nx is not a multiple of 4, and the four cells of a thread are copied and stored one by one.
+template <int K, bool kRagged>
 __global__ void __launch_bounds__(kPpThreads, 1) k_plane_pipe(const float *__restrict__ src, float *__restrict__ dst,
                                                               int nx, int ny, int nz, long long pitch, PpCut cut,
                                                               float w) {
@@ -132,6 +132,9 @@ __global__ void __launch_bounds__(kPpThreads, 1) k_plane_pipe(const float *__res
     // the thread's four cells in rows y-1, y and y+1 of a plane
     const int xa = wrap(col, nx);
     const int row_of[3] = {wrap(y - 1, ny) * nx + xa, wrap(y, ny) * nx + xa, wrap(y + 1, ny) * nx + xa};
+    int off[4];  // the thread's cells from its first one
+#pragma unroll
+    for (int e = 0; e < 4; ++e) off[e] = wrap(col + e, nx) - xa;
     // first elements of planes q-1, q, q+1 of S(t); z: plane q+1
     struct At {
         int m, o, p, z;
@@ -158,7 +161,13 @@ __global__ void __launch_bounds__(kPpThreads, 1) k_plane_pipe(const float *__res
 #pragma unroll
         for (int v = 0; v < 6; ++v) {  // velocity v + 1: +x -x +y -y +z -z, before the +-x shift
             const int from = (v == 4 ? far.m : v == 5 ? far.p : far.o) + row_of[v == 2 ? 0 : v == 3 ? 2 : 1];
-            copy_async<16>(ring_at + to * kStage + v * kRow + t * 16, src + (v + 1) * pitch + from);
+            const unsigned at = ring_at + to * kStage + v * kRow + t * 16;
+            if constexpr (kRagged) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) copy_async<4>(at + 4 * e, src + (v + 1) * pitch + (from + off[e]));
+            } else {
+                copy_async<16>(at, src + (v + 1) * pitch + from);
+            }
         }
         next_plane(far);
     };
@@ -265,10 +274,17 @@ __global__ void __launch_bounds__(kPpThreads, 1) k_plane_pipe(const float *__res
         if constexpr (all) {
             const float2 *from[6] = {r.px, r.mx, r.py, r.my, r.pz, r.mz};
 #pragma unroll
-            for (int v = 0; v < 6; ++v)
-                if (live)
-                    *reinterpret_cast<float4 *>(dst + (v + 1) * pitch + to) =
-                        make_float4(from[v][0].x, from[v][1].x, from[v][0].y, from[v][1].y);
+            for (int v = 0; v < 6; ++v) {
+                float *at = dst + (v + 1) * pitch + to;
+                if constexpr (kRagged) {
+                    const float f[4] = {from[v][0].x, from[v][1].x, from[v][0].y, from[v][1].y};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (live && col + e < nx) at[e] = f[e];
+                } else if (live) {
+                    *reinterpret_cast<float4 *>(at) = make_float4(from[v][0].x, from[v][1].x, from[v][0].y, from[v][1].y);
+                }
+            }
         }
         free_slot = slot;
         if (++slot == kPpStages) slot = 0;

@@ -66,12 +66,14 @@ __device__ __forceinline__ void copy_wait() {
 // Memory side of the pipelines: fetch() starts the copy of a lane's four cells of a velocity into its
 // own slot of shared memory (kLane bytes at `to`; BFP16: and kLaneEx bytes at `to_ex`), take() reads
 // the slot and widens it, store() rounds and stores four cells, round() is what a stored and reloaded
-// value holds (not for BFP16).  `idx` is an element of one velocity
+// value holds (not for BFP16).  kRagged: for any nx, with the four cells copied and stored one by one (their
+// rows start at any element, and may wrap between them).  `idx` is an element of one velocity
 // array starting at `base` (BFP16: with its exponent bytes at `ex`).  kAlign: a strip's first column is
 // a multiple of it.
 struct RpF32 {
     using Elem = float;
     static constexpr int kAlign = 4, kLane = 16, kLaneEx = 0;
+    static constexpr bool kRagged = false;
     static __host__ __device__ const uint8_t *exps(const float *, long long) { return nullptr; }
     __device__ static __forceinline__ void fetch(unsigned to, unsigned, const float *__restrict__ base, const uint8_t *,
                                                  int idx) {
@@ -86,11 +88,17 @@ struct RpF32 {
     }
 };
 
+// FP32 at widths that are not multiples of 4.
+struct RpF32Ragged : RpF32 {
+    static constexpr bool kRagged = true;
+};
+
 // FP16 and BF16: S g / f*, rounded to nearest even.
 template <class T>
 struct Rp16 {
     using Elem = T;
     static constexpr int kAlign = 4, kLane = 8, kLaneEx = 0;
+    static constexpr bool kRagged = false;
     static __host__ __device__ const uint8_t *exps(const T *, long long) { return nullptr; }
     __device__ static __forceinline__ void fetch(unsigned to, unsigned, const T *__restrict__ base, const uint8_t *, int idx) {
         copy_async<8>(to, base + idx);
@@ -118,6 +126,7 @@ template <int Q>
 struct RpBfp {
     using Elem = Bfp16;
     static constexpr int kAlign = 8, kLane = 8, kLaneEx = 4;
+    static constexpr bool kRagged = false;
     static __host__ __device__ const uint8_t *exps(const Bfp16 *g, long long pitch) { return bfp_exps<Q>(g, pitch); }
     __device__ static __forceinline__ void fetch(unsigned to, unsigned to_ex, const Bfp16 *__restrict__ base,
                                                  const uint8_t *__restrict__ ex, int idx) {
@@ -189,6 +198,10 @@ __device__ __forceinline__ void rp_tile(const typename IO::Elem *__restrict__ sr
         v %= n;
         return v < 0 ? v + n : v;
     };
+    // the lane's cells from its first one
+    int off[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) off[e] = wrap(col + e, nx) - wrap(col, nx);
     // A row of S(t) and the lane's element in it: the next to fetch and the next to use
     struct At {
         int row, idx;
@@ -213,7 +226,12 @@ __device__ __forceinline__ void rp_tile(const typename IO::Elem *__restrict__ sr
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             const unsigned at = ring_at + to * kStage + v * kRow;
-            IO::fetch(at + lane * IO::kLane, at + 32 * IO::kLane + lane * IO::kLaneEx, in[v], in_ex[v], far.idx);
+            if constexpr (IO::kRagged) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) copy_async<4>(at + lane * IO::kLane + 4 * e, in[v] + (far.idx + off[e]));
+            } else {
+                IO::fetch(at + lane * IO::kLane, at + 32 * IO::kLane + lane * IO::kLaneEx, in[v], in_ex[v], far.idx);
+            }
         }
         next_row(far);
     };
@@ -308,8 +326,17 @@ __device__ __forceinline__ void rp_tile(const typename IO::Elem *__restrict__ sr
             const bool st = live && (p == 0 || k + 1 < rows);
             const float2 *from[4] = {r.px, r.mx, r.py, r.my};
 #pragma unroll
-            for (int v = 0; v < 4; ++v)
-                IO::store(out[v], out_ex[v], to, make_float4(from[v][0].x, from[v][1].x, from[v][0].y, from[v][1].y), st);
+            for (int v = 0; v < 4; ++v) {
+                const float4 q = make_float4(from[v][0].x, from[v][1].x, from[v][0].y, from[v][1].y);
+                if constexpr (IO::kRagged) {
+                    const float f[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (st && col + e < nx) out[v][to + e] = f[e];
+                } else {
+                    IO::store(out[v], out_ex[v], to, q, st);
+                }
+            }
             to += nx;
         });
     }

@@ -274,7 +274,7 @@ struct SetImpl {
     static cudaError_t with_steps(int k, Fn &&fn) {
         switch (k) {
         case 2:
-            if constexpr (std::is_same<IO, RpF32>::value) return fn(std::integral_constant<int, 2>{});
+            if constexpr (std::is_base_of<RpF32, IO>::value) return fn(std::integral_constant<int, 2>{});
             return cudaErrorInvalidValue;
         case 3: return fn(std::integral_constant<int, 3>{});
         case 4: return fn(std::integral_constant<int, 4>{});
@@ -285,7 +285,7 @@ struct SetImpl {
         }
     }
     template <class Fn>
-    static cudaError_t with_pipe(int storage, int k, Fn &&fn) {
+    static cudaError_t with_pipe(int storage, int nx, int k, Fn &&fn) {
         if constexpr (S::D != 2) {
             return cudaErrorInvalidValue;
         } else {
@@ -297,18 +297,18 @@ struct SetImpl {
             case LEE_STORE_BFP16: return go((RpBfp<S::Q> *)nullptr);
             case LEE_STORE_F16: return go((Rp16<__half> *)nullptr);
             case LEE_STORE_BF16: return go((Rp16<__nv_bfloat16> *)nullptr);
-            case LEE_STORE_F32: return go((RpF32 *)nullptr);
+            case LEE_STORE_F32: return nx % 4 == 0 ? go((RpF32 *)nullptr) : go((RpF32Ragged *)nullptr);
             default: return cudaErrorInvalidValue;
             }
         }
     }
-    static cudaError_t stepk_prepare(int k, int storage) {
-        return with_pipe(storage, k, [](auto *io, auto Kc) {
+    static cudaError_t stepk_prepare(int k, int storage, int nx) {
+        return with_pipe(storage, nx, k, [](auto *io, auto Kc) {
             return row_pipe_prepare<decltype(Kc)::value, std::remove_pointer_t<decltype(io)>>();
         });
     }
     static cudaError_t stepk(const StepLaunch &L, int k) {
-        return with_pipe(L.storage, k, [&](auto *io, auto Kc) {
+        return with_pipe(L.storage, L.nx, k, [&](auto *io, auto Kc) {
             return row_pipe_launch<decltype(Kc)::value, std::remove_pointer_t<decltype(io)>>(L);
         });
     }

@@ -133,7 +133,7 @@ cudaError_t row_pipe_prepare_stages() {
 template <int K, class IO, int kStages>
 cudaError_t row_pipe_launch_stages(const StepLaunch &L) {
     using E = typename IO::Elem;
-    if (L.open || L.nx % IO::kAlign != 0 || L.nx % 4 != 0) return cudaErrorInvalidValue;
+    if (L.open || (!IO::kRagged && L.nx % IO::kAlign != 0)) return cudaErrorInvalidValue;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -157,7 +157,7 @@ cudaError_t row_pipe_launch_stages(const StepLaunch &L) {
 }
 template <int K, class IO>
 cudaError_t row_pipe_prepare() {
-    if constexpr (std::is_same<IO, RpF32>::value) {
+    if constexpr (std::is_base_of<RpF32, IO>::value) {
         const cudaError_t e = row_pipe_prepare_stages<K, IO, kRpStagesNear>();
         return e != cudaSuccess ? e : row_pipe_prepare_stages<K, IO, kRpStagesFar>();
     } else {
@@ -166,7 +166,7 @@ cudaError_t row_pipe_prepare() {
 }
 template <int K, class IO>
 cudaError_t row_pipe_launch(const StepLaunch &L) {
-    if constexpr (std::is_same<IO, RpF32>::value) {
+    if constexpr (std::is_base_of<RpF32, IO>::value) {
         return 8LL * (long long)sizeof(float) * L.nx * L.ny <= kRpNearL2Bytes
                    ? row_pipe_launch_stages<K, IO, kRpStagesNear>(L)
                    : row_pipe_launch_stages<K, IO, kRpStagesFar>(L);
@@ -177,42 +177,51 @@ cudaError_t row_pipe_launch(const StepLaunch &L) {
 
 // Plane pipeline (planepipe.cuh): the resident blocks of a device, set by plane_pipe_prepare outside any
 // stream capture, and the launch.
-inline int *plane_pipe_capacity() {
+template <bool kRagged>
+int *plane_pipe_capacity() {
     static int cap[64] = {0};
     return cap;
 }
-inline cudaError_t plane_pipe_prepare() {
+template <bool kRagged>
+cudaError_t plane_pipe_prepare_for() {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (plane_pipe_capacity()[dev]) return cudaSuccess;
+    if (plane_pipe_capacity<kRagged>()[dev]) return cudaSuccess;
+    auto kern = k_plane_pipe<kPpDeep, kRagged>;
     constexpr int smem = pp_smem_bytes<kPpDeep>();
     int per_sm = 0, sms = 0;
-    e = cudaFuncSetAttribute(k_plane_pipe<kPpDeep>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_plane_pipe<kPpDeep>, kPpThreads, smem);
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPpThreads, smem);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    plane_pipe_capacity()[dev] = per_sm * sms > 0 ? per_sm * sms : 1;
+    plane_pipe_capacity<kRagged>()[dev] = per_sm * sms > 0 ? per_sm * sms : 1;
     return cudaSuccess;
 }
-inline cudaError_t plane_pipe_launch(const StepLaunch &L) {
-    if (L.storage != LEE_STORE_F32 || L.open || L.nx % 4 != 0) return cudaErrorInvalidValue;
+template <bool kRagged>
+cudaError_t plane_pipe_launch_for(const StepLaunch &L) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    const int capacity = plane_pipe_capacity()[dev];
+    const int capacity = plane_pipe_capacity<kRagged>()[dev];
     if (capacity == 0) return cudaErrorNotReady;  // prepare first
     const PpCut cut = plane_pipe_cut(kPpDeep, pp_halo<kPpDeep>(), L.nx, L.ny, L.nz, capacity);
     const long long gy = cut.C ? (L.ny + cut.height - 1) / cut.height : 0, gz = cut.C ? (L.nz + cut.HZ - 1) / cut.HZ : 0;
     if (cut.C == 0 || gy > 65535 || gz > 65535) return cudaErrorInvalidValue;
     const CollideCoef<float> cf = make_coef<float>(L.omega, L.coefM, L.coefN);
-    k_plane_pipe<kPpDeep><<<dim3((L.nx + cut.width - 1) / cut.width, (unsigned)gy, (unsigned)gz), kPpThreads,
-                            pp_smem_bytes<kPpDeep>(), L.stream>>>(static_cast<const float *>(L.src),
-                                                                  static_cast<float *>(L.dst), L.nx, L.ny, L.nz, L.pitch,
-                                                                  cut, cf.M[1][1]);
+    k_plane_pipe<kPpDeep, kRagged><<<dim3((L.nx + cut.width - 1) / cut.width, (unsigned)gy, (unsigned)gz), kPpThreads,
+                                     pp_smem_bytes<kPpDeep>(), L.stream>>>(
+        static_cast<const float *>(L.src), static_cast<float *>(L.dst), L.nx, L.ny, L.nz, L.pitch, cut, cf.M[1][1]);
     return cudaGetLastError();
+}
+inline cudaError_t plane_pipe_prepare(int nx) {
+    return nx % 4 == 0 ? plane_pipe_prepare_for<false>() : plane_pipe_prepare_for<true>();
+}
+inline cudaError_t plane_pipe_launch(const StepLaunch &L) {
+    if (L.storage != LEE_STORE_F32 || L.open) return cudaErrorInvalidValue;
+    return L.nx % 4 == 0 ? plane_pipe_launch_for<false>(L) : plane_pipe_launch_for<true>(L);
 }
 
 }  // namespace lee

@@ -10,7 +10,9 @@ pytestmark = pytest.mark.gpu
 # (grids of fewer cells take single steps) narrower than the halo, a row or a plane thin, long in each
 # direction, ragged tiles, strips and segments of several sizes
 SHAPES = [(4, 300, 700), (8, 1, 98400), (786436, 1, 1), (12, 65539, 1), (1600, 520, 1), (400, 3, 700), (132, 83, 75),
-          (100, 97, 91), (256, 72, 48)]
+          (100, 97, 91), (256, 72, 48),
+          # widths that are not multiples of 4
+          (1, 1600, 1400), (3, 911, 815), (49, 230, 191), (2097155, 1, 1), (193, 107, 110)]
 
 
 def _run(lee, monkeypatch, name, shape, storage, n, g0, single=False, **kw):

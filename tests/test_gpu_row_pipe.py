@@ -9,7 +9,9 @@ pytestmark = pytest.mark.gpu
 
 # narrower than a strip's halo, one strip less one chunk, one strip, one more chunk, several strips; rows
 # fewer than the levels, odd, and many segments
-SHAPES = [(4, 3, 1), (12, 5, 1), (108, 7, 1), (112, 16, 1), (116, 9, 1), (240, 4, 1), (260, 41, 1), (456, 1003, 1)]
+SHAPES = [(4, 3, 1), (12, 5, 1), (108, 7, 1), (112, 16, 1), (116, 9, 1), (240, 4, 1), (260, 41, 1), (456, 1003, 1),
+          # widths that are not multiples of 4
+          (1, 3, 1), (2, 5, 1), (3, 4, 1), (13, 9, 1), (113, 16, 1), (115, 7, 1), (222, 33, 1), (457, 1003, 1)]
 
 
 def _state(lee, monkeypatch, shape, storage, n, g0, single, name="D2Q5", **kw):
