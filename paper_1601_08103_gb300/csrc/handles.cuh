@@ -31,6 +31,9 @@ struct lee_lbm {
     cudaStream_t st = nullptr;
     long long steps = 0;
     double scale = 1.0;
+    // the collision's folded coefficients (fold_coefficients; set at create time: its long double arithmetic
+    // runs in software on Arm hosts and took about 10 us of every step call)
+    double omega = 0.0, coefM[4][4] = {}, coefN[4][4] = {};
     bool poisoned = false;
     std::string err;
     // learned boundary: entering populations [4][ghost_L] in the arithmetic type, and the

@@ -503,6 +503,9 @@ lee_status lee_lbm_create(const lee_lbm_config *cfg, lee_lbm **out) {
         h->pitch = ((long long)(h->nl + 2) * h->plane + 63) / 64 * 64;
     }
     h->st = static_cast<cudaStream_t>(cfg->cuda_stream);
+    h->omega = omega_for(cfg->storage, cfg->tau);
+    fold_coefficients(cfg->set, cfg->storage == LEE_STORE_F16 || cfg->storage == LEE_STORE_BF16, h->omega, h->coefM,
+                      h->coefN);
     if (const char *ev = std::getenv("LEE_TB_STEPS")) {
         if (ev[0] >= '1' && ev[0] <= '4' && ev[1] == 0) {
             h->tb_steps = ev[0] - '0';
@@ -633,9 +636,9 @@ lee_status lee_lbm_step(lee_lbm *h, int64_t n) {
     L.pitch = h->pitch;
     L.open = h->cfg.bc != LEE_BC_PERIODIC && h->cfg.bc != LEE_BC_SLAB;
     L.slab = h->slab ? 1 : 0;
-    L.omega = omega_for(h->cfg.storage, h->cfg.tau);
-    const bool is16 = h->cfg.storage == LEE_STORE_F16 || h->cfg.storage == LEE_STORE_BF16;
-    fold_coefficients(h->cfg.set, is16, L.omega, L.coefM, L.coefN);
+    L.omega = h->omega;
+    std::memcpy(L.coefM, h->coefM, sizeof(L.coefM));
+    std::memcpy(L.coefN, h->coefN, sizeof(L.coefN));
     L.sponge_w = sponge_active(h) ? h->cfg.sponge_width : 0;
     L.sponge_smax = h->cfg.sponge_strength;
     L.ghost = learned ? h->ghost : nullptr;
