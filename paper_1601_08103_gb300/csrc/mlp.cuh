@@ -64,9 +64,6 @@ __device__ __forceinline__ float bf16_hi(uint32_t v) { return __uint_as_float(v 
 __device__ __forceinline__ uint32_t ldw(const __nv_bfloat16 *p) { return *reinterpret_cast<const unsigned int *>(p); }
 
 __device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_grad(float z) {
-    return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * expf(-0.5f * z * z) * 0.39894228040143268f;
-}
 
 // Forward pass of one warp's 16 rows.  ax: A fragment of the input (BF16).  Outputs the two
 // rows' results in lanes with t == 0 (y_lo for row g, y_hi for row g + 8), plus, when the
