@@ -28,6 +28,7 @@ struct SetConsts {
     double scale;    // 16-bit storage scale S (1 otherwise)
     double eqA[2][4], eqB[2][4], eqC[2][4];
     double dec[4], enc[4], ew[4];
+    double te[2][4];  // energy weights of theta': kE ew ([1]: of stored 16-bit values, kE ew dec)
     double inv_rho0, kE, kR;
 };
 
@@ -121,6 +122,68 @@ __global__ void k_init_equilibrium(const double *__restrict__ rho, const double 
             g[(long long)i * pitch + x] = e;
             if (rest_static<S>() && i == 0) other[x] = e;
         });
+    }
+}
+
+// An estimate of the largest |g_i^eq / f*_i| of the initial fields in FP32, and the largest sum of the magnitudes
+// that a value was put together from: the estimate is off by less than kInitError times that (a dozen roundings
+// of 2^-24 of them).  The host needs the maximum's place between two powers of two only, so this decides it for
+// nearly all fields; k_init_maxabs, bound by the FP64 pipe, is left for those where it does not (and for fields
+// outside 1e-30 .. 1e30, where the estimate is infinite or small).  NaN is left out as there.  D2Q5, 8192^2 FP16: init_fields
+// 3.07 -> 1.91 ms.
+struct InitCoef {
+    float A[4], B[4], C[4];  // eqA[1], eqB[1], eqC[1] for a scale of 1
+};
+constexpr double kInitError = 1.0 / (1 << 20);
+template <class S>
+__global__ void k_init_estimate(const double *__restrict__ rho, const double *__restrict__ u,
+                                const double *__restrict__ theta, long long cells, InitCoef k,
+                                unsigned int *__restrict__ maxbits) {
+    float most = 0.f, sum = 0.f;
+    for (long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x; x < cells; x += (long long)gridDim.x * blockDim.x) {
+        const float r = to_f32(rho[x]), th = to_f32(theta[x]);
+        float v[3] = {0.f, 0.f, 0.f}, in = fmaxf(fabsf(r), fabsf(th));
+#pragma unroll
+        for (int a = 0; a < S::D; ++a) {
+            v[a] = fabsf(to_f32(u[(long long)a * cells + x]));
+            in = fmaxf(in, v[a]);
+        }
+        if (in > 1e30f) most = __int_as_float(0x7F800000);
+        static_for<4>([&](auto Sx) {
+            constexpr int s = decltype(Sx)::value;
+            if constexpr (shell_present<S>(s)) {
+                const float ar = k.A[s] * r, bt = k.B[s] * th;
+                float base = fabsf(ar + bt), parts = fabsf(ar) + fabsf(bt);
+                if constexpr (s > 0) {  // the largest |c_i . u'| of the shell: of its velocities without a negative component
+                    float cu = 0.f;
+                    bool first = true;
+                    static_for<S::Q>([&](auto I) {
+                        constexpr int i = decltype(I)::value;
+                        if constexpr (S::shell(i) == s && S::c(i, 0) >= 0 && S::c(i, 1) >= 0 && S::c(i, 2) >= 0) {
+                            float t = 0.f;
+                            static_for<3>([&](auto A) {
+                                if constexpr (S::c(i, decltype(A)::value) != 0) t += v[decltype(A)::value];
+                            });
+                            cu = first ? t : fmaxf(cu, t);
+                            first = false;
+                        }
+                    });
+                    base = fmaf(k.C[s], cu, base);
+                    parts = fmaf(k.C[s], cu, parts);
+                }
+                most = fmaxf(most, base);
+                sum = fmaxf(sum, parts);
+            }
+        });
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        most = fmaxf(most, __shfl_xor_sync(kFull, most, off));
+        sum = fmaxf(sum, __shfl_xor_sync(kFull, sum, off));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(maxbits, __float_as_uint(most));
+        atomicMax(maxbits + 1, __float_as_uint(sum));
     }
 }
 
@@ -302,11 +365,19 @@ __device__ __forceinline__ unsigned long long fix_square(unsigned bits, int shif
     const int s = 2 * shift;
     return (((unsigned long long)m * m) << kFixBitsSq) >> (s < 63 ? s : 63);
 }
-// v 2^e as FP64 (v rounded once, the exponent moved on the integer pipe).
+// v 2^e as FP64, v rounded once to nearest even: two dozen integer instructions, which cost less than the one
+// conversion of the FP64 pipe (2 against 128 lanes per clock).
 template <class I>
 __device__ __forceinline__ double fix_double(I v, int e) {
-    const double d = (double)v;
-    return v == 0 ? 0.0 : __hiloint2double(__double2hiint(d) + (e << 20), __double2loint(d));
+    bool minus = false;
+    if constexpr (std::is_signed<I>::value) minus = v < 0;
+    const unsigned long long u = minus ? 0ull - (unsigned long long)v : (unsigned long long)v;
+    const int n = __clzll((long long)u);
+    const unsigned long long m = u << (n & 63);  // the leading bit on top
+    unsigned long long q = m >> 11;
+    q += (((unsigned)m & 0x7FFu) + 0x3FFu + ((unsigned)q & 1u)) >> 11;  // (a carry out of 53 bits raises the exponent)
+    const int hi = (int)(q >> 32) + ((1023 + 63 - 1 - n + e) << 20);
+    return u == 0 ? 0.0 : __hiloint2double(minus ? hi | (int)0x80000000 : hi, (int)(unsigned)q);
 }
 template <class T>
 __host__ __device__ constexpr bool fixed_sums() {
@@ -314,8 +385,8 @@ __host__ __device__ constexpr bool fixed_sums() {
 }
 
 // Per-cell moments (Sec. 4 discrete moments, Sec. 5 temperature) in FP64.
-// D3Q7 384^3 FP32: 2.89 ms with FP64 sums and conversions, 1.26 ms with integer ones (0.57 at the copy rate);
-// D3Q19 256^3: 2.44 -> 0.46 ms.
+// D3Q7 384^3 FP32: 2.89 ms with FP64 sums and conversions, 0.92 ms with integer ones (0.57 at the copy rate);
+// D3Q19 256^3: 2.44 -> 0.43 ms.
 template <class S, class T>
 __global__ void k_moments(const T *__restrict__ g, long long cells, long long pitch, SetConsts k, double *__restrict__ rho,
                           double *__restrict__ u, double *__restrict__ theta) {
@@ -394,18 +465,15 @@ __global__ void k_moments(const T *__restrict__ g, long long cells, long long pi
                 }
             }
         }
-        double r = scaled ? -0.0 : total, e = -0.0, j[3] = {-0.0, -0.0, -0.0};
+        double r = scaled ? -0.0 : total, j[3] = {-0.0, -0.0, -0.0};
         static_for<4>([&](auto Sx) {
             constexpr int s = decltype(Sx)::value;
-            if constexpr (shell_present<S>(s)) {
+            if constexpr (shell_present<S>(s) && scaled) {
                 constexpr int kk = shell_slot<S>(s);
-                if constexpr (scaled) r = fma(P[kk], k.dec[s], r);
-                if constexpr (s > 0) {  // (the rest shell has no energy and no momentum)
-                    e = fma(k.ew[s], scaled ? P[kk] * k.dec[s] : P[kk], e);
-                    if constexpr (scaled) {
+                r = fma(P[kk], k.dec[s], r);
+                if constexpr (s > 0) {  // (the rest shell has no momentum)
 #pragma unroll
-                        for (int a = 0; a < D; ++a) j[a] = fma(J[kk][a], k.dec[s], j[a]);
-                    }
+                    for (int a = 0; a < D; ++a) j[a] = fma(J[kk][a], k.dec[s], j[a]);
                 }
             }
         });
@@ -417,7 +485,14 @@ __global__ void k_moments(const T *__restrict__ g, long long cells, long long pi
                 u[(long long)a * cells + x] = k.inv_rho0 == 1.0 ? ja : ja * k.inv_rho0;
             }
         }
-        if (theta) theta[x] = fma(k.kE, e, -k.kR * r);
+        if (theta) {
+            double th = -k.kR * r;
+            static_for<4>([&](auto Sx) {  // (the rest shell has no energy)
+                constexpr int s = decltype(Sx)::value;
+                if constexpr (s > 0 && shell_present<S>(s)) th = fma(k.te[scaled ? 1 : 0][s], P[shell_slot<S>(s)], th);
+            });
+            theta[x] = th;
+        }
     }
 }
 

@@ -532,7 +532,7 @@ lee_status lee_lbm_create(const lee_lbm_config *cfg, lee_lbm **out) {
     h->nblocks = reduce_blocks(cells);
     if (e == cudaSuccess) e = cudaMalloc(&h->partial, sizeof(double) * kReduceMax * (size_t)h->nblocks);
     if (e == cudaSuccess) e = cudaMalloc(&h->red_out, sizeof(double) * kReduceMax);
-    if (e == cudaSuccess) e = cudaMalloc(&h->maxbits, sizeof(unsigned int));
+    if (e == cudaSuccess) e = cudaMalloc(&h->maxbits, 2 * sizeof(unsigned int));
     for (int k = 0; k < 4 && h->slab && e == cudaSuccess; ++k)
         e = cudaMalloc(&h->halo[k], h->elem * (size_t)h->crossing * (size_t)h->plane);
     if (e == cudaSuccess && cfg->bc == LEE_BC_OPEN_LEARNED) {
@@ -594,20 +594,24 @@ lee_status lee_lbm_init_fields(lee_lbm *h, const double *rho, const double *u, c
         dt = ft;
     }
     if (scaled_storage(h->cfg.storage) && h->cfg.store_scale == 0.0) {
-        LEE_CK(h, cudaMemsetAsync(h->maxbits, 0, sizeof(unsigned int), h->st), "memset maxbits");
-        LEE_CK(h, h->ops->init_maxabs(dr, du, dt, h->cells, consts_for(h->cfg.set, 1.0), h->maxbits, h->st), "init_maxabs");
-        unsigned int bits = 0;
-        LEE_CK(h, cudaMemcpyAsync(&bits, h->maxbits, sizeof(bits), cudaMemcpyDeviceToHost, h->st), "D2H maxbits");
+        // largest power of two with S * m <= 1024
+        auto scale_for = [](double m) { return std::ldexp(1.0, (int)std::floor(std::log2(1024.0 / m))); };
+        const SetConsts one = consts_for(h->cfg.set, 1.0);
+        float m[2];
+        LEE_CK(h, cudaMemsetAsync(h->maxbits, 0, 2 * sizeof(unsigned int), h->st), "memset maxbits");
+        LEE_CK(h, h->ops->init_estimate(dr, du, dt, h->cells, one, h->maxbits, h->st), "init_estimate");
+        LEE_CK(h, cudaMemcpyAsync(m, h->maxbits, 2 * sizeof(float), cudaMemcpyDeviceToHost, h->st), "D2H maxbits");
         LEE_SYNC(h);
-        float m;
-        std::memcpy(&m, &bits, sizeof(m));
-        double S = 1.0;
-        if (m > 0.0f && std::isfinite(m)) {
-            // largest power of two with S * m <= 1024
-            int ex = (int)std::floor(std::log2(1024.0 / (double)m));
-            S = std::ldexp(1.0, ex);
+        const double off = kInitError * m[1], least = m[0] - off, most = m[0] + off;
+        if (std::isfinite(most) && least > 1e-30 && scale_for(least) == scale_for(most)) {
+            h->scale = scale_for(most);
+        } else {
+            LEE_CK(h, cudaMemsetAsync(h->maxbits, 0, sizeof(unsigned int), h->st), "memset maxbits");
+            LEE_CK(h, h->ops->init_maxabs(dr, du, dt, h->cells, one, h->maxbits, h->st), "init_maxabs");
+            LEE_CK(h, cudaMemcpyAsync(m, h->maxbits, sizeof(float), cudaMemcpyDeviceToHost, h->st), "D2H maxbits");
+            LEE_SYNC(h);
+            h->scale = m[0] > 0.0f && std::isfinite(m[0]) ? scale_for(m[0]) : 1.0;
         }
-        h->scale = S;
     }
     const SetConsts k = consts_for(h->cfg.set, h->scale);
     LEE_CK(h, h->ops->init(h->cfg.storage, dr, du, dt, state(h, 0), state(h, 1), h->cells, h->pitch, k, h->st), "init kernel");

@@ -73,7 +73,10 @@ struct SetOps {
     // those alone (rest_static)
     cudaError_t (*init)(int storage, const double *rho, const double *u, const double *theta, void *g, void *other,
                         long long cells, long long pitch, const SetConsts &k, cudaStream_t st);
-    // max |g^eq / f*| of the fields into *maxbits (float bits; caller zeroes it)
+    // an FP32 estimate of max |g^eq / f*| of the fields into maxbits[0] and the base of its error bound into
+    // maxbits[1] (k_init_estimate), and that maximum itself into *maxbits (float bits; caller zeroes them)
+    cudaError_t (*init_estimate)(const double *rho, const double *u, const double *theta, long long cells,
+                                 const SetConsts &k, unsigned int *maxbits, cudaStream_t st);
     cudaError_t (*init_maxabs)(const double *rho, const double *u, const double *theta, long long cells, const SetConsts &k,
                                unsigned int *maxbits, cudaStream_t st);
     cudaError_t (*moments)(int storage, const void *g, long long cells, long long pitch, const SetConsts &k, double *rho,
@@ -176,6 +179,10 @@ SetConsts host_consts(double scale) {
     k.inv_rho0 = 1.0 / k.rho0;
     k.kE = (k.gamma - 1.0) / k.rho0;
     k.kR = k.theta0 / k.rho0;
+    for (int s = 0; s < 4; ++s) {
+        k.te[0][s] = k.kE * k.ew[s];
+        k.te[1][s] = k.te[0][s] * k.dec[s];
+    }
     return k;
 }
 

@@ -94,6 +94,17 @@ struct SetImpl {
             return cudaGetLastError();
         });
     }
+    static cudaError_t init_estimate(const double *rho, const double *u, const double *theta, long long cells,
+                                     const SetConsts &k, unsigned int *maxbits, cudaStream_t st) {
+        InitCoef c;
+        for (int s = 0; s < 4; ++s) {
+            c.A[s] = (float)k.eqA[1][s];
+            c.B[s] = (float)k.eqB[1][s];
+            c.C[s] = (float)k.eqC[1][s];
+        }
+        k_init_estimate<S><<<aux_blocks(cells), 256, 0, st>>>(rho, u, theta, cells, c, maxbits);
+        return cudaGetLastError();
+    }
     static cudaError_t init_maxabs(const double *rho, const double *u, const double *theta, long long cells,
                                    const SetConsts &k, unsigned int *maxbits, cudaStream_t st) {
         k_init_maxabs<S><<<aux_blocks(cells), 256, 0, st>>>(rho, u, theta, cells, k, maxbits);
@@ -368,6 +379,7 @@ struct SetImpl {
         o.Q = S::Q;
         o.step = &step;
         o.init = &init;
+        o.init_estimate = &init_estimate;
         o.init_maxabs = &init_maxabs;
         o.moments = &moments;
         o.reduce_partial = &reduce_partial;
