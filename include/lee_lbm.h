@@ -196,6 +196,9 @@ lee_status lee_lbm_init_fields(lee_lbm *h, const double *rho, const double *u, c
  *  - periodic 3D FP32 grids of D3Q7 and diatomic D3Q7 advance four steps per launch (a pipeline of the
  *    planes), then, with nx a multiple of 4, two (a z-marching tile), then one; grids of fewer than
  *    786432 cells (2097152 where nx is not a multiple of 4), where that is slower, take single steps (LEE_TB_STEPS=1 or 2 fixes the count);
+ *  - periodic 3D FP32 grids of D3Q9, D3Q13 and D3Q19 advance two steps per launch where their copies are well beyond L2
+ *    (from 883011 cells of D3Q19, 1290555 of D3Q13, 3728270 of D3Q9) and the grid fills the launch's tiles of 60 x 14
+ *    cells (lee_lbm_steps_per_launch reports 1; not with LEE_TB_STEPS or LEE_SINGLE_STEP);
  *  - BFP16 storage on those periodic 2D grids with nx a multiple of 8 uses the same kernels (four steps
  *    per launch, the rest as single steps; or three with LEE_TB_STEPS=3), but keeps the
  *    intermediate states in FP32 and encodes only the last one: a launch of k steps equals decoding

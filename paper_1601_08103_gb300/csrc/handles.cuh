@@ -34,6 +34,7 @@ struct lee_lbm {
     // the collision's folded coefficients (fold_coefficients; set at create time: its long double arithmetic
     // runs in software on Arm hosts and took about 10 us of every step call)
     double omega = 0.0, coefM[4][4] = {}, coefN[4][4] = {};
+    int cut3d[4] = {};  // 3D: how a launch of several steps cuts the grid (SetOps::step3dk_prepare)
     bool poisoned = false;
     std::string err;
     // learned boundary: entering populations [4][ghost_L] in the arithmetic type, and the

@@ -202,7 +202,16 @@ bool plane_pipe(const lee_lbm *h) {
            !h->tb_env && !tma_tile(h) && plane_pipe_eligible(h->cfg.ny);
 }
 
-constexpr long long kFuse3dCells = 3LL << 18, kFuse3dRaggedCells = 1LL << 21;
+constexpr long long kFuse3dCells = 3LL << 18, kFuse3dRaggedCells = 1LL << 21, kPairBytes = 128LL << 20;
+
+// Cells from which a 3D grid on the plane pipelines takes several steps per launch.  For the two steps of the sets
+// with diagonal velocities: both copies well beyond L2, in which single steps run otherwise (us per step of one
+// / two steps per launch: D3Q19 64^3 5.9 / 9.4, 96^3 22.6 / 18.5, 128^3 52.3 / 44.2; D3Q13 96^3 9.9 / 10.8, 128^3 32.3 / 25.1; D3Q9
+// 128^3 17.9 / 19.2, 256^3 153 / 116).
+long long fuse_3d_cells(const lee_lbm *h) {
+    if (h->ops->deep3d == 2) return (h->Q > 9 ? kPairBytes : 2 * kPairBytes) / (2 * h->Q * (long long)sizeof(float));
+    return h->cfg.nx % 4 == 0 ? kFuse3dCells : kFuse3dRaggedCells;
+}
 
 // Whether this is a 2D FP32 grid for the row pipeline's form for widths that are not multiples of 4
 // (steps_per_launch is 1 there; the bits are those of single steps).
@@ -228,9 +237,9 @@ int next_launch(const lee_lbm *h, int unit, long long left) {
         if (left >= kRpDeep && h->cfg.storage != LEE_STORE_BFP16) return kRpDeep;
         if (left < unit && left > 1 && h->cfg.storage == LEE_STORE_F32) return (int)left;
     }
-    if (h->D == 3 && plane_pipe(h)) {
-        if (h->cells < (h->cfg.nx % 4 == 0 ? kFuse3dCells : kFuse3dRaggedCells)) return 1;
-        if (left >= kPpDeep) return kPpDeep;
+    if (h->D == 3 && plane_pipe(h) && h->cut3d[3] > 0) {
+        if (h->cells < fuse_3d_cells(h)) return 1;
+        if (left >= h->ops->deep3d) return h->ops->deep3d;
     }
     return left >= unit ? unit : 1;
 }
@@ -547,7 +556,7 @@ lee_status lee_lbm_create(const lee_lbm_config *cfg, lee_lbm **out) {
             if (e == cudaSuccess && k > 0 && (h->tb_env ? k == h->tb_steps : k != 2 || cfg->storage == LEE_STORE_F32))
                 e = o->stepk_prepare(k, cfg->storage, (int)cfg->nx);
     }
-    if (e == cudaSuccess && plane_pipe(h)) e = o->step3dk_prepare((int)cfg->nx);
+    if (e == cudaSuccess && plane_pipe(h)) e = o->step3dk_prepare((int)cfg->nx, (int)cfg->ny, (int)cfg->nz, h->cut3d);
     if (e == cudaSuccess && h->tb_steps >= 2 && tiled_3d(h)) e = o->step3d2_prepare(cfg->storage, tma_tile(h) ? 1 : 0);
     if (e == cudaSuccess && tma_tile(h)) {
         e = cudaHostAlloc(reinterpret_cast<void **>(&h->wait_host), sizeof(unsigned), cudaHostAllocMapped);
@@ -651,6 +660,7 @@ lee_status lee_lbm_step(lee_lbm *h, int64_t n) {
     L.bfp_cells = h->bfp_cells;
     L.store_scale = h->scale;
     L.t3_tma = tma_tile(h) ? 1 : 0;
+    std::memcpy(L.cut3d, h->cut3d, sizeof(L.cut3d));
     L.wait_flag = h->wait_dev;
     L.wait_ns = g_stage_wait_ns.load(std::memory_order_relaxed);
     L.t3_inject = g_inject_stage.load(std::memory_order_relaxed);
@@ -716,7 +726,7 @@ lee_status lee_lbm_step(lee_lbm *h, int64_t n) {
         L.src = h->buf[from];
         L.dst = h->buf[from ^ 1];
         L.stream = st;
-        if (h->D == 3) return k == kPpDeep ? h->ops->step3dk(L) : h->ops->step3d2(L);
+        if (h->D == 3) return k == h->ops->deep3d ? h->ops->step3dk(L) : h->ops->step3d2(L);
         return h->ops->stepk(L, k);
     };
     auto launches_of = [&](int64_t steps) {

@@ -46,6 +46,7 @@ struct StepLaunch {
     unsigned *wait_flag;
     long long wait_ns;
     int t3_inject;
+    int cut3d[4];  // 3D: the cut of the grid for step3dk (all 0: none made)
     cudaStream_t stream;
 };
 
@@ -64,10 +65,11 @@ struct SetOps {
     // and kernel (tma = 1: the TMA-fed tile, which also needs t3t_eligible grids)
     cudaError_t (*step3d2)(const StepLaunch &);
     cudaError_t (*step3d2_prepare)(int storage, int tma);
-    // kPpDeep fused steps per launch for the same sets (FP32, plane_pipe_eligible grids), and its one-time
-    // set-up for a width
+    // deep3d fused steps per launch of the 3D sets (FP32, plane_pipe_eligible grids; kPpDeep for the axis sets,
+    // 2 for the others), and the set-up of a grid for it (its cut goes into StepLaunch::cut3d)
+    int deep3d;
     cudaError_t (*step3dk)(const StepLaunch &);
-    cudaError_t (*step3dk_prepare)(int nx);
+    cudaError_t (*step3dk_prepare)(int nx, int ny, int nz, int (&cut)[4]);
     // g = g^eq(fields) (fields FP64 on device).  init, import_f64 and sponge_damp write a whole state
     // copy g; `other` is the other copy, whose rest populations they write too where a step leaves
     // those alone (rest_static)

@@ -395,8 +395,15 @@ struct SetImpl {
         o.stepk_prepare = S::D == 2 ? &stepk_prepare : nullptr;
         o.step3d2 = axis_only<S>() ? &step3d2 : nullptr;
         o.step3d2_prepare = axis_only<S>() ? &step3d2_prepare : nullptr;
-        o.step3dk = axis_only<S>() ? &plane_pipe_launch : nullptr;
-        o.step3dk_prepare = axis_only<S>() ? &plane_pipe_prepare : nullptr;
+        if constexpr (axis_only<S>()) {
+            o.step3dk = &plane_pipe_launch;
+            o.step3dk_prepare = &plane_pipe_prepare;
+            o.deep3d = kPpDeep;
+        } else if constexpr (S::D == 3) {
+            o.step3dk = &plane_pair_launch<S>;
+            o.step3dk_prepare = &plane_pair_prepare<S>;
+            o.deep3d = 2;
+        }
         o.edge_fixup = S::D == 2 ? &edge_fixup : nullptr;
         for (int i = 0; i < S::Q; ++i) {
             for (int a = 0; a < 3; ++a) o.c[i][a] = S::c(i, a);

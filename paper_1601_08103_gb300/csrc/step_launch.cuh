@@ -5,6 +5,7 @@
 #pragma once
 
 #include "ops.cuh"
+#include "planepair.cuh"
 #include "planepipe.cuh"
 #include "rowpipe.cuh"
 
@@ -175,39 +176,48 @@ cudaError_t row_pipe_launch(const StepLaunch &L) {
     }
 }
 
-// Plane pipeline (planepipe.cuh): the resident blocks of a device, set by plane_pipe_prepare outside any
-// stream capture, and the launch.
+// Plane pipeline (planepipe.cuh): its cut of a grid, made once by plane_pipe_prepare (the search takes tens of
+// microseconds), and the launch.
 template <bool kRagged>
 int *plane_pipe_capacity() {
     static int cap[64] = {0};
     return cap;
 }
-template <bool kRagged>
-cudaError_t plane_pipe_prepare_for() {
+// The resident blocks of `kern` on the current device, kept in cap[device] and asked for outside any stream
+// capture.
+template <class Kern>
+cudaError_t resident_blocks(Kern kern, int threads, int smem, int *cap, int &blocks) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (plane_pipe_capacity<kRagged>()[dev]) return cudaSuccess;
-    auto kern = k_plane_pipe<kPpDeep, kRagged>;
-    constexpr int smem = pp_smem_bytes<kPpDeep>();
-    int per_sm = 0, sms = 0;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPpThreads, smem);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (cap[dev] == 0) {
+        int per_sm = 0, sms = 0;
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+        cap[dev] = per_sm * sms > 0 ? per_sm * sms : 1;
+    }
+    blocks = cap[dev];
+    return cudaSuccess;
+}
+template <bool kRagged>
+cudaError_t plane_pipe_prepare_for(int nx, int ny, int nz, int (&cut)[4]) {
+    int blocks = 0;
+    const cudaError_t e = resident_blocks(k_plane_pipe<kPpDeep, kRagged>, kPpThreads, pp_smem_bytes<kPpDeep>(),
+                                          plane_pipe_capacity<kRagged>(), blocks);
     if (e != cudaSuccess) return e;
-    plane_pipe_capacity<kRagged>()[dev] = per_sm * sms > 0 ? per_sm * sms : 1;
+    const PpCut c = plane_pipe_cut(kPpDeep, pp_halo<kPpDeep>(), nx, ny, nz, blocks);
+    cut[0] = c.C;
+    cut[1] = c.width;
+    cut[2] = c.height;
+    cut[3] = c.HZ;
     return cudaSuccess;
 }
 template <bool kRagged>
 cudaError_t plane_pipe_launch_for(const StepLaunch &L) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    const int capacity = plane_pipe_capacity<kRagged>()[dev];
-    if (capacity == 0) return cudaErrorNotReady;  // prepare first
-    const PpCut cut = plane_pipe_cut(kPpDeep, pp_halo<kPpDeep>(), L.nx, L.ny, L.nz, capacity);
+    const PpCut cut{L.cut3d[0], L.cut3d[1], L.cut3d[2], L.cut3d[3]};
     const long long gy = cut.C ? (L.ny + cut.height - 1) / cut.height : 0, gz = cut.C ? (L.nz + cut.HZ - 1) / cut.HZ : 0;
     if (cut.C == 0 || gy > 65535 || gz > 65535) return cudaErrorInvalidValue;
     const CollideCoef<float> cf = make_coef<float>(L.omega, L.coefM, L.coefN);
@@ -216,12 +226,47 @@ cudaError_t plane_pipe_launch_for(const StepLaunch &L) {
         static_cast<const float *>(L.src), static_cast<float *>(L.dst), L.nx, L.ny, L.nz, L.pitch, cut, cf.M[1][1]);
     return cudaGetLastError();
 }
-inline cudaError_t plane_pipe_prepare(int nx) {
-    return nx % 4 == 0 ? plane_pipe_prepare_for<false>() : plane_pipe_prepare_for<true>();
+inline cudaError_t plane_pipe_prepare(int nx, int ny, int nz, int (&cut)[4]) {
+    return nx % 4 == 0 ? plane_pipe_prepare_for<false>(nx, ny, nz, cut) : plane_pipe_prepare_for<true>(nx, ny, nz, cut);
 }
 inline cudaError_t plane_pipe_launch(const StepLaunch &L) {
     if (L.storage != LEE_STORE_F32 || L.open) return cudaErrorInvalidValue;
     return L.nx % 4 == 0 ? plane_pipe_launch_for<false>(L) : plane_pipe_launch_for<true>(L);
+}
+
+// Two steps per launch of the sets with diagonal velocities (planepair.cuh), likewise.
+template <class S, bool kRagged>
+int *plane_pair_capacity() {
+    static int cap[64] = {0};
+    return cap;
+}
+template <class S, bool kRagged>
+cudaError_t plane_pair_prepare_for(int nx, int ny, int nz, int (&cut)[4]) {
+    int blocks = 0;
+    const cudaError_t e = resident_blocks(k_plane_pair<S, kRagged>, kPairThreads, pair_smem_bytes<S>(),
+                                          plane_pair_capacity<S, kRagged>(), blocks);
+    if (e == cudaSuccess) cut[3] = plane_pair_segment(nx, ny, nz, blocks);
+    return e;
+}
+template <class S, bool kRagged>
+cudaError_t plane_pair_launch_for(const StepLaunch &L) {
+    const int HZ = L.cut3d[3];
+    const long long gy = (L.ny + kPairHeight - 1) / kPairHeight;
+    if (HZ == 0 || gy > 65535) return cudaErrorInvalidValue;
+    k_plane_pair<S, kRagged><<<dim3((L.nx + kPairWidth - 1) / kPairWidth, (unsigned)gy, (L.nz + HZ - 1) / HZ),
+                               kPairThreads, pair_smem_bytes<S>(), L.stream>>>(
+        static_cast<const float *>(L.src), static_cast<float *>(L.dst), L.nx, L.ny, L.nz, L.pitch, HZ,
+        make_coef<float>(L.omega, L.coefM, L.coefN));
+    return cudaGetLastError();
+}
+template <class S>
+cudaError_t plane_pair_prepare(int nx, int ny, int nz, int (&cut)[4]) {
+    return nx % 2 == 0 ? plane_pair_prepare_for<S, false>(nx, ny, nz, cut) : plane_pair_prepare_for<S, true>(nx, ny, nz, cut);
+}
+template <class S>
+cudaError_t plane_pair_launch(const StepLaunch &L) {
+    if (L.storage != LEE_STORE_F32 || L.open) return cudaErrorInvalidValue;
+    return L.nx % 2 == 0 ? plane_pair_launch_for<S, false>(L) : plane_pair_launch_for<S, true>(L);
 }
 
 }  // namespace lee
