@@ -343,23 +343,28 @@ __device__ __forceinline__ bool shell_sums(const T *__restrict__ g, long long pi
 }
 
 // Exact sums of values that are FP32 numbers (every storage but FP64) on the integer pipe.  With E the
-// largest biased exponent among them, a value is its 24-bit mantissa, shifted left by kFixBits and right by
-// its own distance from E: a 64-bit integer in units of 2^(E - 150 - kFixBits).  Nothing is lost down to
+// largest biased exponent among them, a value is its 24-bit mantissa, shifted left by kFixBits (a reduction:
+// kFixBitsSum) and right by its own distance from E: a 64-bit integer in units of 2^(E - 150 - kFixBits).  Nothing is lost down to
 // 2^-34 of the largest value and no more than 2^-58 of it below, which is finer than FP64 sums of them;
 // the sums are rounded to FP64 once.  Zeros and denormals (E of their own 0) shift out to nothing where E is
 // kFixLeast or more; smaller values, infinities and NaN take FP64 sums.
 constexpr int kFixBits = 34, kFixBitsSq = 10;
 constexpr unsigned kFixLeast = 64;
+// Whether the sums of n values stay inside their 64 bits: a value is below 2^(24 + bits) in magnitude and the signed
+// sum below 2^63 (31 values with 34 bits, 63 with 33), a square below 2^(48 + kFixBitsSq) and the unsigned sum below 2^64.
+__host__ __device__ constexpr bool fix_fits(int n, int bits) { return n < 1 << (63 - 24 - bits); }
+__host__ __device__ constexpr bool fix_fits_sq(int n) { return n < 1 << (64 - 48 - kFixBitsSq); }
 __device__ __forceinline__ int fix_shift(unsigned bits, unsigned E) {
     const int s = (int)(E - ((bits >> 23) & 0xFFu));
     return s < 63 ? s : 63;
 }
+template <int kBits = kFixBits>
 __device__ __forceinline__ long long fix_value(unsigned bits, int shift) {
-    const long long m = (long long)(((unsigned long long)((bits & 0x7FFFFFu) | 0x800000u) << kFixBits) >> shift);
+    const long long m = (long long)(((unsigned long long)((bits & 0x7FFFFFu) | 0x800000u) << kBits) >> shift);
     const long long sign = (int)bits >> 31;
     return (m ^ sign) - sign;
 }
-// Its square, in units of 2^(2 (E - 150) - kFixBitsSq); 63 of them fit in 64 bits.
+// Its square, in units of 2^(2 (E - 150) - kFixBitsSq).
 __device__ __forceinline__ unsigned long long fix_square(unsigned bits, int shift) {
     const unsigned m = (bits & 0x7FFFFFu) | 0x800000u;
     const int s = 2 * shift;
@@ -392,6 +397,7 @@ __global__ void k_moments(const T *__restrict__ g, long long cells, long long pi
                           double *__restrict__ u, double *__restrict__ theta) {
     constexpr bool scaled = Store<T>::scaled;
     constexpr int NS = n_shells<S>(), D = S::D;
+    static_assert(fix_fits(S::Q, kFixBits), "signed sums of a cell");
     for (long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x; x < cells; x += (long long)gridDim.x * blockDim.x) {
         // shell sums; where the storage is not scaled their total and the momentum over all shells, else the
         // momentum of each
@@ -555,13 +561,26 @@ __device__ __forceinline__ void reduce_cell(const double *__restrict__ g, long l
 // of a thread's group are added as integers and reach the FP64 accumulators as one value per sum
 // (D3Q7 384^3 FP32: 4.32 ms with FP64 sums of every value, 0.70 ms so, 0.24 at the copy rate; D3Q19 256^3 3.81 ->
 // 0.70 ms).
-constexpr int kReduceGroup = 4;
+// The group of a shell of 12 velocities (D3Q13, D3Q19) has 48 values of one sign and size in an ordinary field, 2^5.6 of
+// them: one bit less than the moments' sums.
+constexpr int kReduceGroup = 4, kFixBitsSum = kFixBits - 1;
+template <class S>
+__host__ __device__ constexpr int most_in_shell() {
+    int most = 0;
+    for (int s = 0; s < 4; ++s) {
+        int n = 0;
+        for (int i = 0; i < S::Q; ++i) n += S::shell(i) == s ? 1 : 0;
+        most = n > most ? n : most;
+    }
+    return most;
+}
 template <class S, class T>
 __global__ void __launch_bounds__(kReduceThreads) k_reduce_partial(const T *__restrict__ g, long long cells, long long pitch,
                                                                    double *__restrict__ partial) {
     constexpr int NS = n_shells<S>(), D = S::D, NR = reduce_nraw<S>(), G = kReduceGroup;
     static_assert(NR <= kReduceMax, "raw accumulators do not fit");
-    static_assert(G * 12 <= 63, "integer sums of a shell of up to 12 velocities");
+    static_assert(fix_fits(G * most_in_shell<S>(), kFixBitsSum), "signed sums of a group's shell");
+    static_assert(fix_fits_sq(G * most_in_shell<S>()), "sums of squares of a group's shell");
     double acc[NR];
 #pragma unroll
     for (int v = 0; v < NR; ++v) acc[v] = 0.0;
@@ -604,7 +623,7 @@ __global__ void __launch_bounds__(kReduceThreads) k_reduce_partial(const T *__re
                         constexpr int i = decltype(I)::value;
                         constexpr int s = shell_slot<S>(S::shell(i));
                         const int shift = fix_shift(b[c][i], E);
-                        const long long v = fix_value(b[c][i], shift);
+                        const long long v = fix_value<kFixBitsSum>(b[c][i], shift);
                         p[s] += v;
                         q[s] += fix_square(b[c][i], shift);
                         static_for<D>([&](auto A) {
@@ -617,11 +636,11 @@ __global__ void __launch_bounds__(kReduceThreads) k_reduce_partial(const T *__re
                 const int e = (int)E - 150;
                 static_for<NS>([&](auto Kx) {
                     constexpr int k = decltype(Kx)::value;
-                    acc[k] += fix_double(p[k], e - kFixBits);
+                    acc[k] += fix_double(p[k], e - kFixBitsSum);
                     acc[NS + k] += fix_double(q[k], 2 * e - kFixBitsSq);
                     if constexpr (k > 0) {
 #pragma unroll
-                        for (int a = 0; a < D; ++a) acc[2 * NS + k * D + a] += fix_double(j[k][a], e - kFixBits);
+                        for (int a = 0; a < D; ++a) acc[2 * NS + k * D + a] += fix_double(j[k][a], e - kFixBitsSum);
                     }
                 });
                 continue;
