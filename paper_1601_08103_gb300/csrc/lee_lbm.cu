@@ -226,11 +226,11 @@ bool ragged_2d(const lee_lbm *h) {
 // or three that remain in one launch too (a 16-bit state would be rounded at other steps); 3D grids on the
 // plane pipeline take kPpDeep.  3D FP32 grids of fewer than kFuse3dCells cells take single steps: their few
 // tiles leave SMs idle in either fused kernel (us per step of one / two / four steps per launch: 64^3 2.5 /
-// 3.7 / 2.9, 80^3 3.7 / 4.8 / 3.8, 96^3 4.8 / 5.9 / 4.5, 128^3 - / 10.2 / 7.9; widths that are not multiples of 4,
+// 3.7 / 2.9, 80^3 3.7 / 4.8 / 3.8, 96^3 4.8 / 5.9 / 4.1, 128^3 - / 10.2 / 7.2; widths that are not multiples of 4,
 // copied word by word, 97x99x98 8.2 / - / 8.4, 193x161x135 33.7 / - / 27.1).
 // 2D FP32 at such widths: 2047x2045 160 GLUPS with single steps, 920 on the row pipeline.
 // Measured on GB300, GLUPS: D2Q5 FP32 2048^2 / 8192^2 four steps per launch 740 / 811, eight 1490 / 1611; D3Q7
-// FP32 384^3 / 256^3 two 259 / 232, four 373 / 334.
+// FP32 384^3 / 256^3 two 259 / 232, four 426 / 373.
 int next_launch(const lee_lbm *h, int unit, long long left) {
     if (ragged_2d(h)) return left >= kRpDeep ? kRpDeep : left >= 4 ? 4 : (int)left;
     if (unit > 1 && h->D == 2 && !h->tb_env) {

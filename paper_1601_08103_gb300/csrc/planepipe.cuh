@@ -10,8 +10,9 @@
 // the neighbouring lane, at a warp's ends through a word of shared memory; +-y come through shared memory.
 // Words and rows in shared memory have two slots that alternate with the iterations.  Whatever crosses
 // threads was made one iteration earlier, so one barrier per iteration orders all levels, and the reads
-// of all levels can go out together.  S(t) reaches the threads through cp.async into slots of their own,
-// kPpStages - 1 planes ahead.
+// of all levels can go out together.  S(t) reaches the threads through cp.async into a ring of slots,
+// kPpStages - 1 planes ahead.  A warp's end lanes read their neighbours' slots too, so a slot is refilled only
+// after the barrier that follows its reads.
 //
 // Level l is right on all but the tile's l-1 outermost rows and l outermost columns: pp_halo columns
 // and K-1 rows on either side are computed and not stored, and a segment of planes costs 2 (K-1) iterations
@@ -22,10 +23,11 @@
 // launch gives the bits of K single steps.  (16-bit storage stays on the one-step kernel in 3D: it is
 // rounded after every step there, whatever the calls.)
 //
-// What bounds it: K = 4 moves 12 bytes of DRAM per FP32 update, 0.68 of the measured copy on D3Q7 384^3 (382
-// GLUPS; the two-step tile of tb3d.cuh 259, one step per launch 147); a third of the computed cells are halo,
+// What bounds it: K = 4 moves 12 bytes of DRAM per FP32 update, 0.76 of the measured copy on D3Q7 384^3 (426
+// GLUPS, 256^3 373; the two-step tile of tb3d.cuh 259, one step per launch 147); a third of the computed cells are halo,
 // and the warps wait for the barrier and the shared-memory queue (12 warps per SM at 152 registers).
-// Measured on 384^3 / 256^3 and not taken: a row of 128 columns per warp with the +-y of S(t) in
+// Refilled before the barrier, with the end lanes' words copied into slots of their own, 385 / 346.
+// Measured on 384^3 / 256^3 with the refill before the barrier and not taken: a row of 128 columns per warp with the +-y of S(t) in
 // registers (260 / 219); two rows per thread, 256 threads (352 / 345) or 384 (spills, 312 / 287); three
 // levels with 512 threads (302 / 264); levels behind branches on the iteration (307 / 278); the warps' end
 // words stored under a branch (315 / 283); two stages instead of three (367 / 331).
@@ -260,10 +262,11 @@ __global__ void __launch_bounds__(kPpThreads, 1) k_plane_pipe(const float *__res
     auto iteration = [&](int i, auto P, auto kAll) {
         constexpr bool all = decltype(kAll)::value;
         copy_wait<kPpStages - 2>();
+        // The plane, and levels 1 .. K-1 of the iteration before, are visible; their other slots are free, and so is
+        // the ring slot of the plane before, which the neighbouring warps read too (first): it is fetched into from here.
+        __syncthreads();
         fetch(free_slot);  // (the last ones of a segment are not used)
         copy_commit();
-        // The plane, and levels 1 .. K-1 of the iteration before, are visible; their other slots are free.
-        __syncthreads();
         PpRow r;
         first(r);
         static_for<K - 1>([&](auto Lx) {
