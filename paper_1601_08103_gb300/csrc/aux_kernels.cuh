@@ -342,29 +342,87 @@ __device__ __forceinline__ bool shell_sums(const T *__restrict__ g, long long pi
     return finite;
 }
 
-// Exact sums of values that are FP32 numbers (every storage but FP64) on the integer pipe.  With E the
-// largest biased exponent among them, a value is its 24-bit mantissa, shifted left by kFixBits (a reduction:
-// kFixBitsSum) and right by its own distance from E: a 64-bit integer in units of 2^(E - 150 - kFixBits).  Nothing is lost down to
-// 2^-34 of the largest value and no more than 2^-58 of it below, which is finer than FP64 sums of them;
-// the sums are rounded to FP64 once.  Zeros and denormals (E of their own 0) shift out to nothing where E is
-// kFixLeast or more; smaller values, infinities and NaN take FP64 sums.
-constexpr int kFixBits = 34, kFixBitsSq = 10;
-constexpr unsigned kFixLeast = 64;
-// Whether the sums of n values stay inside their 64 bits: a value is below 2^(24 + bits) in magnitude and the signed
-// sum below 2^63 (31 values with 34 bits, 63 with 33), a square below 2^(48 + kFixBitsSq) and the unsigned sum below 2^64.
-__host__ __device__ constexpr bool fix_fits(int n, int bits) { return n < 1 << (63 - 24 - bits); }
-__host__ __device__ constexpr bool fix_fits_sq(int n) { return n < 1 << (64 - 48 - kFixBitsSq); }
+// Sums of values that are FP32 numbers (every storage but FP64) on the integer pipe.  With E the largest biased
+// exponent among them, a value is its 24-bit mantissa, shifted left by kFixBits and right by its own distance from E: a
+// 64-bit integer in units of 2^(E - 150 - kFixBits), added exactly and rounded to FP64 once.  Zeros shift out to
+// nothing.  Where values are so far apart that bits of the smaller ones are shifted out (FixRange::exact is false; not in
+// FP16, whose range is narrow), they add those bits in FP64 (fix_rest): a sum of small values beside large ones of another sum
+// keeps the precision of an FP64 sum of its own terms.  Infinities and NaN take FP64 sums.
+constexpr int kFixBits = 33, kFixBitsSq = 10;
+// Whether the sums of n values stay inside their 64 bits: a value is below 2^(24 + kFixBits) in magnitude and the signed
+// sum below 2^63, a square below 2^(48 + kFixBitsSq) and the unsigned sum below 2^64.
+__host__ __device__ constexpr bool fix_fits(int n) {
+    return n < 1 << (63 - 24 - kFixBits) && n < 1 << (64 - 48 - kFixBitsSq);
+}
+template <class T>
+__host__ __device__ constexpr bool fixed_sums() {
+    return !std::is_same<T, double>::value;
+}
+// Exponents by which two values may differ so that no bit is shifted out: kFixBits and the trailing zeros that the
+// storage leaves in 24 bits (FP16: 11-bit mantissas, and no values further apart than 2^40).
+template <class T>
+__host__ __device__ constexpr int fix_spread() {
+    return kFixBits + (std::is_same<T, __half>::value ? 13 : std::is_same<T, __nv_bfloat16>::value ? 16 : 0);
+}
+template <class T>
+__host__ __device__ constexpr bool fix_always_exact() {
+    return std::is_same<T, __half>::value;
+}
+// Magnitudes of a set of values: the largest one's bits, and those of the smallest that is not zero, less 1, of the moving
+// and of the rest populations.  (Of fields with theta' in balance with rho' the rest populations are what rounding
+// leaves of zero, far below the moving ones: they alone are looked at then.)
+template <class T>
+struct FixRange {
+    unsigned most = 0, least[2] = {0xFFFFFFFFu, 0xFFFFFFFFu};
+    __device__ __forceinline__ void add(unsigned bits, bool rest) {
+        const unsigned a = bits & 0x7FFFFFFFu;
+        most = a > most ? a : most;
+        if constexpr (!fix_always_exact<T>()) least[rest] = a - 1u < least[rest] ? a - 1u : least[rest];
+    }
+    __device__ __forceinline__ bool finite() const { return most < 0x7F800000u; }
+    __device__ __forceinline__ unsigned exponent() const { return most >> 23; }
+    // whether none of the moving (rest) values loses bits
+    __device__ __forceinline__ bool exact(bool rest) const {
+        return fix_always_exact<T>() || least[rest] == 0xFFFFFFFFu ||
+               (most >> 23) - ((least[rest] + 1u) >> 23) <= (unsigned)fix_spread<T>();
+    }
+};
+// Zeros shift out from an exponent of 57 on.  Values that are all smaller than 2^-63 are multiplied by 2^kFixLift first,
+// which makes their denormals normal numbers too; returns the factor's exponent.
+constexpr int kFixLift = 100;
+template <class T, int N, int Q>
+__device__ __forceinline__ int fix_lift(unsigned (&b)[N][Q], FixRange<T> &range) {
+    if (fix_always_exact<T>() || range.most >= 64u << 23) return 0;
+    range = FixRange<T>();
+#pragma unroll
+    for (int c = 0; c < N; ++c)
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            b[c][i] = __float_as_uint(__uint_as_float(b[c][i]) * 0x1p100f);
+            range.add(b[c][i], i == 0);
+        }
+    return kFixLift;
+}
 __device__ __forceinline__ int fix_shift(unsigned bits, unsigned E) {
     const int s = (int)(E - ((bits >> 23) & 0xFFu));
     return s < 63 ? s : 63;
 }
-template <int kBits = kFixBits>
 __device__ __forceinline__ long long fix_value(unsigned bits, int shift) {
-    const long long m = (long long)(((unsigned long long)((bits & 0x7FFFFFu) | 0x800000u) << kBits) >> shift);
+    const long long m = (long long)(((unsigned long long)((bits & 0x7FFFFFu) | 0x800000u) << kFixBits) >> shift);
     const long long sign = (int)bits >> 31;
     return (m ^ sign) - sign;
 }
-// Its square, in units of 2^(2 (E - 150) - kFixBitsSq).
+// The part of a value that fix_value shifts out (exact in FP32), by exponent E and lift of its set.
+__device__ __forceinline__ double fix_rest(float value, unsigned E, int lift) {
+    if (lift) value *= 0x1p100f;
+    const unsigned bits = __float_as_uint(value);
+    const int n = fix_shift(bits, E) - kFixBits;  // mantissa bits
+    const unsigned kept = n <= 0 ? bits : n < 24 ? bits & ~((1u << n) - 1u) : 0u;
+    const double rest = (double)(value - __uint_as_float(kept));
+    return lift ? rest * 0x1p-100 : rest;
+}
+// Its square, in units of 2^(2 (E - 150) - kFixBitsSq); squares add up, so what small ones lose (2^-58 of the largest)
+// is less than an FP64 sum's rounding.
 __device__ __forceinline__ unsigned long long fix_square(unsigned bits, int shift) {
     const unsigned m = (bits & 0x7FFFFFu) | 0x800000u;
     const int s = 2 * shift;
@@ -384,44 +442,39 @@ __device__ __forceinline__ double fix_double(I v, int e) {
     const int hi = (int)(q >> 32) + ((1023 + 63 - 1 - n + e) << 20);
     return u == 0 ? 0.0 : __hiloint2double(minus ? hi | (int)0x80000000 : hi, (int)(unsigned)q);
 }
-template <class T>
-__host__ __device__ constexpr bool fixed_sums() {
-    return !std::is_same<T, double>::value;
-}
 
 // Per-cell moments (Sec. 4 discrete moments, Sec. 5 temperature) in FP64.
-// D3Q7 384^3 FP32: 2.89 ms with FP64 sums and conversions, 0.92 ms with integer ones (0.57 at the copy rate);
-// D3Q19 256^3: 2.44 -> 0.43 ms.
+// D3Q7 384^3 FP32: 2.89 ms with FP64 sums and conversions, 0.97 ms with integer ones (0.57 at the copy rate);
+// D3Q19 256^3: 2.44 -> 0.53 ms.
 template <class S, class T>
 __global__ void k_moments(const T *__restrict__ g, long long cells, long long pitch, SetConsts k, double *__restrict__ rho,
                           double *__restrict__ u, double *__restrict__ theta) {
     constexpr bool scaled = Store<T>::scaled;
     constexpr int NS = n_shells<S>(), D = S::D;
-    static_assert(fix_fits(S::Q, kFixBits), "signed sums of a cell");
+    static_assert(fix_fits(S::Q), "integer sums of a cell");
     for (long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x; x < cells; x += (long long)gridDim.x * blockDim.x) {
         // shell sums; where the storage is not scaled their total and the momentum over all shells, else the
         // momentum of each
         constexpr int NJ = scaled ? NS : 1;
-        double P[NS], J[NJ][3], total = 0.0;
+        double P[NS], J[NJ][3] = {}, total = 0.0;
         bool done = false;
         if constexpr (fixed_sums<T>()) {
-            unsigned b[S::Q], most = 0;
+            unsigned b[1][S::Q];
+            FixRange<T> range;
             static_for<S::Q>([&](auto I) {
                 constexpr int i = decltype(I)::value;
-                b[i] = __float_as_uint((float)load_elem<S, T>(g, pitch, (long long)i * pitch + x));
-                const unsigned a = b[i] & 0x7FFFFFFFu;
-                most = a > most ? a : most;
+                b[0][i] = __float_as_uint((float)load_elem<S, T>(g, pitch, (long long)i * pitch + x));
+                range.add(b[0][i], i == 0);
             });
-            const unsigned E = most >> 23;
-            if (most == 0) {
+            if (range.most == 0) {
                 done = true;
 #pragma unroll
                 for (int s = 0; s < NS; ++s) P[s] = 0.0;
-#pragma unroll
-                for (int s = 0; s < NJ; ++s) J[s][0] = J[s][1] = J[s][2] = 0.0;
-            } else if (E >= kFixLeast && E < 255u) {
+            } else if (range.finite()) {
                 done = true;
-                long long p[NS], j[NJ][3];
+                const int lift = fix_lift<T>(b, range);
+                const unsigned E = range.exponent();
+                long long p[NS], j[NJ][3], all = 0;
 #pragma unroll
                 for (int s = 0; s < NS; ++s) p[s] = 0;
 #pragma unroll
@@ -429,7 +482,7 @@ __global__ void k_moments(const T *__restrict__ g, long long cells, long long pi
                 static_for<S::Q>([&](auto I) {
                     constexpr int i = decltype(I)::value;
                     constexpr int s = shell_slot<S>(S::shell(i)), sj = scaled ? s : 0;
-                    const long long v = fix_value(b[i], fix_shift(b[i], E));
+                    const long long v = fix_value(b[0][i], fix_shift(b[0][i], E));
                     p[s] += v;
                     static_for<D>([&](auto A) {
                         constexpr int a = decltype(A)::value;
@@ -437,8 +490,7 @@ __global__ void k_moments(const T *__restrict__ g, long long cells, long long pi
                         if constexpr (S::c(i, a) == -1) j[sj][a] -= v;
                     });
                 });
-                const int e = (int)E - 150 - kFixBits;
-                long long all = 0;
+                const int e = (int)E - 150 - kFixBits - lift;
 #pragma unroll
                 for (int s = 0; s < NS; ++s) {
                     all += p[s];
@@ -450,6 +502,40 @@ __global__ void k_moments(const T *__restrict__ g, long long cells, long long pi
                     for (int s = 0; s < NJ; ++s)
 #pragma unroll
                         for (int a = 0; a < D; ++a) J[s][a] = fix_double(j[s][a], e);
+                }
+                // and what was shifted out
+                if (!range.exact(true)) {
+                    const double v = fix_rest(load_elem<S, T>(g, pitch, x), E, lift);
+                    if constexpr (scaled) P[0] += v;
+                    else total += v;
+                }
+                if (!range.exact(false)) {  // (of values read again: they need no registers till here)
+                    long long again = x;
+                    asm volatile("" : "+l"(again));
+                    double Pr[NS], Jr[NJ][3], totalr = 0.0;
+#pragma unroll
+                    for (int s = 0; s < NS; ++s) Pr[s] = 0.0;
+#pragma unroll
+                    for (int s = 0; s < NJ; ++s) Jr[s][0] = Jr[s][1] = Jr[s][2] = 0.0;
+                    static_for<S::Q - 1>([&](auto I) {
+                        constexpr int i = 1 + decltype(I)::value;
+                        constexpr int s = shell_slot<S>(S::shell(i)), sj = scaled ? s : 0;
+                        const double v = fix_rest(load_elem<S, T>(g, pitch, (long long)i * pitch + again), E, lift);
+                        Pr[s] += v;
+                        if constexpr (!scaled) totalr += v;
+                        static_for<D>([&](auto A) {
+                            constexpr int a = decltype(A)::value;
+                            if constexpr (S::c(i, a) == 1) Jr[sj][a] += v;
+                            if constexpr (S::c(i, a) == -1) Jr[sj][a] -= v;
+                        });
+                    });
+#pragma unroll
+                    for (int s = 1; s < NS; ++s) P[s] += Pr[s];
+                    total += totalr;
+#pragma unroll
+                    for (int s = 0; s < NJ; ++s)
+#pragma unroll
+                        for (int a = 0; a < D; ++a) J[s][a] += Jr[s][a];
                 }
             }
         }
@@ -514,7 +600,7 @@ __host__ __device__ constexpr int reduce_nraw() {
     return 2 * n_shells<S>() + n_shells<S>() * S::D + 1;
 }
 
-// Adds one cell in FP64: the cells that the integer form leaves.
+// Adds one cell in FP64: the cells of a group with infinities or NaN.
 template <class S, class T>
 __device__ __forceinline__ void reduce_cell(const T *__restrict__ g, long long pitch, long long x,
                                             double (&acc)[reduce_nraw<S>()]) {
@@ -557,13 +643,37 @@ __device__ __forceinline__ void reduce_cell(const double *__restrict__ g, long l
     });
 }
 
-// One block's share: chunks of kReduceGroup cells per thread, a block's width apart.  FP32 and 16-bit values
-// of a thread's group are added as integers and reach the FP64 accumulators as one value per sum
-// (D3Q7 384^3 FP32: 4.32 ms with FP64 sums of every value, 0.70 ms so, 0.24 at the copy rate; D3Q19 256^3 3.81 ->
-// 0.70 ms).
-// The group of a shell of 12 velocities (D3Q13, D3Q19) has 48 values of one sign and size in an ordinary field, 2^5.6 of
-// them: one bit less than the moments' sums.
-constexpr int kReduceGroup = 4, kFixBitsSum = kFixBits - 1;
+// The values of four cells from cell x (zeros from `cells` on), as FP32 bits.  wide: every velocity's elements lie so
+// that four of them can be read at once.
+template <class S, class T>
+__device__ __forceinline__ void load_group(const T *__restrict__ g, long long pitch, long long x, long long cells,
+                                           bool wide, unsigned (&b)[4][S::Q]) {
+    if (wide && x + 4 <= cells) {
+        static_for<S::Q>([&](auto I) {
+            constexpr int i = decltype(I)::value;
+            const long long at = (long long)i * pitch + x;
+            float v[4];
+            if constexpr (std::is_same<T, Bfp16>::value) bfp_load_vec<4>(g + at, bfp_exps<S::Q>(g, pitch) + (at >> 3), v);
+            else load_vec<T, 4>(g + at, v);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) b[c][i] = __float_as_uint(v[c]);
+        });
+    } else {
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            static_for<S::Q>([&](auto I) {
+                constexpr int i = decltype(I)::value;
+                b[c][i] = x + c < cells ? __float_as_uint((float)load_elem<S, T>(g, pitch, (long long)i * pitch + x + c)) : 0u;
+            });
+    }
+}
+
+// One block's share.  FP32 and 16-bit values of a thread's kReduceGroup cells, which lie side by side (so that
+// their values are of one size in a smooth field), are added as integers and reach the FP64 accumulators as one value
+// per sum; the group of a shell of 12 velocities (D3Q13, D3Q19) has 48 of them.
+// (D3Q7 384^3 FP32: 4.32 ms with FP64 sums of every value, 0.75 ms so, 0.24 at the copy rate; D3Q19 256^3 3.81 ->
+// 0.61 ms; with cells a block's width apart 0.72 and 0.66, but 1.78 and 3.19 where a pulse falls off, now 0.47 and 0.64).
+constexpr int kReduceGroup = 4;
 template <class S>
 __host__ __device__ constexpr int most_in_shell() {
     int most = 0;
@@ -574,13 +684,17 @@ __host__ __device__ constexpr int most_in_shell() {
     }
     return most;
 }
+// Blocks per SM: the launch has three (reduce_blocks) where their registers fit.
+template <class S>
+__host__ __device__ constexpr int reduce_min_blocks() {
+    return S::Q <= 9 ? 3 : S::Q <= 13 ? 2 : 1;
+}
 template <class S, class T>
-__global__ void __launch_bounds__(kReduceThreads) k_reduce_partial(const T *__restrict__ g, long long cells, long long pitch,
+__global__ void __launch_bounds__(kReduceThreads, reduce_min_blocks<S>()) k_reduce_partial(const T *__restrict__ g, long long cells, long long pitch,
                                                                    double *__restrict__ partial) {
     constexpr int NS = n_shells<S>(), D = S::D, NR = reduce_nraw<S>(), G = kReduceGroup;
     static_assert(NR <= kReduceMax, "raw accumulators do not fit");
-    static_assert(fix_fits(G * most_in_shell<S>(), kFixBitsSum), "signed sums of a group's shell");
-    static_assert(fix_fits_sq(G * most_in_shell<S>()), "sums of squares of a group's shell");
+    static_assert(G == 4 && fix_fits(G * most_in_shell<S>()), "integer sums of a group's shell");
     double acc[NR];
 #pragma unroll
     for (int v = 0; v < NR; ++v) acc[v] = 0.0;
@@ -593,66 +707,81 @@ __global__ void __launch_bounds__(kReduceThreads) k_reduce_partial(const T *__re
         each.bad = 0.0;
     }
     const long long span = (long long)kReduceThreads * G;
-    for (long long x0 = (long long)blockIdx.x * span + threadIdx.x; x0 < cells; x0 += (long long)gridDim.x * span) {
-        if constexpr (fixed_sums<T>()) {
-            unsigned b[G][S::Q], most = 0;
+    if constexpr (fixed_sums<T>()) {
+        const bool wide = pitch % 4 == 0 && reinterpret_cast<unsigned long long>(g) % (4 * sizeof(T)) == 0;
+        for (long long x0 = (long long)blockIdx.x * span + G * threadIdx.x; x0 < cells; x0 += (long long)gridDim.x * span) {
+            unsigned b[G][S::Q];
+            load_group<S, T>(g, pitch, x0, cells, wide, b);
+            FixRange<T> range;
+#pragma unroll
+            for (int c = 0; c < G; ++c)
+#pragma unroll
+                for (int i = 0; i < S::Q; ++i) range.add(b[c][i], i == 0);
+            if (range.most == 0) continue;  // (zeros add nothing)
+            if (!range.finite()) {
+#pragma unroll 1
+                for (long long x = x0; x < x0 + G && x < cells; ++x) reduce_cell<S, T>(g, pitch, x, acc);
+                continue;
+            }
+            const int lift = fix_lift<T>(b, range);
+            const unsigned E = range.exponent();
+            long long p[NS], j[NS][3];
+            unsigned long long q[NS];
+#pragma unroll
+            for (int s = 0; s < NS; ++s) {
+                q[s] = 0;
+                p[s] = j[s][0] = j[s][1] = j[s][2] = 0;
+            }
 #pragma unroll
             for (int c = 0; c < G; ++c) {
-                const long long x = x0 + (long long)c * kReduceThreads;
-                const bool in = x < cells;
                 static_for<S::Q>([&](auto I) {
                     constexpr int i = decltype(I)::value;
-                    b[c][i] = in ? __float_as_uint((float)load_elem<S, T>(g, pitch, (long long)i * pitch + x)) : 0u;
-                    const unsigned a = b[c][i] & 0x7FFFFFFFu;
-                    most = a > most ? a : most;
+                    constexpr int s = shell_slot<S>(S::shell(i));
+                    const int shift = fix_shift(b[c][i], E);
+                    const long long v = fix_value(b[c][i], shift);
+                    p[s] += v;
+                    q[s] += fix_square(b[c][i], shift);
+                    static_for<D>([&](auto A) {
+                        constexpr int a = decltype(A)::value;
+                        if constexpr (S::c(i, a) == 1) j[s][a] += v;
+                        if constexpr (S::c(i, a) == -1) j[s][a] -= v;
+                    });
                 });
             }
-            const unsigned E = most >> 23;
-            if (most == 0) continue;  // (zeros add nothing)
-            if (E >= kFixLeast && E < 255u) {
-                long long p[NS], j[NS][3];
-                unsigned long long q[NS];
+            const int e = (int)E - 150 - lift;
+            static_for<NS>([&](auto Kx) {
+                constexpr int k = decltype(Kx)::value;
+                acc[k] += fix_double(p[k], e - kFixBits);
+                acc[NS + k] += fix_double(q[k], 2 * e - kFixBitsSq);
+                if constexpr (k > 0) {
 #pragma unroll
-                for (int s = 0; s < NS; ++s) {
-                    q[s] = 0;
-                    p[s] = j[s][0] = j[s][1] = j[s][2] = 0;
+                    for (int a = 0; a < D; ++a) acc[2 * NS + k * D + a] += fix_double(j[k][a], e - kFixBits);
                 }
-#pragma unroll
-                for (int c = 0; c < G; ++c) {
-                    static_for<S::Q>([&](auto I) {
-                        constexpr int i = decltype(I)::value;
+            });
+            // and what was shifted out, of values read again
+            if (!range.exact(true)) {
+#pragma unroll 1
+                for (long long x = x0; x < x0 + G && x < cells; ++x) acc[0] += fix_rest(load_elem<S, T>(g, pitch, x), E, lift);
+            }
+            if (!range.exact(false)) {
+#pragma unroll 1
+                for (long long x = x0; x < x0 + G && x < cells; ++x) {
+                    static_for<S::Q - 1>([&](auto I) {
+                        constexpr int i = 1 + decltype(I)::value;
                         constexpr int s = shell_slot<S>(S::shell(i));
-                        const int shift = fix_shift(b[c][i], E);
-                        const long long v = fix_value<kFixBitsSum>(b[c][i], shift);
-                        p[s] += v;
-                        q[s] += fix_square(b[c][i], shift);
+                        const double v = fix_rest(load_elem<S, T>(g, pitch, (long long)i * pitch + x), E, lift);
+                        acc[s] += v;
                         static_for<D>([&](auto A) {
                             constexpr int a = decltype(A)::value;
-                            if constexpr (S::c(i, a) == 1) j[s][a] += v;
-                            if constexpr (S::c(i, a) == -1) j[s][a] -= v;
+                            if constexpr (S::c(i, a) == 1) acc[2 * NS + s * D + a] += v;
+                            if constexpr (S::c(i, a) == -1) acc[2 * NS + s * D + a] -= v;
                         });
                     });
                 }
-                const int e = (int)E - 150;
-                static_for<NS>([&](auto Kx) {
-                    constexpr int k = decltype(Kx)::value;
-                    acc[k] += fix_double(p[k], e - kFixBitsSum);
-                    acc[NS + k] += fix_double(q[k], 2 * e - kFixBitsSq);
-                    if constexpr (k > 0) {
-#pragma unroll
-                        for (int a = 0; a < D; ++a) acc[2 * NS + k * D + a] += fix_double(j[k][a], e - kFixBitsSum);
-                    }
-                });
-                continue;
             }
         }
-        if constexpr (fixed_sums<T>()) {
-#pragma unroll 1
-            for (int c = 0; c < G; ++c) {
-                const long long x = x0 + (long long)c * kReduceThreads;
-                if (x < cells) reduce_cell<S, T>(g, pitch, x, acc);
-            }
-        } else {
+    } else {
+        for (long long x0 = (long long)blockIdx.x * span + threadIdx.x; x0 < cells; x0 += (long long)gridDim.x * span) {
 #pragma unroll
             for (int c = 0; c < G; ++c) {
                 const long long x = x0 + (long long)c * kReduceThreads;
