@@ -622,24 +622,53 @@ __device__ __forceinline__ void reduce_cell(const T *__restrict__ g, long long p
         }
     });
 }
-// FP64 accumulators of a thread for FP64 states: one sum per velocity and one sum of squares per shell (two
-// FP64 instructions per value; the shells' sums and momenta are put together once, at the end).
-template <class S>
-struct ReduceSums {
-    double g[S::Q], sq[n_shells<S>()], bad;
-};
-template <class S>
-__device__ __forceinline__ void reduce_cell(const double *__restrict__ g, long long pitch, long long x,
-                                            ReduceSums<S> &acc) {
-    static_for<S::Q>([&](auto I) {
-        constexpr int i = decltype(I)::value;
-        const double v = g[(long long)i * pitch + x];
-        if (isfinite(v)) {
-            acc.g[i] += v;
-            acc.sq[shell_slot<S>(S::shell(i))] = fma(v, v, acc.sq[shell_slot<S>(S::shell(i))]);
-        } else {
-            acc.bad += 1.0;
+// Adds an FP64 state's values of N cells (one or four), `stride` apart.  A pair of opposite velocities
+// gives a sum and a difference, so that momentum adds up the differences, which may be far smaller than the populations; the
+// cells are added to one another before they reach the accumulator.  With one accumulator per velocity, and momentum from them at the
+// end, there would be a third fewer FP64 instructions, but momentum would carry the roundings of the populations' sums.
+template <class S, int N>
+__device__ __forceinline__ void reduce_group(const double *__restrict__ g, long long pitch, long long x, long long stride,
+                                             double (&acc)[reduce_nraw<S>()], int &bad) {
+    constexpr int NS = n_shells<S>(), D = S::D;
+    auto load = [&](int i, double (&v)[N]) {
+#pragma unroll
+        for (int c = 0; c < N; ++c) v[c] = __ldg(g + (long long)i * pitch + x + c * stride);
+#pragma unroll
+        for (int c = 0; c < N; ++c)
+            if ((((unsigned)__double2hiint(v[c]) >> 20) & 0x7FFu) == 0x7FFu) {  // (counted and left out)
+                v[c] = 0.0;
+                ++bad;
+            }
+    };
+    auto sum = [](const double (&v)[N]) {
+        if constexpr (N == 1) return v[0];
+        else return (v[0] + v[1]) + (v[2] + v[3]);
+    };
+    double r[N];
+    load(0, r);
+    acc[0] += sum(r);
+#pragma unroll
+    for (int c = 0; c < N; ++c) acc[NS] = fma(r[c], r[c], acc[NS]);
+    static_for<S::Q / 2>([&](auto H) {
+        constexpr int i = 1 + 2 * decltype(H)::value;
+        constexpr int k = shell_slot<S>(S::shell(i));
+        double v[N], o[N], t[N];
+        load(i, v);
+        load(i + 1, o);
+#pragma unroll
+        for (int c = 0; c < N; ++c) {
+            t[c] = v[c] + o[c];
+            acc[NS + k] = fma(o[c], o[c], fma(v[c], v[c], acc[NS + k]));
         }
+        acc[k] += sum(t);
+#pragma unroll
+        for (int c = 0; c < N; ++c) t[c] = v[c] - o[c];
+        const double d = sum(t);
+        static_for<D>([&](auto A) {
+            constexpr int a = decltype(A)::value;
+            if constexpr (S::c(i, a) == 1) acc[2 * NS + k * D + a] += d;
+            if constexpr (S::c(i, a) == -1) acc[2 * NS + k * D + a] -= d;
+        });
     });
 }
 
@@ -698,16 +727,8 @@ __global__ void __launch_bounds__(kReduceThreads, reduce_min_blocks<S>()) k_redu
     double acc[NR];
 #pragma unroll
     for (int v = 0; v < NR; ++v) acc[v] = 0.0;
-    [[maybe_unused]] ReduceSums<S> each;
-    if constexpr (!fixed_sums<T>()) {
-#pragma unroll
-        for (int v = 0; v < S::Q; ++v) each.g[v] = 0.0;
-#pragma unroll
-        for (int v = 0; v < NS; ++v) each.sq[v] = 0.0;
-        each.bad = 0.0;
-    }
-    const long long span = (long long)kReduceThreads * G;
     if constexpr (fixed_sums<T>()) {
+        const long long span = (long long)kReduceThreads * G;
         const bool wide = pitch % 4 == 0 && reinterpret_cast<unsigned long long>(g) % (4 * sizeof(T)) == 0;
         for (long long x0 = (long long)blockIdx.x * span + G * threadIdx.x; x0 < cells; x0 += (long long)gridDim.x * span) {
             unsigned b[G][S::Q];
@@ -781,28 +802,12 @@ __global__ void __launch_bounds__(kReduceThreads, reduce_min_blocks<S>()) k_redu
             }
         }
     } else {
-        for (long long x0 = (long long)blockIdx.x * span + threadIdx.x; x0 < cells; x0 += (long long)gridDim.x * span) {
-#pragma unroll
-            for (int c = 0; c < G; ++c) {
-                const long long x = x0 + (long long)c * kReduceThreads;
-                if (x < cells) reduce_cell<S>(g, pitch, x, each);
-            }
-        }
-    }
-    if constexpr (!fixed_sums<T>()) {
-        static_for<S::Q>([&](auto I) {
-            constexpr int i = decltype(I)::value;
-            constexpr int k = shell_slot<S>(S::shell(i));
-            acc[k] += each.g[i];
-            static_for<D>([&](auto A) {
-                constexpr int a = decltype(A)::value;
-                if constexpr (S::c(i, a) == 1) acc[2 * NS + k * D + a] += each.g[i];
-                if constexpr (S::c(i, a) == -1) acc[2 * NS + k * D + a] -= each.g[i];
-            });
-        });
-#pragma unroll
-        for (int k = 0; k < NS; ++k) acc[NS + k] = each.sq[k];
-        acc[NR - 1] = each.bad;
+        const long long stride = (long long)gridDim.x * kReduceThreads;
+        int bad = 0;
+        long long x = (long long)blockIdx.x * kReduceThreads + threadIdx.x;
+        for (; x + (G - 1) * stride < cells; x += G * stride) reduce_group<S, G>(g, pitch, x, stride, acc, bad);
+        for (; x < cells; x += stride) reduce_group<S, 1>(g, pitch, x, stride, acc, bad);
+        acc[NR - 1] = (double)bad;
     }
     __shared__ double sh[kReduceThreads / 32][NR];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;

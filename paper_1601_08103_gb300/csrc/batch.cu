@@ -501,7 +501,7 @@ lee_status lee_batch_create(int32_t set, int32_t storage, const lee_batch_domain
     b->total_cells = total;
     b->max_cells = maxc;
     b->st = static_cast<cudaStream_t>(cuda_stream);
-    b->red_blocks = reduce_blocks(maxc);
+    b->red_blocks = reduce_blocks(maxc, storage);
     cudaError_t e = cudaGetDevice(&b->device);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaMalloc(&b->buf[0], b->elem * (size_t)off);
@@ -643,7 +643,7 @@ lee_status lee_batch_reduce(lee_batch *b, int32_t d, double *out, int32_t on_dev
     if (s != LEE_OK) return s;
     if (d < 0 || d >= b->count || !out) return bfail(b, LEE_ERR_INVALID_ARGUMENT, "reduce: bad args");
     const long long c = b->cells[d];
-    const int nblocks = reduce_blocks(c);
+    const int nblocks = reduce_blocks(c, b->storage);
     const SetConsts k = consts_for(b->set, 1.0);
     BCK(b, b->ops->reduce_partial(b->storage, dom_ptr(b, b->cur, d), c, b->pitch[d], k, b->partial, nblocks, b->st),
         "reduce_partial");

@@ -538,7 +538,7 @@ lee_status lee_lbm_create(const lee_lbm_config *cfg, lee_lbm **out) {
     const size_t bytes = state_bytes(cfg->storage, h->D, h->Q, h->pitch);
     if (e == cudaSuccess) e = cudaMalloc(&h->buf[0], bytes);
     if (e == cudaSuccess) e = cudaMalloc(&h->buf[1], bytes);
-    h->nblocks = reduce_blocks(cells);
+    h->nblocks = reduce_blocks(cells, cfg->storage);
     if (e == cudaSuccess) e = cudaMalloc(&h->partial, sizeof(double) * kReduceMax * (size_t)h->nblocks);
     if (e == cudaSuccess) e = cudaMalloc(&h->red_out, sizeof(double) * kReduceMax);
     if (e == cudaSuccess) e = cudaMalloc(&h->maxbits, 2 * sizeof(unsigned int));

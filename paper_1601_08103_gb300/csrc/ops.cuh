@@ -222,12 +222,18 @@ inline int aux_blocks(long long cells, int threads = 256) {
 
 // Blocks of a reduction: as many as fit on the SMs at once.  A block's own reduction (a dozen FP64 sums over its
 // warps) costs as much as some thousand cells on GB300's FP64 pipe: with the 16 blocks per SM of the other
-// auxiliary kernels it took 45 us of a 2048^2 FP32 reduction.
-inline int reduce_blocks(long long cells) {
-    constexpr int kMost = 152 * 3;
+// auxiliary kernels it took 45 us of a 2048^2 FP32 reduction.  Up to there a thread takes one cell of an FP64 or split
+// state (137x197 cells: FP64 19 us with four of them one after another, 16 so; split storage 30 and 18) and one group of
+// the others'.  Split storage adds value by value: beyond 64 cells per thread the 16 blocks per SM keep its sums short.
+inline int reduce_blocks(long long cells, int storage) {
+    constexpr long long kMost = 152 * 3;
     static_assert(kMost <= kMaxAuxBlocks, "rows of the partial-sum buffers");
-    const long long b = (cells + kReduceThreads * kReduceGroup - 1) / (kReduceThreads * kReduceGroup);
-    return (int)(b > kMost ? kMost : b < 1 ? 1 : b);
+    const bool single = storage == LEE_STORE_F64 || storage == LEE_STORE_SPLIT16;
+    const int per_block = single ? kReduceThreads : kReduceThreads * kReduceGroup;
+    const long long b = (cells + per_block - 1) / per_block;
+    const bool many = storage == LEE_STORE_SPLIT16 && cells > kMost * kReduceThreads * 64;
+    const long long most = many ? kMaxAuxBlocks : kMost;
+    return (int)(b > most ? most : b < 1 ? 1 : b);
 }
 
 }  // namespace lee

@@ -11,8 +11,8 @@
 //
 // The scratch: kMaxPartials block partials x kReduceMax values in FP64 (2432 x 16 x 8 B =
 // 311,296 bytes).  Every GPU that loads the library holds this array until the process exits.
-// The launch shape is the one lee_lbm_reduce uses (min(ceil(cells / 256), 2432) blocks of 256
-// threads, grid-stride), so the two entry points sum in the same order and agree bit for bit.
+// The launch shape is the one lee_lbm_reduce uses (reduce_blocks), so the two entry points sum in the same order and
+// agree bit for bit.
 #include <cuda_runtime.h>
 
 #include <mutex>
@@ -28,7 +28,7 @@ using namespace lee;
 
 namespace {
 
-constexpr int kMaxPartials = kMaxAuxBlocks;  // rows of partials: the most blocks aux_blocks() gives
+constexpr int kMaxPartials = kMaxAuxBlocks;  // rows of partials: no launch shape has more
 static_assert(kMaxPartials * kReduceMax * sizeof(double) == 311296, "scratch size as documented in lee_lbm.h");
 constexpr int kMaxDevices = 64;
 
@@ -66,7 +66,7 @@ extern "C" lee_status lee_reduce_noalloc(int32_t set, int32_t storage, const voi
     if (cells < 1 || cells >= (1LL << 31) || pitch < cells) return LEE_ERR_INVALID_ARGUMENT;
     const bool is16 = storage == LEE_STORE_F16 || storage == LEE_STORE_BF16;
     if (is16 && !(store_scale > 0.0)) return LEE_ERR_INVALID_ARGUMENT;
-    const int nblocks = reduce_blocks(cells);
+    const int nblocks = reduce_blocks(cells, storage);
     if (nblocks > kMaxPartials) return LEE_ERR_INVALID_ARGUMENT;  // beyond the fixed scratch
     double *partials = nullptr;
     if (partials_on_current_device(&partials) != cudaSuccess) return LEE_ERR_CUDA;
