@@ -173,15 +173,24 @@ struct CollideCoef {
     C N[4][4];
 };
 
-// Open-edge treatment for non-periodic grids.
+// What a step does at the edges of its grid: wraps around, lets zeros enter, damps a frame of cells too (sponge_w of
+// them), or lets the populations `ghost` enter (2D).  Every kind has its own instances of the step kernels: the launches of
+// open grids are short, and in one instance for all of them each paid for the others' code (D2Q5 FP32, us per step,
+// zero edge / frame: 137x197 2.21 / 2.62 in one instance, 1.56 / 1.85 so; 1024^2 4.87 / 6.20 and 4.01 / 4.64).
+enum Edge { kWrapEdge, kZeroEdge, kFrameEdge, kGhostEdge };
 template <class C>
 struct OpenEdge {
-    int sponge_w;        // 0 = no sponge
+    int sponge_w;
     C sponge_smax;
-    const C *ghost;      // nullptr = zero-incoming; else [4][L] entering populations (2D)
+    const C *ghost;      // [4][L] entering populations, or nullptr = zeros
     int ghost_L;
-    int skip_border;     // 2D: leave the border cells unwritten (the learned edge's kernels own them)
+    int skip_border;     // leave the border cells unwritten (the learned edge's kernels own them)
 };
+template <class C>
+__device__ __forceinline__ bool in_frame(int x, int cells, int y, int z, const GridDesc &gd, int D, const OpenEdge<C> &ob) {
+    const int w = ob.sponge_w;
+    return x < w || x + cells > gd.nx - w || (D >= 2 && (y < w || y >= gd.ny - w)) || (D >= 3 && (z < w || z >= gd.nz - w));
+}
 
 // ---------------------------------------------------------------------------------------------
 // collision of one cell (index K of the per-thread vector)
@@ -530,11 +539,13 @@ __device__ __forceinline__ C sponge_factor(int x, int y, int z, const GridDesc &
 // 2D, z in 3D): along that axis nothing wraps -- the rows just before and after the grid are read
 // where they lie in memory, in the halo planes the caller keeps there -- and every other axis is
 // periodic.
-template <class S, class T, int V, bool OPEN, bool CUT = false>
+template <class S, class T, int V, Edge EDGE, bool CUT = false>
 __device__ __forceinline__ void stream_collide_chunk(const T *__restrict__ src, T *__restrict__ dst, const GridDesc &gd,
                                                      const CollideCoef<typename Store<T>::C> &cf,
                                                      const OpenEdge<typename Store<T>::C> &ob, long long raw) {
+    constexpr bool OPEN = EDGE != kWrapEdge;
     static_assert(!(CUT && OPEN), "a slab is periodic across its cut faces' neighbours");
+    static_assert(EDGE != kGhostEdge || S::D == 2, "entering populations of a 2D grid");
     using C = typename Store<T>::C;
     const bool active = raw < gd.nchunks;
     const long long chunk = active ? raw : gd.nchunks - 1;
@@ -545,6 +556,17 @@ __device__ __forceinline__ void stream_collide_chunk(const T *__restrict__ src, 
     const bool has_left = (lane > 0) && (xc > 0);
     const bool has_right = (lane < 31) && (xc < gd.nxc - 1);
 
+    // the frame damps rest populations that a step leaves alone elsewhere
+    [[maybe_unused]] bool framed = false;
+    [[maybe_unused]] C rest[V];
+    auto load_rest = [&] {
+        if (framed) load_vec<T, V>(src + ((long long)z * gd.ny + y) * gd.nx + x0, rest);
+    };
+    if constexpr (EDGE == kFrameEdge && rest_static<S>()) {
+        framed = in_frame(x0, V, y, z, gd, S::D, ob);
+        // Before the pulls in 3D, after them in 2D (us per step: D3Q7 192^3 FP32 56.6 and 62.0; D2Q5 32x32 FP16 2.75 and 2.49).
+        if constexpr (S::D == 3) load_rest();
+    }
     C pull[S::Q][V];
     static_for_carried<S>([&](auto I) {
         constexpr int i = decltype(I)::value;
@@ -566,7 +588,7 @@ __device__ __forceinline__ void stream_collide_chunk(const T *__restrict__ src, 
         } else {
 #pragma unroll
             for (int k = 0; k < V; ++k) v[k] = C(0);
-            if constexpr (OPEN && S::D == 2 && cx == 0) {
+            if constexpr (EDGE == kGhostEdge && cx == 0) {
                 if (ob.ghost != nullptr) {  // entering through the bottom (c_y = +1) or top edge
                     const C *gp = ob.ghost + (cy == 1 ? 2 : 3) * ob.ghost_L + x0;
 #pragma unroll
@@ -587,7 +609,7 @@ __device__ __forceinline__ void stream_collide_chunk(const T *__restrict__ src, 
                 bool out = row_out;
                 if (xs < 0) { if constexpr (OPEN) out = true; else xs += gd.nx; }
                 left = out ? C(0) : Store<T>::load(rowp[xs]);
-                if constexpr (OPEN && S::D == 2 && cy == 0) {
+                if constexpr (EDGE == kGhostEdge && cy == 0) {
                     if (xs < 0 && ob.ghost != nullptr) left = ob.ghost[0 * ob.ghost_L + y];
                 }
             }
@@ -604,7 +626,7 @@ __device__ __forceinline__ void stream_collide_chunk(const T *__restrict__ src, 
                 bool out = row_out;
                 if (xs >= gd.nx) { if constexpr (OPEN) out = true; else xs -= gd.nx; }
                 right = out ? C(0) : Store<T>::load(rowp[xs]);
-                if constexpr (OPEN && S::D == 2 && cy == 0) {
+                if constexpr (EDGE == kGhostEdge && cy == 0) {
                     if (x0 + V >= gd.nx && ob.ghost != nullptr) right = ob.ghost[1 * ob.ghost_L + y];
                 }
             }
@@ -614,31 +636,28 @@ __device__ __forceinline__ void stream_collide_chunk(const T *__restrict__ src, 
         }
     });
 
+    if constexpr (EDGE == kFrameEdge && rest_static<S>() && S::D < 3) load_rest();
     C post[S::Q][V];
     // one cell at a time: this kernel streams at the memory bound, and the packed f32x2 pairs
     // (same bits) cost it 9 to 12 registers and occupancy
     collide_chunk<S, false>(pull, post, cf);
 
-    if constexpr (OPEN) {
-        if (ob.sponge_w > 0) {
+    if constexpr (EDGE == kFrameEdge) {
+        if (rest_static<S>() ? framed : ob.sponge_w > 0) {
 #pragma unroll
             for (int k = 0; k < V; ++k) {
                 const C damp = sponge_factor<C>(x0 + k, y, z, gd, S::D, ob.sponge_w, ob.sponge_smax);
+                if constexpr (rest_static<S>()) rest[k] *= damp;
 #pragma unroll
                 for (int i = rest_static<S>() ? 1 : 0; i < S::Q; ++i) post[i][k] *= damp;
-                if constexpr (rest_static<S>()) {  // the frame damps its rest populations too
-                    if (active && damp != C(1)) {
-                        const long long x = ((long long)z * gd.ny + y) * gd.nx + x0 + k;
-                        dst[x] = Store<T>::make(Store<T>::load(src[x]) * damp);
-                    }
-                }
             }
+            if (rest_static<S>() && active) store_vec<T, V>(dst + ((long long)z * gd.ny + y) * gd.nx + x0, rest);
         }
     }
 
     if (active) {
         T *outp = dst + ((long long)z * gd.ny + y) * gd.nx + x0;
-        if constexpr (OPEN && S::D == 2) {
+        if constexpr (EDGE == kGhostEdge) {
             if (ob.skip_border) {
                 if (y == 0 || y == gd.ny - 1) return;
                 if (x0 == 0 || x0 + V >= gd.nx) {  // a chunk that holds x = 0 or x = nx - 1
@@ -705,11 +724,11 @@ __global__ void __launch_bounds__(1024) k_onchip_1d(T *__restrict__ g, int nx, l
 }
 
 // One fused time step on one grid: one thread per V-cell chunk.
-template <class S, class T, int V, bool OPEN, bool CUT = false>
+template <class S, class T, int V, Edge EDGE, bool CUT = false>
 __global__ void __launch_bounds__(256) k_stream_collide(const T *__restrict__ src, T *__restrict__ dst, GridDesc gd,
                                                         CollideCoef<typename Store<T>::C> cf,
                                                         OpenEdge<typename Store<T>::C> ob) {
-    stream_collide_chunk<S, T, V, OPEN, CUT>(src, dst, gd, cf, ob, (long long)blockIdx.x * blockDim.x + threadIdx.x);
+    stream_collide_chunk<S, T, V, EDGE, CUT>(src, dst, gd, cf, ob, (long long)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 __device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p)); }
@@ -735,7 +754,7 @@ __global__ void __launch_bounds__(512) k_stream_collide_batched(const T *__restr
     const BatchDomain<C> &D = doms[d];
     const long long raw = (long long)(blockIdx.x - D.first_block) * blockDim.x + threadIdx.x;
     const OpenEdge<C> none{0, C(0), nullptr, 0};
-    stream_collide_chunk<S, T, V, false>(src + D.offset, dst + D.offset, D.gd, D.cf, none, raw);
+    stream_collide_chunk<S, T, V, kWrapEdge>(src + D.offset, dst + D.offset, D.gd, D.cf, none, raw);
 }
 
 }  // namespace lee

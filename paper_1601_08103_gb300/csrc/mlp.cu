@@ -766,7 +766,7 @@ __global__ void __launch_bounds__(32 * kBoundaryWarps, learned_min_blocks<T, V>(
     using C = typename Store<T>::C;
     static_assert(32 * kBoundaryWarps == 256, "the interior chunks take 256 threads per block");
     if ((int)blockIdx.x >= nnet) {
-        stream_collide_chunk<S, T, V, true>(src, dst, gd, cf, ob,
+        stream_collide_chunk<S, T, V, kGhostEdge>(src, dst, gd, cf, ob,
                                             (long long)(blockIdx.x - nnet) * blockDim.x + threadIdx.x);
         return;
     }
