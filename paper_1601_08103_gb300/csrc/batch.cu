@@ -593,7 +593,18 @@ lee_status lee_batch_step(lee_batch *b, int64_t n, int32_t mode) {
     }
     if (!b->tuned && (s = tune(b)) != LEE_OK) return s;
     int64_t left = n;
-    if (mode == LEE_BATCH_GRAPH) {
+    // In a graph that the caller captures, an even number of launches where it can be had (see lee_lbm_step).
+    const bool captured = capturing(b->st);
+    if (captured && next_launch(b, left) == kRpDeep) {
+        int count = 0;
+        for (int64_t r = left; r > 0; ++count) r -= next_launch(b, r);
+        for (int k = 0; (count & 1) && k < kRpDeep; k += b->unit) {
+            BCK(b, launch_steps(b, b->cur, b->unit, b->st), "batched launch");
+            b->cur ^= 1;
+            left -= b->unit;
+        }
+    }
+    if (mode == LEE_BATCH_GRAPH && !captured) {
         // up to kMaxGraphSteps steps: one graph of all of them (one launch of the whole run); longer
         // runs: replays of a kChunkSteps graph
         const int64_t steps = left <= lee_batch::kMaxGraphSteps ? left : lee_batch::kChunkSteps;

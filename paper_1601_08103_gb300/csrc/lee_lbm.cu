@@ -244,6 +244,15 @@ int next_launch(const lee_lbm *h, int unit, long long left) {
     return left >= unit ? unit : 1;
 }
 
+// Steps of the first of the launches that can stand for one of k steps, with the same bits, in an even number more or less
+// (all of this size but for the last): 0 where there are none.
+int split_launch(const lee_lbm *h, int unit, int k) {
+    if (h->tb_env || k < 2) return 0;
+    if (h->D == 3) return k != h->ops->deep3d || !plane_pipe(h) ? 0 : k == 4 && unit == 2 ? 2 : 1;
+    if (k == kRpDeep) return 4;
+    return h->cfg.storage == LEE_STORE_F32 ? (k + 1) / 2 : 0;  // (a 16-bit state would be rounded at other steps)
+}
+
 // Whether the 1D on-chip path (all steps of a call in one launch) takes this grid.
 bool onchip(const lee_lbm *h) {
     return h->ops->onchip_1d && h->cfg.storage != LEE_STORE_SPLIT16 && h->cfg.storage != LEE_STORE_BFP16 &&
@@ -703,13 +712,18 @@ lee_status lee_lbm_step(lee_lbm *h, int64_t n) {
         if (e == cudaSuccess) e = cudaStreamWaitEvent(st, h->ev_join, 0);
         return e;
     };
+    // Where the caller captures the call into a graph, its launches leave the state in the copy that they found it in if
+    // they can: an even number of them, so that the graph advances the state each time it is replayed.
     if (n >= 2 && shifted(h)) {
-        L.src = state(h, h->cur);
-        L.dst = state(h, h->cur ^ 1);
         L.stream = h->st;
-        LEE_CK(h, h->ops->shift_1d(L, n), "1D shift launch");
-        h->cur ^= 1;
-        h->steps += n;
+        for (int64_t left = n, k = capturing(h->st) ? 1 : n; left > 0; k = left) {
+            L.src = state(h, h->cur);
+            L.dst = state(h, h->cur ^ 1);
+            LEE_CK(h, h->ops->shift_1d(L, k), "1D shift launch");
+            h->cur ^= 1;
+            h->steps += k;
+            left -= k;
+        }
         return LEE_OK;
     }
     // 1D grids that fit in shared memory: every step in one launch of the on-chip kernel
@@ -739,8 +753,22 @@ lee_status lee_lbm_step(lee_lbm *h, int64_t n) {
         }
         return c;
     };
+    auto run = [&](int k) -> lee_status {
+        LEE_CK(h, launch(h->cur, k, h->st), "step launch");
+        h->cur ^= 1;
+        h->steps += k;
+        return LEE_OK;
+    };
     int64_t left = n;
-    if (launches_of(left) >= kGraphMinLaunches) {
+    const int64_t count = launches_of(n);
+    if (n >= 2 && (count >= kGraphMinLaunches || (count & 1)) && capturing(h->st)) {
+        const int first = next_launch(h, unit, n), part = count & 1 ? split_launch(h, unit, first) : 0;
+        for (int k = part ? first : 0; k > 0; k -= part) {
+            const lee_status s = run(part < k ? part : k);
+            if (s != LEE_OK) return s;
+        }
+        if (part) left -= first;
+    } else if (count >= kGraphMinLaunches) {
         // Runs of up to kMaxGraphSteps steps are one launch of a graph holding all of them; longer runs
         // replay a kChunkGraphSteps graph.  Graphs are captured once per (starting copy, length) on a
         // private stream and replayed on the handle's stream.
@@ -775,10 +803,9 @@ lee_status lee_lbm_step(lee_lbm *h, int64_t n) {
     }
     while (left > 0) {
         const int k = next_launch(h, unit, left);
-        LEE_CK(h, launch(h->cur, k, h->st), "step launch");
-        h->cur ^= 1;
+        const lee_status s = run(k);
+        if (s != LEE_OK) return s;
         left -= k;
-        h->steps += k;
     }
     return LEE_OK;
 }

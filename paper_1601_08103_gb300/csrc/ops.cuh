@@ -18,6 +18,16 @@ constexpr int kRpDeep = 8;
 constexpr int kPpDeep = 4;
 inline bool plane_pipe_eligible(long long ny) { return ny <= 65535; }
 
+// Whether the caller is capturing the work of stream st into a graph of its own.
+inline bool capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &status) != cudaSuccess) {  // (the legacy stream beside another stream's capture)
+        cudaGetLastError();
+        return false;
+    }
+    return status == cudaStreamCaptureStatusActive;
+}
+
 // Launch description of one fused time step.
 struct StepLaunch {
     int storage;         // lee_storage
