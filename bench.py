@@ -47,14 +47,20 @@ KERNEL_SOURCES = ["paper_1601_08103_gb300/csrc/kernels.cuh", "paper_1601_08103_g
                   "paper_1601_08103_gb300/csrc/step_launch.cuh", "paper_1601_08103_gb300/csrc/velsets.cuh"]
 
 
-def steps_of_launch(sv, tma: bool = False) -> int:
-    """Time steps per launch of a long run in the default configuration: grids that fuse runs of steps take two
-    such runs in one launch (BFP16 and the TMA-fed tile one), large FP32 grids of the sets with diagonal velocities
-    two steps (steps_per_launch gives 1 for them)."""
-    spl = max(sv.steps_per_launch, 1)
-    if sv.set_name in ("D3Q9", "D3Q13", "D3Q19") and sv.storage == "f32" and sv.cells >= 1 << 22:
-        return 2
-    return spl if spl == 1 or sv.storage == "bfp16" or tma else 2 * spl
+def launch_bytes(lee, name: str, storage: str) -> float:
+    """Bytes per cell that a step launch reads and writes: the populations that a step changes, in both state copies.
+    (The sets with one moving shell, all but D3Q19, leave the rest population alone.)"""
+    info = lee.lee_velset_info(name)
+    if storage == "split16":
+        return 2 * lee.state_bytes_per_cell(info["D"], info["q"], storage)
+    shells = {sum(x * x for x in c) for c in info["c"]} - {0}
+    return 2 * (info["q"] - (len(shells) == 1)) * lee.STORAGE_BYTES[storage]
+
+
+def traffic_of(nbytes: float, cells: int, steps: int, launches: int, ms: float) -> dict:
+    """Steps per launch, algorithmic bytes per update and algorithmic GB/s of a run."""
+    return {"steps_per_launch": round(steps / launches, 2), "bytes_per_update": round(nbytes * launches / steps, 3),
+            "gbs": round(nbytes * cells * launches / (ms / 1e3) / 1e9, 1)}
 
 
 def kernel_source_sha() -> str:
@@ -222,8 +228,8 @@ def run_ours(args, rank, world, local):
 
     # a job of NSTEPS steps is NSTEPS // spl launches of spl steps, and one of the rest; every launch
     # reads and writes the moving populations once
-    spl = steps_of_launch(sv)
-    step_launches = -(-NSTEPS // spl)
+    step_launches = sv.run_launches(NSTEPS)
+    spl = -(-NSTEPS // step_launches)
     launches_per_step = 1 + step_launches + 1 + 2  # init, steps, moments, reduce (partial + final)
 
     def one_step(ev):
@@ -415,14 +421,12 @@ def forms_3d():
             sv.moments(r, None, None)
             torch.cuda.synchronize()
             ms = e0.elapsed_time(e1)
-            spl = steps_of_launch(sv, tma=label.endswith("tma_tile"))
+            launches = sv.run_launches(steps)
         if label == "f64":
             ref = r
         err = float(torch.linalg.norm(r - ref) / torch.linalg.norm(ref))
-        bpl = 2 * 6 * lee.STORAGE_BYTES[storage]
-        out[label] = {"mlups": round(cells * steps / (ms / 1e3) / 1e6, 1),
-                        "gbs": round(bpl * cells * steps / (ms / 1e3) / 1e9, 1), "rel_l2_rho_vs_f64": err,
-                        "steps_per_launch": spl, "bytes_per_update": round(bpl / max(spl, 1), 3)}
+        out[label] = {"mlups": round(cells * steps / (ms / 1e3) / 1e6, 1), "rel_l2_rho_vs_f64": err,
+                      **traffic_of(launch_bytes(lee, "D3Q7", storage), cells, steps, launches, ms)}
     for label in ("f16", "bf16", "bfp16", "f32_tma_tile", "bfp16_tma_tile"):
         out[label]["mlups_gain_vs_f32"] = round(out[label]["mlups"] / out["f32"]["mlups"], 3)
     return {"workload": "3D D3Q7 periodic 384^3, tau=0.55, pulse A=1e-3 w=16, 500 steps", "storage": out,
@@ -483,13 +487,11 @@ def forms_mixed_2d(n: int = 8192, steps: int = 1000):
             sv.moments(r, None, None)
             torch.cuda.synchronize()
             ms = e0.elapsed_time(e1)
-            spl = steps_of_launch(sv)
+            launches = sv.run_launches(steps)
         if ref is None:
             ref = r
-        bpl = 2 * 4 * lee.STORAGE_BYTES[storage]
-        out[storage] = {"mlups": round(cells * steps / (ms / 1e3) / 1e6, 1), "steps_per_launch": spl,
-                        "bytes_per_update": round(bpl / spl, 3),
-                        "gbs_algorithmic_per_launch": round(bpl * cells * steps / spl / (ms / 1e3) / 1e9, 1),
+        out[storage] = {"mlups": round(cells * steps / (ms / 1e3) / 1e6, 1),
+                        **traffic_of(launch_bytes(lee, "D2Q5", storage), cells, steps, launches, ms),
                         "rel_l2_rho_vs_f64": float(torch.linalg.norm(r - ref) / torch.linalg.norm(ref))}
         del r
         torch.cuda.empty_cache()
@@ -552,12 +554,10 @@ def forms_configs():
             torch.cuda.synchronize()
             ms = e0.elapsed_time(e1)
             finite = sv.check_finite()
-            spl = steps_of_launch(sv)
-        bpl = 2 * info["q"] * lee.STORAGE_BYTES[storage]
+            launches = sv.run_launches(steps)
         out[key] = {"cells": cells, "steps": steps, "ms": round(ms, 3), "us_per_step": round(ms * 1e3 / steps, 3),
                     "mlups": round(cells * steps / (ms / 1e3) / 1e6, 1),
-                    "gbs": round(bpl * cells * steps / (ms / 1e3) / 1e9, 1), "bytes_per_lup": bpl,
-                    "steps_per_launch": spl, "finite": bool(finite)}
+                    **traffic_of(launch_bytes(lee, name, storage), cells, steps, launches, ms), "finite": bool(finite)}
         torch.cuda.empty_cache()
     # the measured FP64 fma rate: the roofline of the FP64 storage forms, whose collision is FP64
     out["fp64_fma_peak"] = {"tflops": round(lee.lee_probe_fp64_fma(1 << 16) / 1e12, 4),
@@ -623,11 +623,12 @@ def forms_split():
             sv.moments(r, None, None)
             torch.cuda.synchronize()
             ms = e0.elapsed_time(e1)
+            launches = sv.run_launches(steps)
         if ref is None:
             ref = r
         bpc = lee.state_bytes_per_cell(3, info["q"], storage)
-        out[storage] = {"mlups": round(cells * steps / (ms / 1e3) / 1e6, 1),
-                        "gbs": round(2 * bpc * cells * steps / (ms / 1e3) / 1e9, 1), "bytes_per_cell_copy": bpc,
+        out[storage] = {"mlups": round(cells * steps / (ms / 1e3) / 1e6, 1), "bytes_per_cell_copy": bpc,
+                        **traffic_of(launch_bytes(lee, name, storage), cells, steps, launches, ms),
                         "rel_l2_rho_vs_f64": float(torch.linalg.norm(r - ref) / torch.linalg.norm(ref))}
     return {"workload": "3D D3Q19 periodic 256^3, tau=0.55, pulse A=1e-3 w=16, 200 steps", "storage": out}
 
@@ -742,11 +743,12 @@ def forms_batched(steps: int = 1000):
                 off += nx * ny
             torch.cuda.synchronize()
             shape = b.tune() if mode != "sequential" else None
+            launches = steps if mode == "sequential" else b.run_launches(steps)
             if mode == "graph" and storage == "f32":
                 out_shape = b.tune_shape()
         key = f"{storage}_{mode}"
         out[key] = {"mlups": round(cells * steps / (ms / 1e3) / 1e6, 1), "ms": round(ms, 3),
-                    "gbs": round(2 * 5 * lee.STORAGE_BYTES[storage] * cells * steps / (ms / 1e3) / 1e9, 1)}
+                    **traffic_of(launch_bytes(lee, "D2Q5", storage), cells, steps, launches, ms)}
         if shape:
             out[key]["tuned_threads_cells_per_thread"] = list(shape)
         rho_by[(storage, mode)] = rho
@@ -860,11 +862,10 @@ def run_case(args):
         torch.cuda.synchronize()
         ms = e0.elapsed_time(e1)
         ok = sv.check_finite()
-    q = lee.lee_velset_info(name)["q"]
-    bpl = 2 * lee.state_bytes_per_cell(D, q, storage)
+        launches = sv.run_launches(args.steps)
     print(json.dumps({"case": args.case, "cells": cells, "steps": args.steps, "ms": ms, "finite": ok,
                       "mlups": cells * args.steps / (ms / 1e3) / 1e6,
-                      "gbs": bpl * cells * args.steps / (ms / 1e3) / 1e9}), flush=True)
+                      **traffic_of(launch_bytes(lee, name, storage), cells, args.steps, launches, ms)}), flush=True)
     return 0 if ok else 1
 
 

@@ -51,8 +51,10 @@ lee_status lee_batch_init_fields(lee_batch *b, int32_t d, const double *rho, con
  * FP32 storage and every nx a multiple of 4, GRAPH and LAUNCH modes advance several steps per
  * launch (the intermediate states kept in registers; tiles of 112 columns), with the count,
  * tile rows and tile order the autotuner picks (lee_batch_tune_shape; LEE_TB_STEPS=1..4 in the
- * environment at create time fixes the count; a count of four that the tuner picked runs eight steps per
- * launch while a call has that many left), bit-identical to single steps. */
+ * environment at create time fixes the count; a count of four that the tuner picked or lee_batch_set_shape
+ * gave runs eight steps per launch while a call has that many left), bit-identical to single steps.
+ * While the caller captures the batch's stream into a graph of its own, a call is launched directly, in an
+ * even number of launches where eight steps can be split for it (see lee_lbm_step). */
 lee_status lee_batch_step(lee_batch *b, int64_t n, int32_t mode);
 
 /* Per-cell moments of domain d (as lee_lbm_moments).  NULL outputs are skipped. */
@@ -63,6 +65,10 @@ lee_status lee_batch_reduce(lee_batch *b, int32_t d, double *out, int32_t on_dev
 
 /* Post-collision populations of domain d as FP64 g[5][cells_d] (library velocity order). */
 lee_status lee_batch_get_populations(lee_batch *b, int32_t d, double *g, int32_t on_device);
+
+/* How many launches of the whole batch lee_batch_step(b, n, LEE_BATCH_GRAPH or LEE_BATCH_LAUNCH) takes with the launch
+ * shape in use (outside a capture; LEE_ERR_INVALID_ARGUMENT while there is none, see lee_batch_tune). */
+lee_status lee_batch_run_launches(lee_batch *b, int64_t n, int64_t *launches);
 
 /* Launch shape of a batch: the one-step batched kernel (threads per block, cells per thread) and
  * the fused multi-step kernel (steps per launch; tiles of 112 columns x tile_rows rows; dispatch

@@ -313,6 +313,10 @@ lee_status lee_lbm_steps_done(lee_lbm *h, int64_t *steps);
  * (see lee_lbm_step). */
 lee_status lee_lbm_steps_per_launch(lee_lbm *h, int32_t *steps);
 
+/* How many launches lee_lbm_step(h, n) takes outside a capture: each reads the current copy of the populations that a
+ * step changes and writes the other one (a step of the learned edge counts as one). */
+lee_status lee_lbm_run_launches(lee_lbm *h, int64_t n, int64_t *launches);
+
 /* The 16-bit storage scale S in use (1 for F64/F32/BFP16 storage). */
 lee_status lee_lbm_store_scale(lee_lbm *h, double *scale);
 

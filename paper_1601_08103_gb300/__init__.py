@@ -95,6 +95,7 @@ _SIGS = {
     "lee_lbm_slab_step": (ctypes.c_int, [_P, _I32, _I64]),
     "lee_lbm_store_scale": (ctypes.c_int, [_P, ctypes.POINTER(_D)]),
     "lee_lbm_steps_per_launch": (ctypes.c_int, [_P, ctypes.POINTER(_I32)]),
+    "lee_lbm_run_launches": (ctypes.c_int, [_P, _I64, ctypes.POINTER(_I64)]),
     "lee_lbm_sync": (ctypes.c_int, [_P]),
     "lee_lbm_last_error": (ctypes.c_char_p, [_P]),
     "lee_lbm_destroy": (ctypes.c_int, [_P]),
@@ -111,6 +112,7 @@ _SIGS = {
     "lee_batch_get_populations": (ctypes.c_int, [_P, _I32, _P, _I32]),
     "lee_batch_tune": (ctypes.c_int, [_P, ctypes.POINTER(_I32), ctypes.POINTER(_I32)]),
     "lee_batch_set_tuning": (ctypes.c_int, [_P, _I32, _I32]),
+    "lee_batch_run_launches": (ctypes.c_int, [_P, _I64, ctypes.POINTER(_I64)]),
     "lee_batch_tune_shape": (ctypes.c_int, [_P, _P]),
     "lee_batch_set_shape": (ctypes.c_int, [_P, _P]),
     "lee_batch_cells": (ctypes.c_int, [_P, ctypes.POINTER(_I64)]),
@@ -346,6 +348,12 @@ def lee_lbm_steps_per_launch(h) -> int:
     return v.value
 
 
+def lee_lbm_run_launches(h, n: int) -> int:
+    v = _I64()
+    _check(_lib.lee_lbm_run_launches(h, int(n), ctypes.byref(v)), "lee_lbm_run_launches", h)
+    return v.value
+
+
 def lee_lbm_store_scale(h) -> float:
     v = _D()
     _check(_lib.lee_lbm_store_scale(h, ctypes.byref(v)), "lee_lbm_store_scale")
@@ -522,6 +530,9 @@ class Solver:
     def steps_per_launch(self) -> int:
         return lee_lbm_steps_per_launch(self.h)
 
+    def run_launches(self, n: int) -> int:
+        return lee_lbm_run_launches(self.h, n)
+
     def sync(self):
         lee_lbm_sync(self.h)
 
@@ -620,6 +631,12 @@ def lee_batch_set_shape(b, threads: int, cells_per_thread: int, steps_per_launch
     _check(_lib.lee_batch_set_shape(b, ctypes.byref(sh)), "lee_batch_set_shape", batch=b)
 
 
+def lee_batch_run_launches(b, n: int) -> int:
+    v = _I64()
+    _check(_lib.lee_batch_run_launches(b, int(n), ctypes.byref(v)), "lee_batch_run_launches", batch=b)
+    return v.value
+
+
 def lee_batch_cells(b) -> int:
     v = _I64()
     _check(_lib.lee_batch_cells(b, ctypes.byref(v)), "lee_batch_cells")
@@ -670,6 +687,9 @@ class Batch:
 
     def set_shape(self, threads, cells_per_thread, steps_per_launch, tile_rows=64, tile_order=0):
         lee_batch_set_shape(self.b, threads, cells_per_thread, steps_per_launch, tile_rows, tile_order)
+
+    def run_launches(self, n: int) -> int:
+        return lee_batch_run_launches(self.b, n)
 
     @property
     def cells(self) -> int:

@@ -413,6 +413,16 @@ int next_launch(const lee_batch *b, int64_t left) {
     if (b->unit > 1 && b->deep_fn && left >= kRpDeep) return kRpDeep;
     return left >= b->unit ? b->unit : 1;
 }
+int64_t run_launches(const lee_batch *b, int64_t steps) {
+    int64_t c = 0;
+    while (steps > 0) {
+        const int k = next_launch(b, steps);
+        const int64_t r = steps / k;  // as many of this size as fit
+        c += r;
+        steps -= r * k;
+    }
+    return c;
+}
 // One launch of k steps reading buffer src_which and writing the other one.
 cudaError_t launch_steps(lee_batch *b, int src_which, int k, cudaStream_t st) {
     const void *src = b->buf[src_which];
@@ -596,9 +606,8 @@ lee_status lee_batch_step(lee_batch *b, int64_t n, int32_t mode) {
     // In a graph that the caller captures, an even number of launches where it can be had (see lee_lbm_step).
     const bool captured = capturing(b->st);
     if (captured && next_launch(b, left) == kRpDeep) {
-        int count = 0;
-        for (int64_t r = left; r > 0; ++count) r -= next_launch(b, r);
-        for (int k = 0; (count & 1) && k < kRpDeep; k += b->unit) {
+        const bool odd = run_launches(b, left) & 1;
+        for (int k = 0; odd && k < kRpDeep; k += b->unit) {
             BCK(b, launch_steps(b, b->cur, b->unit, b->st), "batched launch");
             b->cur ^= 1;
             left -= b->unit;
@@ -608,8 +617,7 @@ lee_status lee_batch_step(lee_batch *b, int64_t n, int32_t mode) {
         // up to kMaxGraphSteps steps: one graph of all of them (one launch of the whole run); longer
         // runs: replays of a kChunkSteps graph
         const int64_t steps = left <= lee_batch::kMaxGraphSteps ? left : lee_batch::kChunkSteps;
-        int flips = 0;
-        for (int64_t r = steps; r > 0; flips ^= 1) r -= next_launch(b, r);
+        const int flips = (int)(run_launches(b, steps) & 1);
         while (steps > 1 && left >= steps) {
             cudaGraphExec_t ex = nullptr;
             if ((s = ensure_graph(b, b->cur, steps, &ex)) != LEE_OK) return s;
@@ -624,6 +632,13 @@ lee_status lee_batch_step(lee_batch *b, int64_t n, int32_t mode) {
         b->cur ^= 1;
         left -= k;
     }
+    return LEE_OK;
+}
+
+lee_status lee_batch_run_launches(lee_batch *b, int64_t n, int64_t *launches) {
+    if (!b) return LEE_ERR_INVALID_ARGUMENT;
+    if (n < 0 || !launches || !b->tuned) return bfail(b, LEE_ERR_INVALID_ARGUMENT, "run_launches: bad args or no launch shape");
+    *launches = run_launches(b, n);
     return LEE_OK;
 }
 

@@ -244,6 +244,18 @@ int next_launch(const lee_lbm *h, int unit, long long left) {
     return left >= unit ? unit : 1;
 }
 
+// Launches of a run of `steps` steps.
+int64_t run_launches(const lee_lbm *h, int unit, int64_t steps) {
+    int64_t c = 0;
+    while (steps > 0) {
+        const int k = next_launch(h, unit, steps);
+        const int64_t r = steps / k;  // as many of this size as fit
+        c += r;
+        steps -= r * k;
+    }
+    return c;
+}
+
 // Steps of the first of the launches that can stand for one of k steps, with the same bits, in an even number more or less
 // (all of this size but for the last): 0 where there are none.
 int split_launch(const lee_lbm *h, int unit, int k) {
@@ -743,16 +755,6 @@ lee_status lee_lbm_step(lee_lbm *h, int64_t n) {
         if (h->D == 3) return k == h->ops->deep3d ? h->ops->step3dk(L) : h->ops->step3d2(L);
         return h->ops->stepk(L, k);
     };
-    auto launches_of = [&](int64_t steps) {
-        int64_t c = 0;
-        while (steps > 0) {
-            const int k = next_launch(h, unit, steps);
-            const int64_t r = steps / k;  // as many of this size as fit
-            c += r;
-            steps -= r * k;
-        }
-        return c;
-    };
     auto run = [&](int k) -> lee_status {
         LEE_CK(h, launch(h->cur, k, h->st), "step launch");
         h->cur ^= 1;
@@ -760,7 +762,7 @@ lee_status lee_lbm_step(lee_lbm *h, int64_t n) {
         return LEE_OK;
     };
     int64_t left = n;
-    const int64_t count = launches_of(n);
+    const int64_t count = run_launches(h, unit, n);
     if (n >= 2 && (count >= kGraphMinLaunches || (count & 1)) && capturing(h->st)) {
         const int first = next_launch(h, unit, n), part = count & 1 ? split_launch(h, unit, first) : 0;
         for (int k = part ? first : 0; k > 0; k -= part) {
@@ -773,7 +775,7 @@ lee_status lee_lbm_step(lee_lbm *h, int64_t n) {
         // replay a kChunkGraphSteps graph.  Graphs are captured once per (starting copy, length) on a
         // private stream and replayed on the handle's stream.
         const int64_t steps = left <= kMaxGraphSteps ? left : kChunkGraphSteps;
-        const int flips = (int)(launches_of(steps) & 1);
+        const int flips = (int)(run_launches(h, unit, steps) & 1);
         while (left >= steps) {
             auto it = h->exec.find({h->cur, steps});
             cudaGraphExec_t ex = it == h->exec.end() ? nullptr : it->second;
@@ -1038,6 +1040,13 @@ lee_status lee_lbm_steps_done(lee_lbm *h, int64_t *steps) {
 lee_status lee_lbm_steps_per_launch(lee_lbm *h, int32_t *steps) {
     if (!h || !steps) return LEE_ERR_INVALID_ARGUMENT;
     *steps = onchip(h) ? 0 : fused_steps(h);
+    return LEE_OK;
+}
+
+lee_status lee_lbm_run_launches(lee_lbm *h, int64_t n, int64_t *launches) {
+    if (!h) return LEE_ERR_INVALID_ARGUMENT;
+    if (n < 0 || !launches) return fail(h, LEE_ERR_INVALID_ARGUMENT, "run_launches: bad args");
+    *launches = n >= 2 && (shifted(h) || onchip(h)) ? 1 : run_launches(h, fused_steps(h), n);
     return LEE_OK;
 }
 
