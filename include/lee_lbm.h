@@ -217,6 +217,9 @@ lee_status lee_lbm_init_fields(lee_lbm *h, const double *rho, const double *u, c
  *  - else a 1D grid (not BFP16) whose two population copies fit in shared memory (2 q nx sizeof(storage) <= 227 KB,
  *    e.g. D1Q3 FP64 up to 4843 cells) runs all n >= 2 steps in one launch: one block, or from
  *    512 cells a thread-block cluster of 8 blocks;
+ *  - a step neither reads nor writes the rest populations of the sets with one moving shell (all but D3Q19; a sponge
+ *    frame damps those of its cells): one that is not finite stays in its cell and is counted there by
+ *    lee_lbm_reduce, while a moving one spreads through the grid;
  *  - OPEN_LEARNED: one launch per step whose first blocks run the boundary network and write the
  *    border cells (pulled with the network's entering populations and collided) while the other
  *    blocks step the interior cells; LEE_LEARNED_STREAMS=1 in the environment at create time runs
