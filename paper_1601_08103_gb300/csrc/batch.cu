@@ -257,6 +257,8 @@ lee_status apply_shape(lee_batch *b, const BatchShape &sh) {
 std::mutex g_cache_mutex;
 std::map<std::string, BatchShape> g_cache;
 
+// The first word names the kernels that a shape was measured on (batch2: tiles of 128 columns through shared memory), so
+// that a file written before they changed is measured anew.
 std::string cache_key(const lee_batch *b) {
     unsigned long long h = 1469598103934665603ULL;  // FNV-1a over the domain extents
     for (const auto &d : b->doms) {
@@ -268,7 +270,7 @@ std::string cache_key(const lee_batch *b) {
             }
     }
     std::ostringstream o;
-    o << "batch2/set" << b->set << "/st" << b->storage << "/n" << b->count << "/c" << b->total_cells << "/u"
+    o << "batch3/set" << b->set << "/st" << b->storage << "/n" << b->count << "/c" << b->total_cells << "/u"
       << b->unit_fixed << "/h" << std::hex << h;
     return o.str();
 }
