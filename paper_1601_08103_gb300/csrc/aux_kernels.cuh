@@ -306,32 +306,20 @@ __global__ void k_sponge_damp(T *__restrict__ g, T *__restrict__ other, GridDesc
     }
 }
 
-// Per-shell sums of one cell's stored populations: P[slot] = sum g, J[slot][a] = sum c_a g (in
-// stored units), Sq[slot] = sum g^2, and whether every value is finite.  Velocities 2k-1 and 2k are
-// opposite, so every pair gives one sum and one difference.
+// Per-shell sums of one cell's stored populations in FP64: P[slot] = sum g, J[slot][a] = sum c_a g (in stored units).
+// Velocities 2k-1 and 2k are opposite, so every pair gives one sum and one difference.
 template <class S, class T>
-__device__ __forceinline__ bool shell_sums(const T *__restrict__ g, long long pitch, long long x,
-                                           double (&P)[n_shells<S>()], double (&J)[n_shells<S>()][3],
-                                           double (&Sq)[n_shells<S>()]) {
-    bool finite = true;
-    static_for<n_shells<S>()>([&](auto K) {
-        constexpr int k = decltype(K)::value;
-        P[k] = -0.0;  // the first addition folds away
-        Sq[k] = 0.0;
-        J[k][0] = J[k][1] = J[k][2] = -0.0;
-    });
-    const double rest = (double)load_elem<S, T>(g, pitch, x);
-    finite = isfinite(rest);
-    P[shell_slot<S>(0)] = rest;
-    Sq[shell_slot<S>(0)] = rest * rest;
+__device__ __forceinline__ void shell_sums(const T *__restrict__ g, long long pitch, long long x,
+                                           double (&P)[n_shells<S>()], double (&J)[n_shells<S>()][3]) {
+#pragma unroll
+    for (int k = 0; k < n_shells<S>(); ++k) P[k] = J[k][0] = J[k][1] = J[k][2] = -0.0;  // the first addition folds away
+    P[shell_slot<S>(0)] = (double)load_elem<S, T>(g, pitch, x);
     static_for<S::Q / 2>([&](auto H) {
         constexpr int i = 1 + 2 * decltype(H)::value;
         constexpr int k = shell_slot<S>(S::shell(i));
         const double v = (double)load_elem<S, T>(g, pitch, (long long)i * pitch + x);
         const double o = (double)load_elem<S, T>(g, pitch, (long long)(i + 1) * pitch + x);
-        finite = finite && isfinite(v) && isfinite(o);
         P[k] += v + o;
-        Sq[k] = fma(o, o, fma(v, v, Sq[k]));
         const double d = v - o;
         static_for<3>([&](auto A) {
             constexpr int a = decltype(A)::value;
@@ -339,7 +327,6 @@ __device__ __forceinline__ bool shell_sums(const T *__restrict__ g, long long pi
             if constexpr (S::c(i, a) == -1) J[k][a] -= d;
         });
     });
-    return finite;
 }
 
 // Sums of values that are FP32 numbers (every storage but FP64) on the integer pipe.  With E the largest biased
@@ -540,8 +527,8 @@ __global__ void k_moments(const T *__restrict__ g, long long cells, long long pi
             }
         }
         if (!done) {
-            double Js[NS][3], Sq[NS];
-            shell_sums<S, T>(g, pitch, x, P, Js, Sq);
+            double Js[NS][3];
+            shell_sums<S, T>(g, pitch, x, P, Js);
             total = -0.0;
 #pragma unroll
             for (int s = 0; s < NS; ++s) total += P[s];

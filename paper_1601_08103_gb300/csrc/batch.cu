@@ -175,8 +175,8 @@ lee_status launch_one(lee_batch *b, int src_which, cudaStream_t st) {
 
 int full_vec(int storage) { return storage == LEE_STORE_F32 ? 4 : 2; }
 
-// Tile rows of the fused kernel before tuning (on the 96-domain workload, hand-swept with the
-// four-step kernel: 64 rows 374 GLUPS, 48-80 rows 360-366, 128 rows 367, 256 rows 359).
+// Tile rows of the fused kernel before tuning (96 domains of 128^2 to 1024^2, eight steps per launch, GLUPS: 32 rows 1234,
+// 48 1290, 64 1340, 96 1335, 128 1283, 256 1177).
 constexpr int kBatchTileRows = 64;
 
 // Tiles of kRpBatchWidth columns x `rows` rows (fewer for short domains), in dispatch order

@@ -458,36 +458,36 @@ __device__ __forceinline__ void collide_shells_pair(const float (&g)[S::Q][V], f
 template <class S, int K, int V>
 __device__ __forceinline__ void collide_axis_pair(const float (&g)[S::Q][V], float (&out)[S::Q][V],
                                                   const CollideCoef<float> &cf) {
-            const float w = cf.M[1][1];
-            auto in = [&](int i) { return make_float2(g[i][K], g[i][K + 1]); };
-            auto put = [&](int i, float c, float2 t) {
-                const float2 r = __ffma2_rn(splat2(c), t, in(i));
-                out[i][K] = r.x;
-                out[i][K + 1] = r.y;
-            };
-            if constexpr (S::D == 1) {
-    #pragma unroll
-                for (int i = 1; i < 3; ++i) {
-                    out[i][K] = g[i][K];
-                    out[i][K + 1] = g[i][K + 1];
-                }
-            } else if constexpr (S::D == 2) {
-                const float2 d = __fadd2_rn(__fadd2_rn(in(3), in(4)), neg2(__fadd2_rn(in(1), in(2))));
-                put(1, w, d);
-                put(2, w, d);
-                put(3, -w, d);
-                put(4, -w, d);
-            } else {
-                const float2 sx = __fadd2_rn(in(1), in(2)), sy = __fadd2_rn(in(3), in(4)), sz = __fadd2_rn(in(5), in(6));
-                const float2 P = __fadd2_rn(__fadd2_rn(sx, sy), sz), m3 = splat2(-3.0f);
-                const float2 tx = __ffma2_rn(m3, sx, P), ty = __ffma2_rn(m3, sy, P), tz = __ffma2_rn(m3, sz, P);
-                put(1, w, tx);
-                put(2, w, tx);
-                put(3, w, ty);
-                put(4, w, ty);
-                put(5, w, tz);
-                put(6, w, tz);
-            }
+    const float w = cf.M[1][1];
+    auto in = [&](int i) { return make_float2(g[i][K], g[i][K + 1]); };
+    auto put = [&](int i, float c, float2 t) {
+        const float2 r = __ffma2_rn(splat2(c), t, in(i));
+        out[i][K] = r.x;
+        out[i][K + 1] = r.y;
+    };
+    if constexpr (S::D == 1) {
+#pragma unroll
+        for (int i = 1; i < 3; ++i) {
+            out[i][K] = g[i][K];
+            out[i][K + 1] = g[i][K + 1];
+        }
+    } else if constexpr (S::D == 2) {
+        const float2 d = __fadd2_rn(__fadd2_rn(in(3), in(4)), neg2(__fadd2_rn(in(1), in(2))));
+        put(1, w, d);
+        put(2, w, d);
+        put(3, -w, d);
+        put(4, -w, d);
+    } else {
+        const float2 sx = __fadd2_rn(in(1), in(2)), sy = __fadd2_rn(in(3), in(4)), sz = __fadd2_rn(in(5), in(6));
+        const float2 P = __fadd2_rn(__fadd2_rn(sx, sy), sz), m3 = splat2(-3.0f);
+        const float2 tx = __ffma2_rn(m3, sx, P), ty = __ffma2_rn(m3, sy, P), tz = __ffma2_rn(m3, sz, P);
+        put(1, w, tx);
+        put(2, w, tx);
+        put(3, w, ty);
+        put(4, w, ty);
+        put(5, w, tz);
+        put(6, w, tz);
+    }
 }
 
 template <class S, int K, int V>

@@ -78,12 +78,12 @@ __global__ void __launch_bounds__(32 * kMlpWarps) k_mlp_forward(MlpDev WG, const
     const MlpDev W = stage_forward_weights(WG, wsm);  // ends with a block barrier
     uint32_t ax[4];
     a_frag_from_tile(tile[warp], ax);
-    MlpFwd F;
-    mlp_forward_warp(W, ax, F);
+    float y_lo, y_hi;
+    mlp_forward_warp(W, ax, y_lo, y_hi);
     const int g = lane >> 2, t = lane & 3;
     if (t == 0) {
-        if (row0 + g < rows) y[row0 + g] = F.y_lo;
-        if (row0 + g + 8 < rows) y[row0 + g + 8] = F.y_hi;
+        if (row0 + g < rows) y[row0 + g] = y_lo;
+        if (row0 + g + 8 < rows) y[row0 + g + 8] = y_hi;
     }
 }
 

@@ -65,59 +65,43 @@ __device__ __forceinline__ uint32_t ldw(const __nv_bfloat16 *p) { return *reinte
 
 __device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
 
-// Forward pass of one warp's 16 rows.  ax: A fragment of the input (BF16).  Outputs the two
-// rows' results in lanes with t == 0 (y_lo for row g, y_hi for row g + 8), plus, when the
-// pointers are given, the FP32 pre-activations z1, z2 in C-fragment layout.
-struct MlpFwd {
-    float z1[8][4];
-    float z2[8][4];
-    uint32_t h1[8][2];  // BF16 pairs: [tile][0] = row g, [tile][1] = row g + 8 (cols 8j+2t..)
-    uint32_t h2[8][2];
-    float y_lo, y_hi;
-};
-
-__device__ __forceinline__ void mlp_forward_warp(const MlpDev &W, const uint32_t (&ax)[4], MlpFwd &F) {
+// Forward pass of one warp's 16 rows.  ax: A fragment of the input (BF16).  The rows' results, in lanes with t == 0: y_lo for
+// row g, y_hi for row g + 8.
+__device__ __forceinline__ void mlp_forward_warp(const MlpDev &W, const uint32_t (&ax)[4], float &y_lo, float &y_hi) {
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    uint32_t h1[8][2], h2[8][2];  // BF16 pairs: [tile][0] = row g, [tile][1] = row g + 8 (cols 8j+2t..)
+    auto activate = [&](float (&z)[4], const float *b, int j, uint32_t (&h)[2]) {
+        const float bb0 = b[8 * j + 2 * t], bb1 = b[8 * j + 2 * t + 1];
+        h[0] = pack_bf16(gelu(z[0] + bb0), gelu(z[1] + bb1));
+        h[1] = pack_bf16(gelu(z[2] + bb0), gelu(z[3] + bb1));
+    };
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-        F.z1[j][0] = F.z1[j][1] = F.z1[j][2] = F.z1[j][3] = 0.f;
+        float z[4] = {0.f, 0.f, 0.f, 0.f};
         const __nv_bfloat16 *w = W.w1 + (8 * j + g) * kMlpIn + 2 * t;
-        mma16816(F.z1[j], ax, ldw(w), ldw(w + 8));
-        const float bb0 = W.b1[8 * j + 2 * t], bb1 = W.b1[8 * j + 2 * t + 1];
-        F.z1[j][0] += bb0;
-        F.z1[j][1] += bb1;
-        F.z1[j][2] += bb0;
-        F.z1[j][3] += bb1;
-        F.h1[j][0] = pack_bf16(gelu(F.z1[j][0]), gelu(F.z1[j][1]));
-        F.h1[j][1] = pack_bf16(gelu(F.z1[j][2]), gelu(F.z1[j][3]));
+        mma16816(z, ax, ldw(w), ldw(w + 8));
+        activate(z, W.b1, j, h1[j]);
     }
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-        F.z2[j][0] = F.z2[j][1] = F.z2[j][2] = F.z2[j][3] = 0.f;
+        float z[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
-            const uint32_t a[4] = {F.h1[2 * kk][0], F.h1[2 * kk][1], F.h1[2 * kk + 1][0], F.h1[2 * kk + 1][1]};
+            const uint32_t a[4] = {h1[2 * kk][0], h1[2 * kk][1], h1[2 * kk + 1][0], h1[2 * kk + 1][1]};
             const __nv_bfloat16 *w = W.w2 + (8 * j + g) * kMlpHid + 16 * kk + 2 * t;
-            mma16816(F.z2[j], a, ldw(w), ldw(w + 8));
+            mma16816(z, a, ldw(w), ldw(w + 8));
         }
-        const float bb0 = W.b2[8 * j + 2 * t], bb1 = W.b2[8 * j + 2 * t + 1];
-        F.z2[j][0] += bb0;
-        F.z2[j][1] += bb1;
-        F.z2[j][2] += bb0;
-        F.z2[j][3] += bb1;
-        F.h2[j][0] = pack_bf16(gelu(F.z2[j][0]), gelu(F.z2[j][1]));
-        F.h2[j][1] = pack_bf16(gelu(F.z2[j][2]), gelu(F.z2[j][3]));
+        activate(z, W.b2, j, h2[j]);
     }
     float z3[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) {
-        const uint32_t a[4] = {F.h2[2 * kk][0], F.h2[2 * kk][1], F.h2[2 * kk + 1][0], F.h2[2 * kk + 1][1]};
+        const uint32_t a[4] = {h2[2 * kk][0], h2[2 * kk][1], h2[2 * kk + 1][0], h2[2 * kk + 1][1]};
         const __nv_bfloat16 *w = W.w3 + g * kMlpHid + 16 * kk + 2 * t;
         mma16816(z3, a, ldw(w), ldw(w + 8));
     }
-    const float b3 = W.b3[0];
-    F.y_lo = z3[0] + b3;  // column 0 lives in lanes with t == 0
-    F.y_hi = z3[2] + b3;
+    y_lo = z3[0] + W.b3[0];  // column 0 lives in lanes with t == 0
+    y_hi = z3[2] + W.b3[0];
 }
 
 // Copies the forward weights (w1, w2, w3 and the biases: packed bytes [0, kPkW2T) and

@@ -1,7 +1,7 @@
 // step_launch.cuh -- launch configuration of the fused stream-collide kernels for one velocity set:
-// the one-step kernel (cells per thread, grid) the 2D row pipeline (segment height from the
-// resident capacity) and the 3D plane pipeline (tiles and segments likewise).  Together with kernels.cuh and velsets.cuh this fixes what the
-// profiled hot-path launches execute.
+// the one-step kernel (cells per thread, grid), the 2D row pipeline (segment height from the
+// resident capacity) and the 3D plane pipelines (tiles and segments likewise).  Together with
+// kernels.cuh, rowpipe.cuh and velsets.cuh this fixes what the profiled hot-path launches execute.
 #pragma once
 
 #include "ops.cuh"
