@@ -310,10 +310,10 @@ __device__ __forceinline__ void stream_collide_chunk_bfp(const Bfp16 *__restrict
     });
 }
 
-// One block of 256 threads per 2048 cells; three blocks per SM at 78 registers (D3Q7, 8 cells per
+// One block of 256 threads per 2048 cells; three blocks per SM at 72 registers (D3Q7, 8 cells per
 // lane).  The kernel is bound by instruction issue (four blocks per SM at 64 registers: the same
-// time), so decoding and encoding cost it against FP16: D3Q7 384^3 at 196 GLUPS, 5.8 TB/s in
-// algorithmic bytes, against 251 GLUPS for FP16.
+// time), so decoding and encoding cost it against FP16: D3Q7 384^3 at 231 GLUPS, 5.9 TB/s in
+// algorithmic bytes, against 292 GLUPS for FP16.
 template <class S, int V, Edge EDGE>
 __global__ void __launch_bounds__(256) k_stream_collide_bfp(const Bfp16 *__restrict__ src, Bfp16 *__restrict__ dst,
                                                             GridDesc gd, CollideCoef<float> cf, OpenEdge<float> ob) {

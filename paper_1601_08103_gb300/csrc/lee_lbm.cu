@@ -225,9 +225,9 @@ bool ragged_2d(const lee_lbm *h) {
 // bits of two launches; BFP16 would need wider halos for that and stays on units), and FP32 ones the two
 // or three that remain in one launch too (a 16-bit state would be rounded at other steps); 3D grids on the
 // plane pipeline take kPpDeep.  3D FP32 grids of fewer than kFuse3dCells cells take single steps: their few
-// tiles leave SMs idle in either fused kernel (us per step of one / two / four steps per launch: 64^3 2.5 /
-// 3.7 / 2.9, 80^3 3.7 / 4.8 / 3.8, 96^3 4.8 / 5.9 / 4.1, 128^3 - / 10.2 / 7.2; widths that are not multiples of 4,
-// copied word by word, 97x99x98 8.2 / - / 8.4, 193x161x135 33.7 / - / 27.1).
+// tiles leave SMs idle in either fused kernel (us per step of one / two / four steps per launch: 64^3 2.4 /
+// 3.6 / 2.7, 80^3 3.6 / 4.7 / 3.4, 96^3 4.7 / 5.8 / 4.1, 128^3 9.9 / 10.1 / 7.2; widths that are not multiples of 4,
+// copied word by word, 97x99x98 8.1 / - / 8.0, 129x127x125 16.3 / - / 13.8, 193x161x135 33.4 / - / 25.3).
 // 2D FP32 at such widths: 2047x2045 160 GLUPS with single steps, 920 on the row pipeline.
 // Measured on GB300, GLUPS: D2Q5 FP32 2048^2 / 8192^2 four steps per launch 740 / 811, eight 1490 / 1611; D3Q7
 // FP32 384^3 / 256^3 two 259 / 232, four 426 / 373.

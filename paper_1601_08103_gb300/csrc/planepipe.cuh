@@ -25,7 +25,8 @@
 //
 // What bounds it: K = 4 moves 12 bytes of DRAM per FP32 update, 0.76 of the measured copy on D3Q7 384^3 (426
 // GLUPS, 256^3 373; the two-step tile of tb3d.cuh 259, one step per launch 147); a third of the computed cells are halo,
-// and the warps wait for the barrier and the shared-memory queue (12 warps per SM at 152 registers).
+// and the warps wait for the shared-memory queue (2.5 of 8.5 cycles per issue; the barrier 0.7) with 12 warps per SM at 164
+// registers, issue slots 35 % busy (256^3).
 // Refilled before the barrier, with the end lanes' words copied into slots of their own, 385 / 346.
 // Measured on 384^3 / 256^3 with the refill before the barrier and not taken: a row of 128 columns per warp with the +-y of S(t) in
 // registers (260 / 219); two rows per thread, 256 threads (352 / 345) or 384 (spills, 312 / 287); three

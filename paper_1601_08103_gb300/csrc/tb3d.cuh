@@ -4,7 +4,7 @@
 // LEE_TB_STEPS=2 asks for it, and for BFP16 storage (bfp.cuh; level 1 then stays in FP32,
 // so a launch rounds to the storage once) when LEE_TB_STEPS=2 asks for it: with FP16/BF16, and with
 // BFP16's decoding and encoding, this latency-bound tile measured slower than the one-step kernel
-// (below; BFP16 on D3Q7 384^3: 124 against 196 GLUPS).
+// (below; BFP16 on D3Q7 256^3: 145 against 229 GLUPS).
 //
 // A block of W = TY + 2 warps owns a tile of 128 columns x TY rows and marches through planes
 // z0 .. z0 + HZ - 1.  Warp w works on row y = y0 - 1 + w at both levels, lane L on the four
