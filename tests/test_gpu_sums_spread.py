@@ -20,6 +20,9 @@ def _sizes(kind, c, shape, rng):
         s[1:] = 1e-15
     elif kind == "denormal moving":
         s[1:] = 1e-39
+    elif kind == "all tiny":  # normal numbers below the integer form's range, and denormals
+        s *= 1e-30
+        s[:, ::3] = 1e-40
     elif kind == "tiny rest":
         s[0] = 1e-14
     elif kind == "last axis tiny":  # velocities along the last axis alone; only they carry its momentum in the axis sets
@@ -35,7 +38,7 @@ def _sizes(kind, c, shape, rng):
     return s
 
 
-@pytest.mark.parametrize("kind", ["tiny moving", "denormal moving", "tiny rest", "last axis tiny", "one cell in four",
+@pytest.mark.parametrize("kind", ["tiny moving", "denormal moving", "all tiny", "tiny rest", "last axis tiny", "one cell in four",
                                   "falling off", "edge of the integer form"])
 @pytest.mark.parametrize("storage", ["f32", "bf16", "bfp16"])
 @pytest.mark.parametrize("name,shape", SETS)
