@@ -187,9 +187,11 @@ lee_status lee_lbm_init_fields(lee_lbm *h, const double *rho, const double *u, c
  * collision kernel per step.  Asynchronous.  Calls of eight launches or more are replayed from a CUDA
  * graph (one graph holding all n steps for n <= 4096, else repeated 96-step graphs), captured on
  * first use of that length on a private stream and cached in the handle; results are identical to
- * direct launches.  While the caller captures the handle's stream into a graph of its own, the call is launched
- * directly, in an even number of launches where one gives the same bits (not for n = 1, and not where a 16-bit state would be
- * rounded at other steps); replays of a graph with an even number of launches advance the state by n steps each.  Every form below also gives the same bits as single one-step launches:
+ * direct launches.  While the caller captures the handle's stream into a graph of its own, the call is
+ * launched directly, in an even number of launches where one gives the same bits (not for n = 1, and not
+ * where a 16-bit state would be rounded at other steps); replays of a graph with an even number of
+ * launches advance the state by n steps each.  Every form below also gives the same
+ * bits as single one-step launches:
  *  - periodic 2D FP32 grids advance several steps per launch, the
  *    intermediate states kept in registers (temporal blocking): eight while the call has that many
  *    left, then four, then the two or three or one that remain.  LEE_TB_STEPS=1..4 in the

@@ -609,10 +609,11 @@ __device__ __forceinline__ void reduce_cell(const T *__restrict__ g, long long p
         }
     });
 }
-// Adds an FP64 state's values of N cells (one or four), `stride` apart.  A pair of opposite velocities
-// gives a sum and a difference, so that momentum adds up the differences, which may be far smaller than the populations; the
-// cells are added to one another before they reach the accumulator.  With one accumulator per velocity, and momentum from them at the
-// end, there would be a third fewer FP64 instructions, but momentum would carry the roundings of the populations' sums.
+// Adds an FP64 state's values of N cells (one or four), `stride` apart.  A pair of opposite velocities gives a sum
+// and a difference, so that momentum adds up the differences, which may be far smaller than the populations; the
+// cells are added to one another before they reach the accumulator.  With one accumulator per velocity, and
+// momentum from them at the end, there would be a third fewer FP64 instructions, but momentum would carry the
+// roundings of the populations' sums.  (D3Q7 384^3: 3.57 ms value by value, 2.06 so.)
 template <class S, int N>
 __device__ __forceinline__ void reduce_group(const double *__restrict__ g, long long pitch, long long x, long long stride,
                                              double (&acc)[reduce_nraw<S>()], int &bad) {
@@ -706,8 +707,8 @@ __host__ __device__ constexpr int reduce_min_blocks() {
     return S::Q <= 9 ? 3 : S::Q <= 13 ? 2 : 1;
 }
 template <class S, class T>
-__global__ void __launch_bounds__(kReduceThreads, reduce_min_blocks<S>()) k_reduce_partial(const T *__restrict__ g, long long cells, long long pitch,
-                                                                   double *__restrict__ partial) {
+__global__ void __launch_bounds__(kReduceThreads, reduce_min_blocks<S>())
+    k_reduce_partial(const T *__restrict__ g, long long cells, long long pitch, double *__restrict__ partial) {
     constexpr int NS = n_shells<S>(), D = S::D, NR = reduce_nraw<S>(), G = kReduceGroup;
     static_assert(NR <= kReduceMax, "raw accumulators do not fit");
     static_assert(G == 4 && fix_fits(G * most_in_shell<S>()), "integer sums of a group's shell");

@@ -243,11 +243,13 @@ __device__ __forceinline__ void stream_collide_chunk_bfp(const Bfp16 *__restrict
             if (zs < 0) { if constexpr (OPEN) row_out = true; else zs += gd.nz; }
             if (zs >= gd.nz) { if constexpr (OPEN) row_out = true; else zs -= gd.nz; }
         }
+        // (rows outside the grid: the cell's own is read for them, so that no load waits on a branch)
+        if constexpr (OPEN && cy != 0) ys = row_out ? y : ys;
+        if constexpr (OPEN && cz != 0) zs = row_out ? z : zs;
         const long long rowi = (long long)i * gd.pitch + ((long long)zs * gd.ny + ys) * gd.nx;
         C v[V];
-        if (!row_out) {
-            bfp_load_vec<V>(src + rowi + x0, sx + ((rowi + x0) >> 3), v);
-        } else {
+        bfp_load_vec<V>(src + rowi + x0, sx + ((rowi + x0) >> 3), v);
+        if (OPEN && (cy != 0 || cz != 0) && row_out) {
 #pragma unroll
             for (int k = 0; k < V; ++k) v[k] = C(0);
         }
@@ -261,9 +263,10 @@ __device__ __forceinline__ void stream_collide_chunk_bfp(const Bfp16 *__restrict
                 left = prev;
             } else {
                 int xs = x0 - 1;
-                bool out = row_out;
-                if (xs < 0) { if constexpr (OPEN) out = true; else xs += gd.nx; }
-                left = out ? C(0) : bfp_load1(src, sx, rowi + xs);
+                const bool out = xs < 0;
+                if (out) xs = OPEN ? x0 : xs + gd.nx;
+                left = bfp_load1(src, sx, rowi + xs);
+                if (OPEN && (out || row_out)) left = C(0);
             }
             pull[i][0] = left;
 #pragma unroll
@@ -275,9 +278,10 @@ __device__ __forceinline__ void stream_collide_chunk_bfp(const Bfp16 *__restrict
                 right = next;
             } else {
                 int xs = x0 + V;
-                bool out = row_out;
-                if (xs >= gd.nx) { if constexpr (OPEN) out = true; else xs -= gd.nx; }
-                right = out ? C(0) : bfp_load1(src, sx, rowi + xs);
+                const bool out = xs >= gd.nx;
+                if (out) xs = OPEN ? x0 : xs - gd.nx;
+                right = bfp_load1(src, sx, rowi + xs);
+                if (OPEN && (out || row_out)) right = C(0);
             }
 #pragma unroll
             for (int k = 0; k < V - 1; ++k) pull[i][k] = v[k + 1];
@@ -314,9 +318,17 @@ __device__ __forceinline__ void stream_collide_chunk_bfp(const Bfp16 *__restrict
 // lane).  The kernel is bound by instruction issue (four blocks per SM at 64 registers: the same
 // time), so decoding and encoding cost it against FP16: D3Q7 384^3 at 231 GLUPS, 5.9 TB/s in
 // algorithmic bytes, against 292 GLUPS for FP16.
+// Blocks per SM for which the compiler lays out the kernel (see step_min_blocks; us per step, its choice and the
+// bound: D2Q5 1024^2 frame 5.72 and 5.03; D3Q9 160^3 zero edge 42.3 and 35.7, frame 54.7 and 49.0).
 template <class S, int V, Edge EDGE>
-__global__ void __launch_bounds__(256) k_stream_collide_bfp(const Bfp16 *__restrict__ src, Bfp16 *__restrict__ dst,
-                                                            GridDesc gd, CollideCoef<float> cf, OpenEdge<float> ob) {
+__host__ __device__ constexpr int step_min_blocks_bfp() {
+    if (S::Q == 5 && EDGE == kFrameEdge) return 4;
+    return S::Q == 9 && V == 8 && EDGE != kWrapEdge ? (EDGE == kFrameEdge ? 2 : 3) : 0;
+}
+template <class S, int V, Edge EDGE>
+__global__ void __launch_bounds__(256, step_min_blocks_bfp<S, V, EDGE>())
+    k_stream_collide_bfp(const Bfp16 *__restrict__ src, Bfp16 *__restrict__ dst, GridDesc gd, CollideCoef<float> cf,
+                         OpenEdge<float> ob) {
     stream_collide_chunk_bfp<S, V, EDGE>(src, dst, gd, cf, ob, (long long)blockIdx.x * blockDim.x + threadIdx.x);
 }
 

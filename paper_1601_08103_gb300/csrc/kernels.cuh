@@ -176,7 +176,7 @@ struct CollideCoef {
 // What a step does at the edges of its grid: wraps around, lets zeros enter, damps a frame of cells too (sponge_w of
 // them), or lets the populations `ghost` enter (2D).  Every kind has its own instances of the step kernels: the launches of
 // open grids are short, and in one instance for all of them each paid for the others' code (D2Q5 FP32, us per step,
-// zero edge / frame: 137x197 2.21 / 2.62 in one instance, 1.56 / 1.85 so; 1024^2 4.87 / 6.20 and 4.01 / 4.64).
+// zero edge / frame: 137x197 2.21 / 2.62 in one instance, 1.42 / 1.59 so; 1024^2 4.87 / 6.20 and 3.93 / 4.30).
 enum Edge { kWrapEdge, kZeroEdge, kFrameEdge, kGhostEdge };
 template <class C>
 struct OpenEdge {
@@ -556,17 +556,14 @@ __device__ __forceinline__ void stream_collide_chunk(const T *__restrict__ src, 
     const bool has_left = (lane > 0) && (xc > 0);
     const bool has_right = (lane < 31) && (xc < gd.nxc - 1);
 
-    // the frame damps rest populations that a step leaves alone elsewhere
-    [[maybe_unused]] bool framed = false;
+    // The frame damps rest populations that a step leaves alone elsewhere.  In 2D those of the chunks that touch it are
+    // read, after the pulls (32x32 FP16 2.32 us per step; before them 2.75); in 3D, where a frame is most of a small
+    // grid, those of all, before the pulls (D3Q13 100^3 FP32 16.3; of the frame's chunks 17.2; after the pulls 17.4).
+    constexpr bool REST = EDGE == kFrameEdge && rest_static<S>();
     [[maybe_unused]] C rest[V];
-    auto load_rest = [&] {
-        if (framed) load_vec<T, V>(src + ((long long)z * gd.ny + y) * gd.nx + x0, rest);
-    };
-    if constexpr (EDGE == kFrameEdge && rest_static<S>()) {
-        framed = in_frame(x0, V, y, z, gd, S::D, ob);
-        // Before the pulls in 3D, after them in 2D (us per step: D3Q7 192^3 FP32 56.6 and 62.0; D2Q5 32x32 FP16 2.75 and 2.49).
-        if constexpr (S::D == 3) load_rest();
-    }
+    [[maybe_unused]] const bool framed = !REST || S::D == 3 || in_frame(x0, V, y, z, gd, S::D, ob);
+    auto load_rest = [&] { load_vec<T, V>(src + ((long long)z * gd.ny + y) * gd.nx + x0, rest); };
+    if constexpr (REST && S::D == 3) load_rest();
     C pull[S::Q][V];
     static_for_carried<S>([&](auto I) {
         constexpr int i = decltype(I)::value;
@@ -581,11 +578,13 @@ __device__ __forceinline__ void stream_collide_chunk(const T *__restrict__ src, 
             if (zs < 0) { if constexpr (OPEN) row_out = true; else zs += gd.nz; }
             if (zs >= gd.nz) { if constexpr (OPEN) row_out = true; else zs -= gd.nz; }
         }
+        // (rows outside the grid: the cell's own is read for them, so that no load waits on a branch)
+        if constexpr (OPEN && cy != 0) ys = row_out ? y : ys;
+        if constexpr (OPEN && cz != 0) zs = row_out ? z : zs;
         const T *rowp = src + (long long)i * gd.pitch + ((long long)zs * gd.ny + ys) * gd.nx;
         C v[V];
-        if (!row_out) {
-            load_vec<T, V>(rowp + x0, v);
-        } else {
+        load_vec<T, V>(rowp + x0, v);
+        if (OPEN && (cy != 0 || cz != 0) && row_out) {
 #pragma unroll
             for (int k = 0; k < V; ++k) v[k] = C(0);
             if constexpr (EDGE == kGhostEdge && cx == 0) {
@@ -606,11 +605,12 @@ __device__ __forceinline__ void stream_collide_chunk(const T *__restrict__ src, 
                 left = prev;
             } else {
                 int xs = x0 - 1;
-                bool out = row_out;
-                if (xs < 0) { if constexpr (OPEN) out = true; else xs += gd.nx; }
-                left = out ? C(0) : Store<T>::load(rowp[xs]);
+                const bool out = xs < 0;
+                if (out) xs = OPEN ? x0 : xs + gd.nx;
+                left = Store<T>::load(rowp[xs]);
+                if (OPEN && (out || row_out)) left = C(0);
                 if constexpr (EDGE == kGhostEdge && cy == 0) {
-                    if (xs < 0 && ob.ghost != nullptr) left = ob.ghost[0 * ob.ghost_L + y];
+                    if (out && ob.ghost != nullptr) left = ob.ghost[0 * ob.ghost_L + y];
                 }
             }
             pull[i][0] = left;
@@ -623,11 +623,12 @@ __device__ __forceinline__ void stream_collide_chunk(const T *__restrict__ src, 
                 right = next;
             } else {
                 int xs = x0 + V;
-                bool out = row_out;
-                if (xs >= gd.nx) { if constexpr (OPEN) out = true; else xs -= gd.nx; }
-                right = out ? C(0) : Store<T>::load(rowp[xs]);
+                const bool out = xs >= gd.nx;
+                if (out) xs = OPEN ? x0 : xs - gd.nx;
+                right = Store<T>::load(rowp[xs]);
+                if (OPEN && (out || row_out)) right = C(0);
                 if constexpr (EDGE == kGhostEdge && cy == 0) {
-                    if (x0 + V >= gd.nx && ob.ghost != nullptr) right = ob.ghost[1 * ob.ghost_L + y];
+                    if (out && ob.ghost != nullptr) right = ob.ghost[1 * ob.ghost_L + y];
                 }
             }
 #pragma unroll
@@ -636,22 +637,24 @@ __device__ __forceinline__ void stream_collide_chunk(const T *__restrict__ src, 
         }
     });
 
-    if constexpr (EDGE == kFrameEdge && rest_static<S>() && S::D < 3) load_rest();
+    if constexpr (REST && S::D < 3) {
+        if (framed) load_rest();
+    }
     C post[S::Q][V];
     // one cell at a time: this kernel streams at the memory bound, and the packed f32x2 pairs
     // (same bits) cost it 9 to 12 registers and occupancy
     collide_chunk<S, false>(pull, post, cf);
 
     if constexpr (EDGE == kFrameEdge) {
-        if (rest_static<S>() ? framed : ob.sponge_w > 0) {
+        if (REST ? framed : ob.sponge_w > 0) {
 #pragma unroll
             for (int k = 0; k < V; ++k) {
                 const C damp = sponge_factor<C>(x0 + k, y, z, gd, S::D, ob.sponge_w, ob.sponge_smax);
-                if constexpr (rest_static<S>()) rest[k] *= damp;
+                if constexpr (REST) rest[k] *= damp;
 #pragma unroll
-                for (int i = rest_static<S>() ? 1 : 0; i < S::Q; ++i) post[i][k] *= damp;
+                for (int i = REST ? 1 : 0; i < S::Q; ++i) post[i][k] *= damp;
             }
-            if (rest_static<S>() && active) store_vec<T, V>(dst + ((long long)z * gd.ny + y) * gd.nx + x0, rest);
+            if (REST && active) store_vec<T, V>(dst + ((long long)z * gd.ny + y) * gd.nx + x0, rest);
         }
     }
 
@@ -723,11 +726,26 @@ __global__ void __launch_bounds__(1024) k_onchip_1d(T *__restrict__ g, int nx, l
     for (int k = threadIdx.x; k < S::Q * nx; k += blockDim.x) g[(long long)(k / nx) * pitch + k % nx] = fin[k];
 }
 
+// Blocks per SM for which the compiler lays out the kernels of many registers; 0 is its own choice, which is right
+// elsewhere (a bound of one block makes it take many more).  us per step, its choice and the bound: D3Q13 FP16
+// 160^3 frame 97 and 52; D3Q13 FP32 160^3 zero edge 71 and 63; frames of D3Q7 FP16 160^3 28 and 23, of
+// D3Q9 FP32 160^3 57 and 52.
+template <class S, class T, int V, Edge EDGE>
+__host__ __device__ constexpr int step_min_blocks() {
+    int pulls = 0;  // registers of a thread's pulls
+    for (int i = 0; i < S::Q; ++i) pulls += carried<S>(i) ? V * (int)sizeof(typename Store<T>::C) / 4 : 0;
+    if (!rest_static<S>() || sizeof(T) == 8) return 0;
+    if (EDGE == kWrapEdge) return 0;
+    if (pulls > 64) return 2;
+    if (V == 8) return pulls > 32 ? 3 : 0;
+    return pulls > 32 ? (EDGE == kZeroEdge ? 4 : 0) : pulls == 32 && V == 4 && EDGE == kFrameEdge ? 4 : 0;
+}
+
 // One fused time step on one grid: one thread per V-cell chunk.
 template <class S, class T, int V, Edge EDGE, bool CUT = false>
-__global__ void __launch_bounds__(256) k_stream_collide(const T *__restrict__ src, T *__restrict__ dst, GridDesc gd,
-                                                        CollideCoef<typename Store<T>::C> cf,
-                                                        OpenEdge<typename Store<T>::C> ob) {
+__global__ void __launch_bounds__(256, step_min_blocks<S, T, V, EDGE>())
+    k_stream_collide(const T *__restrict__ src, T *__restrict__ dst, GridDesc gd, CollideCoef<typename Store<T>::C> cf,
+                     OpenEdge<typename Store<T>::C> ob) {
     stream_collide_chunk<S, T, V, EDGE, CUT>(src, dst, gd, cf, ob, (long long)blockIdx.x * blockDim.x + threadIdx.x);
 }
 

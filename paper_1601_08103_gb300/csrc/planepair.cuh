@@ -15,12 +15,13 @@
 // two iterations that store nothing.  Every operation is that of collide_shells_cell, so a launch gives the bits of
 // two single steps.
 //
-// What bounds it: the queue of memory instructions (D3Q19: 2.3 of 10.5 cycles per issue) and the one barrier per plane (1.3)
-// with 16 warps per SM at 128 registers; DRAM moves 76 bytes per D3Q19 update (152 with one step per launch).  us per step on 256^3, one
-// step per launch -> now: D3Q19 393 -> 281 (0.67 of the measured copy rate), D3Q13 235 -> 154, D3Q9 153 -> 116; 255x249x251
-// (4-byte accesses) 431 -> 292, 270 -> 157.  Measured on 256^3 (D3Q19 / D3Q13) and not taken: the cells of a lane in
-// two rows, every access of 4 bytes, 32 columns by 16 rows and two blocks per SM 396 / 174 (64 columns 433 /
-// 175; loads at their use 430 / 180; planes prefetched into L2 466 / 189); +z kept in registers, which spilled, 849 / 154.
+// What bounds it: the queue of memory instructions (D3Q19: 2.3 of 10.5 cycles per issue) and the one barrier per
+// plane (1.3) with 16 warps per SM at 128 registers; DRAM moves 76 bytes per D3Q19 update (152 with one step per
+// launch).  us per step on 256^3, one step per launch -> now: D3Q19 393 -> 281 (0.67 of the measured copy rate),
+// D3Q13 235 -> 154, D3Q9 153 -> 116; 255x249x251 (4-byte accesses) 431 -> 292, 270 -> 157.  Measured on 256^3
+// (D3Q19 / D3Q13) and not taken: the cells of a lane in two rows, every access of 4 bytes, 32 columns by 16 rows and
+// two blocks per SM 396 / 174 (64 columns 433 / 175; loads at their use 430 / 180; planes prefetched into L2
+// 466 / 189); +z kept in registers, which spilled, 849 / 154.
 #pragma once
 
 #include "kernels.cuh"
