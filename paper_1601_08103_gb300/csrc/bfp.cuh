@@ -319,11 +319,11 @@ __device__ __forceinline__ void stream_collide_chunk_bfp(const Bfp16 *__restrict
 // time), so decoding and encoding cost it against FP16: D3Q7 384^3 at 231 GLUPS, 5.9 TB/s in
 // algorithmic bytes, against 292 GLUPS for FP16.
 // Blocks per SM for which the compiler lays out the kernel (see step_min_blocks; us per step, its choice and the
-// bound: D2Q5 1024^2 frame 5.72 and 5.03; D3Q9 160^3 zero edge 42.3 and 35.7, frame 54.7 and 49.0).
+// bound: D2Q5 1024^2 frame 5.72 and 5.03; D3Q9 160^3 41.9 and 32.9, frame 54.7 and 49.0).
 template <class S, int V, Edge EDGE>
 __host__ __device__ constexpr int step_min_blocks_bfp() {
     if (S::Q == 5 && EDGE == kFrameEdge) return 4;
-    return S::Q == 9 && V == 8 && EDGE != kWrapEdge ? (EDGE == kFrameEdge ? 2 : 3) : 0;
+    return S::Q == 9 && V == 8 ? (EDGE == kFrameEdge ? 2 : 3) : 0;
 }
 template <class S, int V, Edge EDGE>
 __global__ void __launch_bounds__(256, step_min_blocks_bfp<S, V, EDGE>())

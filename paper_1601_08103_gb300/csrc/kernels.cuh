@@ -728,15 +728,15 @@ __global__ void __launch_bounds__(1024) k_onchip_1d(T *__restrict__ g, int nx, l
 
 // Blocks per SM for which the compiler lays out the kernels of many registers; 0 is its own choice, which is right
 // elsewhere (a bound of one block makes it take many more).  us per step, its choice and the bound: D3Q13 FP16
-// 160^3 frame 97 and 52; D3Q13 FP32 160^3 zero edge 71 and 63; frames of D3Q7 FP16 160^3 28 and 23, of
+// 160^3 36.7 and 30.7, frame 97 and 52; D3Q13 FP32 160^3 zero edge 71 and 63; frames of D3Q7 FP16 160^3 28 and 23, of
 // D3Q9 FP32 160^3 57 and 52.
 template <class S, class T, int V, Edge EDGE>
 __host__ __device__ constexpr int step_min_blocks() {
     int pulls = 0;  // registers of a thread's pulls
     for (int i = 0; i < S::Q; ++i) pulls += carried<S>(i) ? V * (int)sizeof(typename Store<T>::C) / 4 : 0;
     if (!rest_static<S>() || sizeof(T) == 8) return 0;
-    if (EDGE == kWrapEdge) return 0;
     if (pulls > 64) return 2;
+    if (EDGE == kWrapEdge) return 0;
     if (V == 8) return pulls > 32 ? 3 : 0;
     return pulls > 32 ? (EDGE == kZeroEdge ? 4 : 0) : pulls == 32 && V == 4 && EDGE == kFrameEdge ? 4 : 0;
 }
