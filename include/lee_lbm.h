@@ -199,7 +199,8 @@ lee_status lee_lbm_init_fields(lee_lbm *h, const double *rho, const double *u, c
  *    grids with nx not a multiple of 4 then take single steps);
  *  - periodic 3D FP32 grids of D3Q7 and diatomic D3Q7 advance four steps per launch (a pipeline of the
  *    planes), then, with nx a multiple of 4, two (a z-marching tile), then one; grids of fewer than
- *    786432 cells (2097152 where nx is not a multiple of 4), where that is slower, take single steps (LEE_TB_STEPS=1 or 2 fixes the count);
+ *    786432 cells (2097152 where nx is not a multiple of 4), where that is slower, take single steps (calls of
+ *    fewer than eight steps with up to 262144 cells and nx a multiple of 4: two; LEE_TB_STEPS=1 or 2 fixes the count);
  *  - periodic 3D FP32 grids of D3Q9, D3Q13 and D3Q19 advance two steps per launch where their copies are well beyond L2
  *    (from 883011 cells of D3Q19, 1290555 of D3Q13, 3728270 of D3Q9) and the grid fills the launch's tiles of 60 x 14
  *    cells (lee_lbm_steps_per_launch reports 1; not with LEE_TB_STEPS or LEE_SINGLE_STEP);

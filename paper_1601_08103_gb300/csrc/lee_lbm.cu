@@ -202,7 +202,7 @@ bool plane_pipe(const lee_lbm *h) {
            !h->tb_env && !tma_tile(h) && plane_pipe_eligible(h->cfg.ny);
 }
 
-constexpr long long kFuse3dCells = 3LL << 18, kFuse3dRaggedCells = 1LL << 21, kPairBytes = 128LL << 20;
+constexpr long long kDirectPairCells = 1LL << 18, kFuse3dCells = 3LL << 18, kFuse3dRaggedCells = 1LL << 21, kPairBytes = 128LL << 20;
 
 // Cells from which a 3D grid on the plane pipelines takes several steps per launch.  For the two steps of the sets
 // with diagonal velocities: both copies well beyond L2, in which single steps run otherwise (us per step of one
@@ -231,14 +231,16 @@ bool ragged_2d(const lee_lbm *h) {
 // 2D FP32 at such widths: 2047x2045 160 GLUPS with single steps, 920 on the row pipeline.
 // Measured on GB300, GLUPS: D2Q5 FP32 2048^2 / 8192^2 four steps per launch 740 / 811, eight 1490 / 1611; D3Q7
 // FP32 384^3 / 256^3 two 259 / 232, four 426 / 373.
-int next_launch(const lee_lbm *h, int unit, long long left) {
+// Calls of a few steps are launched directly and are held up by the host, about 4 us per launch: on grids whose two-step launches
+// take less than twice that they use those (12^3, calls of five steps: 4.0 us per step with single ones, 3.4 so).
+int next_launch(const lee_lbm *h, int unit, long long left, bool direct) {
     if (ragged_2d(h)) return left >= kRpDeep ? kRpDeep : left >= 4 ? 4 : (int)left;
     if (unit > 1 && h->D == 2 && !h->tb_env) {
         if (left >= kRpDeep && h->cfg.storage != LEE_STORE_BFP16) return kRpDeep;
         if (left < unit && left > 1 && h->cfg.storage == LEE_STORE_F32) return (int)left;
     }
     if (h->D == 3 && plane_pipe(h) && h->cut3d[3] > 0) {
-        if (h->cells < fuse_3d_cells(h)) return 1;
+        if (h->cells < fuse_3d_cells(h)) return direct && h->cells <= kDirectPairCells && left >= unit ? unit : 1;
         if (left >= h->ops->deep3d) return h->ops->deep3d;
     }
     return left >= unit ? unit : 1;
@@ -247,8 +249,9 @@ int next_launch(const lee_lbm *h, int unit, long long left) {
 // Launches of a run of `steps` steps.
 int64_t run_launches(const lee_lbm *h, int unit, int64_t steps) {
     int64_t c = 0;
+    const bool direct = steps < kGraphMinLaunches;
     while (steps > 0) {
-        const int k = next_launch(h, unit, steps);
+        const int k = next_launch(h, unit, steps, direct);
         const int64_t r = steps / k;  // as many of this size as fit
         c += r;
         steps -= r * k;
@@ -260,7 +263,7 @@ int64_t run_launches(const lee_lbm *h, int unit, int64_t steps) {
 // (all of this size but for the last): 0 where there are none.
 int split_launch(const lee_lbm *h, int unit, int k) {
     if (h->tb_env || k < 2) return 0;
-    if (h->D == 3) return k != h->ops->deep3d || !plane_pipe(h) ? 0 : k == 4 && unit == 2 ? 2 : 1;
+    if (h->D == 3) return !plane_pipe(h) ? 0 : k == 4 && unit == 2 ? 2 : 1;
     if (k == kRpDeep) return 4;
     return h->cfg.storage == LEE_STORE_F32 ? (k + 1) / 2 : 0;  // (a 16-bit state would be rounded at other steps)
 }
@@ -762,9 +765,10 @@ lee_status lee_lbm_step(lee_lbm *h, int64_t n) {
         return LEE_OK;
     };
     int64_t left = n;
+    const bool direct = n < kGraphMinLaunches;
     const int64_t count = run_launches(h, unit, n);
     if (n >= 2 && (count >= kGraphMinLaunches || (count & 1)) && capturing(h->st)) {
-        const int first = next_launch(h, unit, n), part = count & 1 ? split_launch(h, unit, first) : 0;
+        const int first = next_launch(h, unit, n, direct), part = count & 1 ? split_launch(h, unit, first) : 0;
         for (int k = part ? first : 0; k > 0; k -= part) {
             const lee_status s = run(part < k ? part : k);
             if (s != LEE_OK) return s;
@@ -786,7 +790,7 @@ lee_status lee_lbm_step(lee_lbm *h, int64_t n) {
                 cudaError_t e = cudaSuccess;
                 int w = h->cur;
                 for (int64_t r = steps; r > 0 && e == cudaSuccess; w ^= 1) {
-                    const int k = next_launch(h, unit, r);
+                    const int k = next_launch(h, unit, r, false);
                     e = launch(w, k, h->cap);
                     r -= k;
                 }
@@ -804,7 +808,7 @@ lee_status lee_lbm_step(lee_lbm *h, int64_t n) {
         }
     }
     while (left > 0) {
-        const int k = next_launch(h, unit, left);
+        const int k = next_launch(h, unit, left, direct);
         const lee_status s = run(k);
         if (s != LEE_OK) return s;
         left -= k;

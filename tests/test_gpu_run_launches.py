@@ -13,7 +13,9 @@ pytestmark = pytest.mark.gpu
     ("D2Q5", (64, 33, 1), "f32", "open_zero", {8: 8}),
     ("D1Q3", (1000, 1, 1), "f64", "periodic", {1: 1, 2000: 1}),
     ("D1Q3", (1000, 1, 1), "f64", "open_sponge", {1: 1, 2000: 1}),
-    ("D3Q7", (16, 9, 7), "f32", "periodic", {8: 8}),
+    ("D3Q7", (16, 9, 7), "f32", "periodic", {2: 1, 5: 3, 7: 4, 8: 8}),
+    ("D3Q7", (64, 64, 72), "f32", "periodic", {5: 5, 8: 8}),
+    ("D3Q7", (15, 9, 7), "f32", "periodic", {5: 5}),
     ("D3Q7", (132, 83, 75), "f32", "periodic", {3: 2, 4: 1, 8: 2, 43: 12}),
     ("D3Q19", (120, 84, 100), "f32", "periodic", {2: 1, 5: 3}),
 ])
